@@ -224,12 +224,14 @@ def tuning_key(t) -> list:
 PYR_DTYPES = {"f32": (1, 0, 4), "bf16": (2, 1, 2), "f16": (3, 2, 2)}
 
 
-def rig_level_kernels(h: int, widths, levels: int, kernels, tiles=None):
+def rig_level_kernels(h: int, widths, levels: int, kernels, tiles=None, stream_min=STREAM_MIN_PIXELS):
     """Kernel launches of each LK level of a rig, in launch order: for level
     l, [(kernel name, [pairs])], the streamed batch first, then one tiled
     launch per tile shape (in the order of the first pair with it).
     kernels[l] is the level's PANO_LK_* tuning and tiles[l] its (tile_w,
-    tile_h), (0, 0) for the default; AUTO uses the single-pair rules."""
+    tile_h), (0, 0) for the default. AUTO streams the pairs of at least
+    stream_min pixels at the level (0: all of them, as the library does while
+    iters * radius is at most 24)."""
     out = []
     for l in range(levels):
         hl = h
@@ -240,7 +242,7 @@ def rig_level_kernels(h: int, widths, levels: int, kernels, tiles=None):
         tile = tuple(tiles[l]) if tiles else (0, 0)
         st, groups = [], {}
         for k, w in enumerate(ws):
-            use = kernels[l] == PANO_LK_STREAM or (kernels[l] == PANO_LK_AUTO and hl * w >= STREAM_MIN_PIXELS)
+            use = kernels[l] == PANO_LK_STREAM or (kernels[l] == PANO_LK_AUTO and hl * w >= stream_min)
             if use:
                 st.append(k)
                 continue
@@ -579,10 +581,9 @@ def run_gpu(args):
     stream_bytes = 0.0
     for kind, lev, ms in recs:
         if kind == 4:
-            # levels of at least STREAM_MIN_PIXELS run the streamed kernel
-            name = "lk_stream_kernel" if npx[lev] >= STREAM_MIN_PIXELS else "lk_level_kernel"
-            if name == "lk_stream_kernel":
-                stream_bytes += lk_bytes[lev]
+            # every level runs the streamed kernel (5 steps, radius 2)
+            name = "lk_stream_kernel"
+            stream_bytes += lk_bytes[lev]
         else:
             name = names[kind]
         d = per_kind.setdefault(name, {"launches": 0, "ms": 0.0})
@@ -985,7 +986,7 @@ def measure_rig(dev, pairs, pyr_dtype: str, steps: int, warmup: int, world: int 
         recs = rig.trace_read(64 * steps)
         rig.trace_enable(0, 0)
         plan = rig_level_kernels(h, widths, levels, [t["kernel"] for t in tunings],
-                                 [(t["tile_w"], t["tile_h"]) for t in tunings])
+                                 [(t["tile_w"], t["tile_h"]) for t in tunings], stream_min=0)
         names = {1: "luma_kernel", 2: "pyr_down_kernel", 8: "rig_blend_kernel", 16: "luma_reduce_kernel",
                  32: "pyr_tail_kernel"}
         per_kind, lk_seen = {}, {}

@@ -351,10 +351,10 @@ PANO_API pano_status pano_stage_lk(const float* T, const float* J, int h, int w,
  * pano_rig.h). Both kernels compute the same equations with the same order
  * of FP32 operations; results differ only in rounding, because each tile or
  * segment measures its flows against its own reference flow. */
-#define PANO_LK_AUTO   0  /* the kernel pano_flow_pair runs for a level of this size: streamed
-                             for levels of at least 50000 pixels (1 <= iters <= 5), tiled
-                             below (16 x 8 tiles below 16000 pixels) */
-#define PANO_LK_STREAM 1  /* streamed row chunks down column bands (1 <= iters <= 5) */
+#define PANO_LK_AUTO   0  /* the kernel pano_flow_pair runs: streamed for iters >= 1 and
+                             iters * radius <= 24, tiled otherwise (16 x 8 tiles for levels
+                             below 16000 pixels) */
+#define PANO_LK_STREAM 1  /* column bands cut into segments of rows (1 <= iters <= 5) */
 #define PANO_LK_TILE   2  /* output tiles with a halo of iters * radius pixels */
 
 /* pano_stage_lk with the kernel chosen by the caller (a PANO_LK_* value);

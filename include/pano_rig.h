@@ -10,9 +10,9 @@
  *
  *   luma of all strips          one launch
  *   REDUCE of all strips        one launch per level
- *   LK, both directions, every  per level, one persistent launch of the
- *   pair                        streamed kernel over the (pair, direction,
- *                               band, segment) work list and/or one tiled
+ *   LK, both directions, every  per level, one launch of the streamed
+ *   pair                        kernel over every (pair, direction, band,
+ *                               segment) and/or one tiled
  *                               grid per tile shape over those pairs
  *   blend into the canvas       one launch
  *
@@ -63,8 +63,8 @@ typedef struct pano_rig_desc {
 
 typedef struct pano_rig_tuning {
     int kernel;          /* a PANO_LK_* value (pano_flow.h) */
-    int seg_rows;        /* streamed kernel: rows per segment, 0 = automatic (about 256,
-                            rounded to whole waves of the GPU) */
+    int seg_rows;        /* streamed kernel: rows per segment, rounded up to whole CTAs and
+                            limited to a cluster of 8 of them; 0 = automatic */
     int tile_w, tile_h;  /* tiled kernel: output tile; both 0 = the default tile */
     float ms;            /* device time of the level measured by pano_rig_autotune, else 0 */
 } pano_rig_tuning;

@@ -167,14 +167,13 @@ struct LkArgs {
 };
 
 // The same pyramid level of several strip pairs in one launch (all share
-// iters and radius): persistent for the streamed kernel, one grid over every
-// pair and direction for the tiled one (all pairs then share the tile shape).
+// iters and radius): one grid over every pair and direction (the tiled
+// kernel's pairs then share the tile shape, the streamed one's their height).
 struct LkBatch {
     LkArgs pair[kMaxBatch];
     int n;
-    int nb[kMaxBatch], seg[kMaxBatch], nseg[kMaxBatch];  // filled by the launcher
+    int nb[kMaxBatch], nseg[kMaxBatch];                   // filled by the launcher
     int start[kMaxBatch + 1];                             // item prefix sums
-    unsigned* counter;                                    // device work counter
 };
 
 // Code 1 blend or the plain flow warp.
@@ -247,14 +246,29 @@ cudaError_t launch_pyr_down(const PyrDownArgs& a, cudaStream_t s);
 cudaError_t launch_luma_reduce(const LumaReduceArgs& a, cudaStream_t s);
 cudaError_t launch_pyr_tail(const PyrTailArgs& a, cudaStream_t s);
 cudaError_t pyr_tail_prepare(int max_smem_bytes);
-// One LK level: streamed (lk_stream.cu) for levels of at least
-// kStreamMinPixels pixels and 1 <= iters <= 5, tiled (lk.cu) otherwise.
+// One LK level: streamed (lk_stream.cu) for 1 <= iters and iters * radius up
+// to kStreamMaxReach, tiled (lk.cu) otherwise.
+// The streamed kernel has two CTA shapes (lk_stream_impl.cuh): small regions
+// for levels whose pixels times halo (columns and rows lost on each side) are
+// below kStreamSmallWork, because a small level's time is the latency of one
+// CTA; large ones else, because they lose less to the halo. Measured per
+// level, both directions, small / large regions / the tiled kernel in us:
+// 5 steps at radius 2: 120 x 85 pixels 9.0 / 16.9 / 14.5, 500 x 188 11.5 /
+// 16.8 / 28 (its streamed predecessor), 256 x 512 14.1 / 16.9, 1000 x 375 36 /
+// 40, 960 x 1000 69 / 65, 2000 x 750 105 / 83; radius 3: 250 x 250 15.5 / 18.2,
+// 256 x 512 18.8 / 16.2; 8 steps at radius 2: 250 x 250 14.7 / 22.3 / 53,
+// 256 x 512 28.5 / 20.4 / 103. For one pair both take the same time at about
+// 500000 pixels of radius 2; the line is drawn lower because the pairs of a
+// rig, each cut as it is by itself, fill the GPU together.
+// Beyond kStreamMaxReach a region would be mostly halo (at 24, 80 of 128
+// columns are left, and 1000 x 375 pixels take 77 us against 1373 us tiled).
+constexpr long long kStreamSmallWork = 1600000;
+constexpr int kStreamSmallHalo = 16;  // half of a small region is left
+constexpr int kStreamMaxReach = 24;
 // Levels below kSmallTilePixels use small tiles (kSmallTileW x kSmallTileH):
 // their few large tiles would leave most SMs idle, and the time of such a
-// level is the latency of one tile. (Measured on GB300: a 94k-pixel level
-// takes 38 us streamed and 51 us tiled; a 5.9k-pixel level 15 us on 16x8
-// tiles and 21 us on 32x16.)
-constexpr long long kStreamMinPixels = 50000;
+// level is the latency of one tile. (Measured on GB300: a 5.9k-pixel level
+// takes 15 us on 16x8 tiles and 21 us on 32x16.)
 constexpr long long kSmallTilePixels = 16000;
 constexpr int kSmallTileW = 16, kSmallTileH = 8;
 // Tile of the tiled kernel for a level of w x h pixels, given the default.
@@ -266,11 +280,13 @@ inline void lk_level_tile(int w, int h, int def_w, int def_h, int* tw, int* th) 
 cudaError_t launch_lk_level(const LkArgs& a, int ndirs, cudaStream_t s);
 cudaError_t launch_lk_tile(const LkArgs& a, int ndirs, cudaStream_t s);
 cudaError_t launch_lk_tile_batch(const LkBatch& b, cudaStream_t s);
-// Streamed form of the same level (lk_stream.cu), used for 1 <= iters <= 5.
+// Streamed form of the same level (lk_stream.cu). A caller may name it for
+// 1 <= iters <= 5 (lk_stream_supports); lk_auto_streams is launch_lk_level's rule.
 bool lk_stream_supports(int iters, int radius);
+inline bool lk_auto_streams(int iters, int radius) { return iters >= 1 && iters * radius <= kStreamMaxReach; }
 cudaError_t lk_stream_prepare(int max_smem_bytes);
 cudaError_t launch_lk_stream(const LkArgs& a, int ndirs, cudaStream_t s);
-cudaError_t launch_lk_stream_batch(const LkBatch& b, int n_ctas, cudaStream_t s);
+cudaError_t launch_lk_stream_batch(const LkBatch& b, cudaStream_t s, int* kernels);
 size_t lk_smem_bytes(int tile_w, int tile_h, int iters, int radius);
 cudaError_t lk_prepare(int max_smem_bytes);
 cudaError_t launch_blend(const BlendArgs& a, cudaStream_t s);

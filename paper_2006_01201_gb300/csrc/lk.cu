@@ -333,10 +333,7 @@ cudaError_t lk_prepare(int max_smem_bytes) {
 }
 
 cudaError_t launch_lk_level(const LkArgs& a, int ndirs, cudaStream_t s) {
-    // Small levels have too few rows to fill the streamed schedule; tiles
-    // run them in one short wave.
-    if (lk_stream_supports(a.iters, a.radius) && (long long)a.w * a.h >= kStreamMinPixels)
-        return launch_lk_stream(a, ndirs, s);
+    if (lk_auto_streams(a.iters, a.radius)) return launch_lk_stream(a, ndirs, s);
     return launch_lk_tile(a, ndirs, s);
 }
 

@@ -23,16 +23,16 @@ cudaError_t lk_stream_prepare(int max_smem_bytes) {
     return lks::stream_prepare<__half>(max_smem_bytes);
 }
 
-cudaError_t launch_lk_stream_batch(const LkBatch& b, int n_ctas, cudaStream_t s) {
+cudaError_t launch_lk_stream_batch(const LkBatch& b, cudaStream_t s, int* kernels) {
     if (b.n < 1 || b.n > kMaxBatch) return cudaErrorInvalidValue;
     for (int p = 1; p < b.n; ++p)
         if (b.pair[p].pyr != b.pair[0].pyr || b.pair[p].iters != b.pair[0].iters ||
             b.pair[p].radius != b.pair[0].radius)
             return cudaErrorInvalidValue;
     switch (b.pair[0].pyr) {
-        case kPyrF32: return lks::stream_launch_batch<float>(b, n_ctas, s);
-        case kPyrBF16: return lks::stream_launch_batch<__nv_bfloat16>(b, n_ctas, s);
-        case kPyrF16: return lks::stream_launch_batch<__half>(b, n_ctas, s);
+        case kPyrF32: return lks::stream_launch_batch<float>(b, s, kernels);
+        case kPyrBF16: return lks::stream_launch_batch<__nv_bfloat16>(b, s, kernels);
+        case kPyrF16: return lks::stream_launch_batch<__half>(b, s, kernels);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -1,7 +1,7 @@
-// lk_stream_impl.cuh -- internal: the streamed LK kernel, templated on the
-// storage type of the pyramid planes. One pyramid level of dense
-// Lucas-Kanade flow (Section III-C-1), all K steps fused, streamed down
-// column bands. Included once per storage type (lk_stream.cu: float,
+// lk_stream_impl.cuh -- internal: the LK kernel of large levels, templated on
+// the storage type of the pyramid planes. One pyramid level of dense
+// Lucas-Kanade flow (Section III-C-1), all K steps fused, on column bands cut
+// into segments of rows. Included once per storage type (lk_stream.cu: float,
 // lk_stream_bf16.cu, lk_stream_f16.cu), each of which instantiates the entry
 // points at the end of this file for its type only.
 //
@@ -10,36 +10,49 @@
 //   It(q) = J(q + u(q)) - T(q), u(p) <- v,
 // over the (2r+1)^2 box clipped to the image.
 //
-// Schedule. A CTA owns a band of BW output columns and a segment of output
-// rows, plus a halo of K*r columns on each side. It walks down the segment in
-// chunks of CH rows. Step k of the iteration ("stage k") runs r rows behind
-// stage k-1, so that when stage k updates rows [a_k, a_k + CH) the flows it
-// needs from stage k-1 (rows up to a_k + CH + r) are already final. Within a
-// chunk the stages run in order:
-//   X_0 : load T, grad T and the starting flow of the CH newest rows and form
-//         the residual products P = grad T (grad T . u - It) of stage 1;
-//   B_k : column sums of P over 2r+1 rows (stage k); B_1 also forms the
-//         column sums of grad T grad T^T of the newest complete rows;
-//   X_k : row sums, the 2x2 solve and the update of stage k (X_1 first
-//         completes the normal matrices and inverts them), then, for the
-//         same pixels, the products P of stage k+1; X_K writes the output
-//         and loads the target rows of the next chunk.
-// Per-row state (T, grad T, flow, inverse normal matrix) lives in a ring of
-// kRing rows in shared memory; each stage keeps the last 2r rows of its
-// products for the next chunk. The target image J is staged in a second ring
-// of kRing rows: a box of the band shifted by the CTA's reference flow, with
-// a margin of kMX columns and kMY rows, holding clamp-to-edge values; a sample
-// whose four taps fall outside the box is read from global memory instead.
-// The first chunks of a segment start ceil(2 K r / CH) chunks early, so every
-// row a stage must produce is computed from complete windows; the rows before
-// that are discarded. Flows are kept relative to the reference flow (the
-// starting flow at the centre of the band and segment) so that FP32 rounding
-// does not grow with the size of the flow.
+// Schedule. A segment of a band (RW columns, C * RH rows, halo included) is
+// one cluster of C CTAs on top of each other; a thread owns two neighbouring
+// columns of a run of R rows and keeps their flow, template and gradient in
+// registers for all K steps. A step is
+//   A  the residual products P = grad T (grad T . u - It) of the own pixels,
+//      the r outer rows of the run first: they go to the neighbouring run's
+//      halo, in this CTA or the one above or below (st.async, counted by a
+//      barrier there);
+//   B  the column sums over 2r+1 rows of the rows that need no outer halo,
+//      from registers, to shared memory;
+//   C  after a barrier of the warps that share the rows: their row sums, the
+//      2x2 solve and the update;
+// then B and C of the r outer rows, when the neighbours' rows have come. So
+// the rows between the CTAs of a cluster are exchanged, not recomputed, and
+// their way is hidden by the inner rows' work: only the band's sides and the
+// cluster's top and bottom carry a halo of K r pixels, that the steps eat up
+// from outside (108 x 204 of 128 x 224 pixels are left at K r = 10).
 //
-// T and J are read as Ts and widened to FP32: float planes are fetched with
-// cp.async, 16-bit planes with plain loads (their elements are narrower than
-// the 4-byte copies), the target rows of the next chunk into registers before
-// X_K and stored to the ring after it.
+// What bounds it (level 0 of a 4000 x 1500 pair, both directions): the issue
+// of instructions and the shared-memory pipe, at 128 registers a thread and
+// 16 warps an SM. Before, 768 threads worked through 12-row chunks of a ring
+// in shared memory, eleven CTA-wide barriers a chunk: 352 M warp
+// instructions in 568 us. Registers instead of the ring, and two pixels per
+// paired instruction: 177 M instructions. Measured with the same arithmetic:
+// one barrier.cluster a step in place of the counted halos 375 us (every
+// thread's fence in it); the same, sent before and awaited after the inner
+// rows' work, 3% slower on the whole 4000 x 1500 pair than this form;
+// counted halos without the inner rows in between 408 us. Clusters of at most
+// 4 CTAs: 1 to 3% slower; runs of 6 rows: 2 to 6% slower.
+//
+// The two halves of a warp own two runs on top of each other, the lower one
+// upside down. "Outer" rows (towards another warp) and "inner" rows (towards
+// the other half, exchanged by a shuffle) then have the same register names
+// in both halves. The two halves' rows are an odd number apart, and so is the
+// pitch of the staged target: the samples of the two halves, which cover every
+// second column each, fall on different banks.
+//
+// The target J is staged as a box of the CTA's region, shifted by the integer
+// part of the starting flow at its centre, with a margin of kMX columns and
+// kMY rows and clamp-to-edge values; a sample whose four taps fall outside the
+// box is read from global memory instead. Flows are kept relative to the
+// cluster's reference flow (the starting flow at its centre) so that FP32
+// rounding does not grow with the size of the flow.
 #pragma once
 
 #include <type_traits>
@@ -50,64 +63,104 @@
 namespace pano {
 namespace lks {
 
-constexpr int kStreamThreads = 768;
-constexpr int kRing = 32;
-constexpr int kRingOff = 1 << 20;  // keeps ring slots of negative rows non-negative
-constexpr int kMX = 8;             // target box margin, columns
-constexpr int kMY = 3;             // target box margin, rows
-constexpr int kCsT0 = 256;         // first thread of the normal-matrix column sums in B_1
+constexpr int kMX = 8;            // target box margin, columns
+constexpr int kMY = 3;            // target box margin, rows
+constexpr int kMaxCluster = 8;    // CTAs per cluster (the portable limit)
 
-template <int RAD, int K, int BW, int CH>
+template <int RAD, int R, int WX, int WY>
 struct StreamGeom {
-    static constexpr int RW = BW + 2 * K * RAD;  // region columns
-    static constexpr int JW = RW + 2 * kMX + 2;  // target box columns
-    static constexpr int PR = CH + 2 * RAD;      // rows of the product buffer
-    static_assert(CH >= 2 * RAD, "chunk must cover the column-sum history");
-    static_assert(CH + (K + 1) * RAD <= kRing, "row ring too small");
-    static_assert((K - 1) * RAD + CH + 2 * kMY + 2 <= kRing, "target ring too small");
-    static constexpr size_t kT = 0;
-    static constexpr size_t kG = kT + sizeof(float) * kRing * RW;
-    static constexpr size_t kU = kG + sizeof(float2) * kRing * RW;
-    static constexpr size_t kGiA = kU + sizeof(float2) * kRing * RW;
-    static constexpr size_t kGiB = kGiA + sizeof(float2) * kRing * RW;
-    static constexpr size_t kJ = kGiB + sizeof(float) * kRing * RW;
-    static constexpr size_t kP = kJ + sizeof(float) * kRing * JW;
-    static constexpr size_t kH = kP + sizeof(float2) * PR * RW;
-    // sV, sCSA and sCSB are padded by kPad elements on both sides: the row
-    // sums of the column pair at a stage's edge read a window of up to
-    // kPad elements beyond the first or last column (values of pixels the
-    // stage does not update, never used), which then stays in the array
-    static constexpr int kPad = 4;
-    static constexpr size_t kV = kH + sizeof(float2) * K * 2 * RAD * RW + sizeof(float2) * kPad;
-    static constexpr size_t kCSA = kV + sizeof(float2) * (CH * RW + kPad) + sizeof(float2) * kPad;
-    static constexpr size_t kCSB = kCSA + sizeof(float2) * (CH * RW + kPad) + sizeof(float) * kPad;
-    // next chunk's template rows (with a 1-pixel ring) and coarse flow rows
-    static constexpr int TSW = RW + 2, TSH = CH + 2;
-    static constexpr int FSW = RW / 2 + 3, FSH = CH / 2 + 3;
-    static constexpr size_t kTS = kCSB + sizeof(float) * (CH * RW + kPad);
-    static constexpr size_t kFS = (kTS + sizeof(float) * TSH * TSW + 7) / 8 * 8;
-    static constexpr size_t bytes = kFS + sizeof(float2) * FSH * FSW;
+    static constexpr int RW = 32 * WX;               // region columns
+    static constexpr int NP = RW / 2;                // column pairs
+    static constexpr int RH = 2 * R * WY;            // region rows of one CTA
+    static constexpr int threads = 32 * WX * WY;
+    static constexpr int JP = RW + 2 * kMX + 1;      // pitch of the target box (odd), RW + 2 kMX columns used
+    static constexpr int JH = RH + 2 * kMY;
+    static constexpr int VP = NP + 4;                // column sums: two zero pairs on either side
+    static constexpr int TP = RW + 4, TH = RH + 2 * (RAD + 1);  // staged template
+    static constexpr int NJ = JP * JH, NG = RH * NP, NV = RH * VP, NT = TP * TH, NO = 2 * WY * 2 * RAD * NP;
+    static constexpr size_t kJ = 0;
+    static constexpr size_t kGA = (kJ + sizeof(float) * NJ + 15) / 16 * 16;
+    static constexpr size_t kGB = kGA + sizeof(float4) * NG;
+    static constexpr size_t kO = kGB + sizeof(float2) * NG;
+    static constexpr size_t kV = kO + sizeof(float4) * NO;
+    static constexpr size_t kB = kV + sizeof(float4) * NV;  // barriers of the halos [parity][wy][half]
+    static constexpr size_t bytes = kB + sizeof(unsigned long long) * 4 * WY;
+    static constexpr size_t kT = kGA;                // the template is read before the normal matrices are written
+    static_assert(sizeof(float) * NT <= sizeof(float4) * NG + sizeof(float2) * NG, "staged template too large");
+    static_assert(R >= 2 * RAD, "a run must cover the rows it exchanges on both sides");
 };
 
-__device__ __forceinline__ int ring_slot(int y) { return (y + kRingOff) & (kRing - 1); }
+// Halo of K steps, rounded to even so that regions start on even pixels.
+__host__ __device__ constexpr int stream_halo(int iters, int radius) { return (iters * radius + 1) & ~1; }
 
-// Paired FP32 arithmetic (one instruction for the two lanes of a float2;
-// each lane rounds exactly as the scalar operation would).
+// Paired FP32 arithmetic: one instruction for the two pixels of a thread's
+// column pair; each lane rounds exactly as the scalar operation would.
+__device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 
 __device__ __forceinline__ void copy_async4(void* dst_smem, const void* src) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst_smem);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
 }
-__device__ __forceinline__ void copy_async8(void* dst_smem, const void* src) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst_smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
-}
 __device__ __forceinline__ void copy_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void copy_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// address of this CTA's shared address `p` in the CTA of rank `r`
+__device__ __forceinline__ unsigned cluster_map(unsigned p, unsigned r) {
+    unsigned d;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(p), "r"(r));
+    return d;
+}
+// 16 bytes to a CTA of the cluster, counted by the barrier there
+__device__ __forceinline__ void cluster_send(unsigned addr, unsigned bar, float2 a, float2 b) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr),
+                 "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void bar_init(unsigned bar) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+}
+// the barrier's current phase ends when `bytes` have arrived
+__device__ __forceinline__ void bar_expect(unsigned bar, unsigned bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+// Waits until the phase of this parity has ended; false if it has not after
+// a bounded number of tries (some 0.1 s at least), which no launch that the
+// host checks let through reaches.
+__device__ __forceinline__ bool bar_wait(unsigned bar, unsigned parity) {
+    unsigned done = 0;
+    for (int n = 0; n < (1 << 22) && !done; ++n)
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+            : "=r"(done)
+            : "r"(bar), "r"(parity)
+            : "memory");
+    return done != 0;
+}
+// shared-memory load at a byte address plus a constant
+template <int OFF>
+__device__ __forceinline__ float ld_shared(unsigned addr) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1+%2];" : "=f"(v) : "r"(addr), "n"(OFF));
+    return v;
+}
+template <int N>
+__device__ __forceinline__ void named_barrier(int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(N) : "memory"); }
+
+// Starting flow of pixel (x, y): zero, the given one, or twice the coarser
+// level's flow at (x/2, y/2), bilinear.
 __device__ __forceinline__ float2 start_flow_s(const LkArgs& a, const LkDir& D, int x, int y) {
     if (a.mode == 0 || D.uin == nullptr) return make_float2(0.f, 0.f);
     const float2* __restrict__ u = reinterpret_cast<const float2*>(D.uin);
@@ -123,572 +176,626 @@ __device__ __forceinline__ float2 start_flow_s(const LkArgs& a, const LkDir& D, 
     return make_float2(2.f * fmaf(fy, bx - tx, tx), 2.f * fmaf(fy, by - ty, ty));
 }
 
-// What every stage needs to sample J around pixel q.
+__device__ __forceinline__ float2 floor_clamped(float2 v, int w, int h) {
+    return make_float2(floorf(fminf(fmaxf(v.x, -(float)(w + 2)), (float)(w + 2))),
+                       floorf(fminf(fmaxf(v.y, -(float)(h + 2)), (float)(h + 2))));
+}
+
+// A sample outside the staged box (large or non-finite offsets): clamped taps
+// of the global plane. Rare, and kept out of line.
 template <class Ts>
-struct TargetBox {
-    const float* sJ;   // ring of staged target rows
-    const Ts* J;       // global target plane (fallback)
-    int pitchJ, w, h;
-    int fref_x, fref_y;  // integer part of the reference flow
-};
-
-// J(q + ref + u) with clamp-to-edge taps: from the staged box when all four
-// taps lie in it, else from global memory. Both paths read the same values.
-template <int JW, class Ts>
-__device__ __forceinline__ float sample_target(const TargetBox<Ts>& b, int x, int y, int rx, float2 ref, float2 u) {
-    const float2 o = add2(ref, u);
-    const float ox = o.x, oy = o.y;
-    // floor(o) through the FP adder: o + 1.5 * 2^23 rounded down holds floor(o)
-    // in its low mantissa bits while |o| < 2^22; larger or non-finite offsets
-    // give integer parts far outside the box and take the global path
-    const float tx = __fadd_rd(ox, 12582912.0f), ty = __fadd_rd(oy, 12582912.0f);
-    const float fx = tx - 12582912.0f, fy = ty - 12582912.0f;
-    const unsigned uix = __float_as_uint(tx) - 0x4B400000u, uiy = __float_as_uint(ty) - 0x4B400000u;
-    const int ix = (int)uix, iy = (int)uiy;
-    const unsigned bcol_u = (unsigned)rx + uix - (unsigned)b.fref_x + (unsigned)kMX;
-    const int bcol = (int)bcol_u;
-    if (bcol_u < (unsigned)(JW - 1) && uiy - (unsigned)(b.fref_y - kMY) <= (unsigned)(2 * kMY)) {
-        Taps t;
-        t.ax = ox - fx;
-        t.ay = oy - fy;
-        const int o0 = ring_slot(y + iy) * JW + bcol, o1 = ring_slot(y + iy + 1) * JW + bcol;
-        constexpr int NJ = kRing * JW;
-        return bilinear_mix(t, PANO_AT(b.sJ, o0, NJ, 101), PANO_AT(b.sJ, o0 + 1, NJ, 102), PANO_AT(b.sJ, o1, NJ, 103),
-                            PANO_AT(b.sJ, o1 + 1, NJ, 104));
-    }
-    // outside the staged box (large or non-finite offsets): clamped global taps
-    return sample_plane(b.J, b.pitchJ, b.w, b.h, x, y, ox, oy);
+__device__ __noinline__ float far_sample(const Ts* J, int pitch, int w, int h, int x, int y, float ox, float oy) {
+    return sample_plane(J, pitch, w, h, x, y, ox, oy);
 }
 
-// Residual product of one sample q at flow u (relative to ref).
-template <int JW, class Ts>
-__device__ __forceinline__ float2 residual_product(const TargetBox<Ts>& b, int x, int y, int rx, float2 ref,
-                                                   float2 u, float2 g, float t) {
-    const float Jw = sample_target<JW, Ts>(b, x, y, rx, ref, u);
-    const float s = fmaf(g.x, u.x, fmaf(g.y, u.y, t - Jw));
-    return mul2(g, make_float2(s, s));
-}
-
-// Column sums over 2R+1 rows of the product buffer for the output rows
-// [part * CH / S, (part + 1) * CH / S) of one column: the CH / S + 2R values
-// are read once into registers and every output row is summed directly from
-// them (no running sums, which would carry rounding from one row into the
-// next). The part with the last rows also saves the last 2R product rows as
-// the history of this stage for the next chunk.
-template <int RAD, int CH, int RW, int S>
-__device__ __forceinline__ void column_sums(const float2* __restrict__ sP, float2* __restrict__ sV,
-                                            float2* __restrict__ hist, int rx, int part) {
-    static_assert(CH % S == 0, "parts must split the chunk rows evenly");
-    constexpr int HC = CH / S;
-    const int r0 = part * HC;
-    float2 p[HC + 2 * RAD];
+// Sums of 2 RAD + 1 consecutive elements of e: out[j] = e[j] + ... + e[j + 2 RAD].
+template <int RAD, int N>
+__device__ __forceinline__ void window_sums(const float2 (&e)[N + 2 * RAD], float2 (&out)[N]) {
+    float2 s[N + 2 * RAD - 1];  // pairs
 #pragma unroll
-    for (int d = 0; d < HC + 2 * RAD; ++d) p[d] = PANO_AT(sP, (r0 + d) * RW + rx, (CH + 2 * RAD) * RW, 105);
+    for (int i = 0; i < N + 2 * RAD - 1; ++i) s[i] = add2(e[i], e[i + 1]);
 #pragma unroll
-    for (int yy = 0; yy < HC; ++yy) {
-        float2 v = p[yy];
-#pragma unroll
-        for (int d = 1; d <= 2 * RAD; ++d) v = add2(v, p[yy + d]);
-        PANO_AT(sV, (r0 + yy) * RW + rx, CH * RW, 106) = v;
-    }
-    if (part == S - 1) {
-#pragma unroll
-        for (int d = 0; d < 2 * RAD; ++d) PANO_AT(hist, d * RW + rx, 2 * RAD * RW, 107) = p[HC + d];
+    for (int j = 0; j < N; ++j) {
+        if constexpr (RAD == 1) out[j] = add2(s[j], e[j + 2]);
+        else if constexpr (RAD == 2) out[j] = add2(add2(s[j], s[j + 2]), e[j + 4]);
+        else out[j] = add2(add2(add2(s[j], s[j + 2]), s[j + 4]), e[j + 6]);
     }
 }
 
-// One work item: direction `dir`, band `bx` (BW output columns) and segment
-// `by` (rows [by * seg, by * seg + seg)) of the level described by `a`.
-template <int RAD, int K, int BW, int CH, class Ts>
-__device__ __forceinline__ void lk_stream_item(const LkArgs& a, int dir, int bx, int by, int seg,
-                                               unsigned char* smem) {
-    constexpr bool kAsyncT = std::is_same<Ts, float>::value;  // cp.async of 4-byte elements
-    using Geo = StreamGeom<RAD, K, BW, CH>;
-    constexpr int RW = Geo::RW;
-    constexpr int JW = Geo::JW;
-    // Thread layout: thread (ty, tx) works on row ty of every chunk-sized
-    // block of rows and on the columns tx, tx + TX, tx + 2 TX, ...
-    constexpr int TX = kStreamThreads / CH;
-    static_assert(TX * CH == kStreamThreads, "threads must tile the chunk rows");
-    constexpr int kJPT = (Geo::JW + TX - 1) / TX;  // target-row elements per thread (16-bit planes)
-    float jnext[kJPT];
-    (void)jnext;
-    static_assert(2 * RW <= kCsT0 && kCsT0 + 2 * RW <= kStreamThreads && CH % 2 == 0, "B_1 thread groups");
-    float* sT = reinterpret_cast<float*>(smem + Geo::kT);
-    float2* sG = reinterpret_cast<float2*>(smem + Geo::kG);
-    float2* sU = reinterpret_cast<float2*>(smem + Geo::kU);
-    float2* sGiA = reinterpret_cast<float2*>(smem + Geo::kGiA);  // (i11, i12)
-    float* sGiB = reinterpret_cast<float*>(smem + Geo::kGiB);    // i22
+// Sums over the 2 RAD + 1 columns around each of a column pair c: l and r are
+// the neighbouring pairs, ll and rr the columns beyond them (RAD 3).
+template <int RAD>
+__device__ __forceinline__ float2 row_sums(float ll, float2 l, float2 c, float2 r, float rr) {
+    float m = c.x + c.y;
+    if constexpr (RAD == 1) return make_float2(m + l.y, m + r.x);
+    m += l.y + r.x;
+    if constexpr (RAD == 2) return make_float2(m + l.x, m + r.y);
+    m += l.x + r.y;
+    return make_float2(m + ll, m + rr);
+}
+
+// One CTA's part of one segment: direction `dir`, region columns
+// [ox, ox + RW), the cluster's region rows from oyc on; the pixels
+// [x_lo, x_hi) x [y_lo, y_hi) of the result are written. ox and oyc are even
+// and not negative. A float2 holds the same quantity of the thread's two
+// columns.
+template <int RAD, int R, int WX, int WY, class Ts>
+__device__ __forceinline__ void lk_stream_item(const LkArgs& a, int dir, int ox, int oyc, int csize, int x_lo, int x_hi,
+                                               int y_lo, int y_hi, unsigned char* smem) {
+    using Geo = StreamGeom<RAD, R, WX, WY>;
+    constexpr int RW = Geo::RW, RH = Geo::RH, NP = Geo::NP, JP = Geo::JP, JH = Geo::JH, VP = Geo::VP, TP = Geo::TP,
+                  TH = Geo::TH;
+    constexpr int NJ = Geo::NJ, NG = Geo::NG, NV = Geo::NV, NT = Geo::NT, NO = Geo::NO;
+    (void)NG, (void)NV, (void)NT, (void)NO, (void)NJ;
+    constexpr bool kAsync = std::is_same<Ts, float>::value;  // cp.async of 4-byte elements
     float* sJ = reinterpret_cast<float*>(smem + Geo::kJ);
-    float2* sP = reinterpret_cast<float2*>(smem + Geo::kP);
-    float2* sH = reinterpret_cast<float2*>(smem + Geo::kH);
-    float2* sV = reinterpret_cast<float2*>(smem + Geo::kV);
-    float2* sCSA = reinterpret_cast<float2*>(smem + Geo::kCSA);  // (c11, c12)
-    float* sCSB = reinterpret_cast<float*>(smem + Geo::kCSB);    // c22
-    float* sTS = reinterpret_cast<float*>(smem + Geo::kTS);      // staged template rows
-    float2* sFS = reinterpret_cast<float2*>(smem + Geo::kFS);    // staged coarse flow rows
-    constexpr int TSW = Geo::TSW, TSH = Geo::TSH, FSW = Geo::FSW, FSH = Geo::FSH;
-    // element counts of the shared arrays (for the debug build's index checks)
-    constexpr int NR = kRing * RW, NJ = kRing * JW, NP = (CH + 2 * RAD) * RW, NHIST = K * 2 * RAD * RW;
-    constexpr int NCH = CH * RW, NTS = TSH * TSW, NFS = FSH * FSW;
-    (void)NR, (void)NJ, (void)NP, (void)NHIST, (void)NCH, (void)NTS, (void)NFS;
+    float4* sGA = reinterpret_cast<float4*>(smem + Geo::kGA);  // inverse normal matrices: (i11, i11', i12, i12')
+    float2* sGB = reinterpret_cast<float2*>(smem + Geo::kGB);  // (i22, i22')
+    float4* sO = reinterpret_cast<float4*>(smem + Geo::kO);    // outer halos [parity][wy][half][RAD][NP]: (Px, Px', Py, Py')
+    float4* sV = reinterpret_cast<float4*>(smem + Geo::kV);    // column sums, rows in run order: (Vx, Vx', Vy, Vy')
+    float* sT = reinterpret_cast<float*>(smem + Geo::kT);      // template, before the normal matrices
 
     const LkDir D = dir ? a.dir[1] : a.dir[0];
     const int w = a.w, h = a.h;
-    const float lam = a.lambda;
     const Ts* __restrict__ T = static_cast<const Ts*>(D.T);
-    const int pitchT = D.pitchT;
-    const int X0 = bx * BW;
-    const int ox = X0 - K * RAD;
-    const int Y0 = by * seg;
-    const int Y1 = min(h, Y0 + seg);
-    const int tid = threadIdx.x;
-    const int ty = tid / TX, tx = tid - ty * TX;
-    // region columns that lie inside the image: [cmin, cmax)
-    const int cmin = max(0, -ox), cmax = min(RW, w - ox);
+    const Ts* __restrict__ J = static_cast<const Ts*>(D.J);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int wx = warp % WX, wy = warp / WX, half = lane >> 4;
+    const int rank = (int)cluster_rank();
+    const int oy = oyc + rank * RH;
+    const int px = wx * 16 + (lane & 15), rx = 2 * px;    // the thread's column pair
+    const int r0 = wy * 2 * R + (half ? 2 * R - 1 : 0);   // region row of row 0 of the run
+    const int dr = half ? -1 : 1;                         // and the step from one of its rows to the next
+    const int y0 = oy + r0, x0 = ox + rx;
+    const int srow = (wy * 2 + half) * R;                 // the run's rows in the arrays that are in run order
 
-    // reference flow: starting flow at the centre of the band and segment
-    const float2 ref = start_flow_s(a, D, min(X0 + BW / 2, w - 1), min((Y0 + Y1) / 2, h - 1));
-    TargetBox<Ts> box;
-    box.sJ = sJ;
-    box.J = static_cast<const Ts*>(D.J);
-    box.pitchJ = D.pitchJ;
-    box.w = w;
-    box.h = h;
-    box.fref_x = (int)floorf(fminf(fmaxf(ref.x, -(float)(w + 2)), (float)(w + 2)));
-    box.fref_y = (int)floorf(fminf(fmaxf(ref.y, -(float)(h + 2)), (float)(h + 2)));
-    const int jx0 = ox + box.fref_x - kMX;  // image column of box column 0
-
-    const bool stage_flow = a.mode == 1 && D.uin != nullptr;
-    const float2* __restrict__ ucoarse = reinterpret_cast<const float2*>(D.uin);
-    // Asynchronous copies of what X_0 of the chunk with newest rows
-    // [a0n, a0n + CH) reads from global memory: template rows a0n-1 .. a0n+CH
-    // (columns ox-1 .. ox+RW, clamp-to-edge) and, when the level starts from
-    // the coarser level, the coarse flow rows and columns its upsampling taps.
-    // Staged by nw workers, this thread being worker wi.
-    auto stage_inputs = [&](int a0n, int wi, int nw) {
-        for (int i = wi; i < TSH * TSW; i += nw) {
-            const int r = i / TSW, cc = i - r * TSW;
-            const int ys = min(max(a0n - 1 + r, 0), h - 1), xs = min(max(ox - 1 + cc, 0), w - 1);
-            const Ts* src = &PANO_AT(T, (long long)ys * pitchT + xs, (long long)h * pitchT, 110);
-            if constexpr (kAsyncT) copy_async4(&PANO_AT(sTS, i, NTS, 111), src);
-            else PANO_AT(sTS, i, NTS, 111) = ld_f32(src);
-        }
-        if (stage_flow) {
-            const int cy0 = a0n >> 1, cx0 = ox >> 1;
-            for (int i = wi; i < FSH * FSW; i += nw) {
-                const int r = i / FSW, cc = i - r * FSW;
-                const int ys = min(max(cy0 + r, 0), a.in_h - 1), xs = min(max(cx0 + cc, 0), a.in_w - 1);
-                copy_async8(&PANO_AT(sFS, i, NFS, 112),
-                            &PANO_AT(ucoarse, (long long)ys * D.uin_pitch + xs, (long long)a.in_h * D.uin_pitch, 113));
-            }
+    // ---- stage the template and the target box, with clamped borders
+    auto stage = [&](const Ts* __restrict__ src, int pitch, int bx, int by, float* dst, int dp, int n, int rows, int site) {
+        (void)site;
+        constexpr int NC = (RW + 2 * kMX + 31) / 32;
+        int xs[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) xs[c] = min(max(bx + lane + 32 * c, 0), w - 1);
+        for (int r = warp; r < rows; r += WX * WY) {
+            const Ts* row = src + (long long)min(max(by + r, 0), h - 1) * pitch;
+            float* d = dst + r * dp + lane;
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+                if (lane + 32 * c < n) {
+                    if constexpr (kAsync) copy_async4(d + 32 * c, row + PANO_IDX(xs[c], w, site));
+                    else d[32 * c] = ld_f32(row + PANO_IDX(xs[c], w, site));
+                }
         }
         copy_async_commit();
     };
-
-    const int c_first = -((2 * K * RAD + CH - 1) / CH);
-    const int c_last = (Y1 - Y0 + CH - 1) / CH - 1;
-    stage_inputs(Y0 + K * RAD + c_first * CH, tid, kStreamThreads);
-    // Rings start at zero: the column sums of the first chunk read ring rows
-    // that no earlier chunk wrote (their results are discarded, but must
-    // stay finite).
-    for (int i = tid; i < K * 2 * RAD * RW; i += kStreamThreads) PANO_AT(sH, i, NHIST, 114) = make_float2(0.f, 0.f);
-    for (int i = tid; i < kRing * RW; i += kStreamThreads) {
-        PANO_AT(sT, i, NR, 115) = 0.f;
-        PANO_AT(sG, i, NR, 116) = make_float2(0.f, 0.f);
-        PANO_AT(sU, i, NR, 117) = make_float2(0.f, 0.f);
-    }
+    stage(T, D.pitchT, ox - 1, oy - (RAD + 1), sT + 1, TP, RW + 3, TH, 110);
+    // reference flow of the cluster; box shift of the CTA
+    const float2 ref = start_flow_s(a, D, min(ox + RW / 2, w - 1), min(oyc + csize * RH / 2, h - 1));
+    const float2 sh = floor_clamped(start_flow_s(a, D, min(ox + RW / 2, w - 1), min(oy + RH / 2, h - 1)), w, h);
+    const float2 off = make_float2(ref.x - sh.x, ref.y - sh.y);
+    stage(J, D.pitchJ, ox + (int)sh.x - kMX, oy + (int)sh.y - kMY, sJ, JP, RW + 2 * kMX, JH, 111);
+    // the box's unused last column marks samples that fall outside the box
+    if (tid < 4 * WY) bar_init((unsigned)__cvta_generic_to_shared(smem + Geo::kB) + 8 * tid);
+    if (tid < JH) PANO_AT(sJ, tid * JP + JP - 1, NJ, 112) = __int_as_float(0x7fffffff);
     {
-        // target rows of the first chunk
-        const int a0f = Y0 + K * RAD + c_first * CH;
-        const int yb = a0f - (K - 1) * RAD + box.fref_y - kMY;
-        const int n = ((K - 1) * RAD + CH + 2 * kMY + 1) * JW;
-        for (int i = tid; i < n; i += kStreamThreads) {
-            const int yy = i / JW, bc = i - yy * JW;
-            const int yj = yb + yy;
-            const int ys = min(max(yj, 0), h - 1), xs = min(max(jx0 + bc, 0), w - 1);
-            PANO_AT(sJ, ring_slot(yj) * JW + bc, NJ, 118) =
-                ld_f32(&PANO_AT(box.J, (long long)ys * box.pitchJ + xs, (long long)h * box.pitchJ, 119));
-        }
+        const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = tid; i < NO; i += Geo::threads) PANO_AT(sO, i, NO, 113) = z4;
+        for (int i = tid; i < 4 * RH; i += Geo::threads)
+            PANO_AT(sV, (i >> 2) * VP + ((i & 3) < 2 ? (i & 3) : NP + (i & 3)), NV, 114) = z4;
     }
-    copy_async_wait_all();
+    // pixels outside the image have no gradient, and count nowhere
+    const bool edge = oy < RAD || oy + RH + RAD > h || ox + RW > w;
+    const bool cin0 = x0 < w, cin1 = x0 + 1 < w;
+    auto row_in = [&](int j) { return (unsigned)(y0 + dr * j) < (unsigned)h; };
+
+    copy_async_wait<1>();
     __syncthreads();
 
-    for (int c = c_first; c <= c_last; ++c) {
-        const int a0 = Y0 + K * RAD + c * CH;  // newest rows [a0, a0 + CH)
-        // ---- X_0: state of the new rows and the products of stage 1
-        for (int i = tid; i < 2 * RAD * RW; i += kStreamThreads) PANO_AT(sP, i, NP, 120) = PANO_AT(sH, i, NHIST, 121);
+    // ---- template, gradient and the normal matrices
+    float2 t[R], gx[R], gy[R];
+    {
+        float2 q11[R + 2 * RAD], q12[R + 2 * RAD], q22[R + 2 * RAD];
         {
-            const int y = a0 + ty;
-            const bool row_in = y >= 0 && y < h;
-            const int srow = ring_slot(y) * RW;
-            const int tso = (ty + 1) * TSW + 1;  // staged row of y: column rx at sTS[tso + rx]
-            const int cy0 = a0 >> 1, cx0 = ox >> 1;
-            const int fr0 = (y >> 1) - cy0;               // staged coarse row of y / 2
-            const float fy = (y & 1) ? 0.5f : 0.f;
-            const int pro = (2 * RAD + ty) * RW;  // this row's products at sP[pro + rx]
-            for (int rx = tx; rx < RW; rx += TX) {
-                const int x = ox + rx;
-                float t = 0.f;
-                float2 g = make_float2(0.f, 0.f), u = make_float2(0.f, 0.f), P = make_float2(0.f, 0.f);
-                if (row_in && rx >= cmin && rx < cmax) {
-                    t = PANO_AT(sTS, tso + rx, NTS, 122);
-                    g.x = 0.5f * (PANO_AT(sTS, tso + rx + 1, NTS, 123) - PANO_AT(sTS, tso + rx - 1, NTS, 124));
-                    g.y = 0.5f * (PANO_AT(sTS, tso + rx + TSW, NTS, 125) - PANO_AT(sTS, tso + rx - TSW, NTS, 126));
-                    float2 u0;
-                    if (stage_flow) {
-                        // 2 * bilinear(u_coarse)(x/2, y/2) from the staged rows
-                        const int fc0 = (x >> 1) - cx0;
-                        const float fx = (x & 1) ? 0.5f : 0.f;
-                        const int f0 = fr0 * FSW + fc0, f1 = f0 + FSW;
-                        const float2 u00 = PANO_AT(sFS, f0, NFS, 127), u10 = PANO_AT(sFS, f0 + 1, NFS, 128);
-                        const float2 u01 = PANO_AT(sFS, f1, NFS, 129), u11 = PANO_AT(sFS, f1 + 1, NFS, 130);
-                        const float tx0 = fmaf(fx, u10.x - u00.x, u00.x), bx0 = fmaf(fx, u11.x - u01.x, u01.x);
-                        const float ty0 = fmaf(fx, u10.y - u00.y, u00.y), by0 = fmaf(fx, u11.y - u01.y, u01.y);
-                        u0 = make_float2(2.f * fmaf(fy, bx0 - tx0, tx0), 2.f * fmaf(fy, by0 - ty0, ty0));
-                    } else {
-                        u0 = start_flow_s(a, D, x, y);
-                    }
-                    u = make_float2(u0.x - ref.x, u0.y - ref.y);
-                    P = residual_product<JW, Ts>(box, x, y, rx, ref, u, g, t);
+            const int to = (r0 + RAD + 1) * TP + 2 + rx, dt = dr * TP;  // row 0 of the run
+            const float2 hs = dup2(half ? -0.5f : 0.5f);
+            float2 pv = PANO_VEC(const float2, sT, to - (RAD + 1) * dt, 2, NT, 115);
+            float2 cv = PANO_VEC(const float2, sT, to - RAD * dt, 2, NT, 116);
+#pragma unroll
+            for (int i = -RAD; i < R + RAD; ++i) {
+                const float2 nv = PANO_VEC(const float2, sT, to + (i + 1) * dt, 2, NT, 117);
+                const float lf = PANO_AT(sT, to + i * dt - 1, NT, 118), rt = PANO_AT(sT, to + i * dt + 2, NT, 119);
+                float2 hx = make_float2(0.5f * (cv.y - lf), 0.5f * (rt - cv.x)), hy = mul2(hs, sub2(nv, pv));
+                if (edge) {
+                    const bool in = row_in(i);
+                    if (!(in && cin0)) hx.x = hy.x = 0.f;
+                    if (!(in && cin1)) hx.y = hy.y = 0.f;
                 }
-                PANO_AT(sT, srow + rx, NR, 131) = t;
-                PANO_AT(sG, srow + rx, NR, 132) = g;
-                PANO_AT(sU, srow + rx, NR, 133) = u;
-                PANO_AT(sP, pro + rx, NP, 134) = P;
+                if (i >= 0 && i < R) t[i] = cv, gx[i] = hx, gy[i] = hy;
+                q11[i + RAD] = mul2(hx, hx);
+                q12[i + RAD] = mul2(hx, hy);
+                q22[i + RAD] = mul2(hy, hy);
+                pv = cv;
+                cv = nv;
             }
         }
-        __syncthreads();
-        // the staging buffers are free again: every thread starts fetching
-        // part of the next chunk's inputs
-        if (c < c_last) stage_inputs(a0 + CH, tid, kStreamThreads);
-        // ---- B_1: column sums of stage 1 (two threads per column, the
-        //      column's values read once into registers) and its history;
-        //      column sums of grad T grad T^T for the normal matrices of rows
-        //      [a1, a1 + CH)
-        if (tid < 2 * RW) {
-            const int part = tid >= RW;
-            column_sums<RAD, CH, RW, 2>(sP, sV, sH, tid - part * RW, part);
-        } else if (tid >= kCsT0 && tid < kCsT0 + 2 * RW) {
-            // normal-matrix column sums: two threads per column, CH/2 rows each
-            const int rx = (tid - kCsT0) % RW, half = (tid - kCsT0) / RW;
-            constexpr int HC = CH / 2;
-            const int yb = a0 - 2 * RAD + half * HC;   // first ring row of this half's windows
-            float2 g[HC + 2 * RAD];
+        float2 c11[R], c12[R], c22[R];
+        window_sums<RAD, R>(q11, c11);
+        window_sums<RAD, R>(q12, c12);
+        window_sums<RAD, R>(q22, c22);
+        __syncthreads();  // the template is read
 #pragma unroll
-            for (int d = 0; d < HC + 2 * RAD; ++d) g[d] = PANO_AT(sG, ring_slot(yb + d) * RW + rx, NR, 135);
-#pragma unroll
-            for (int yy = 0; yy < HC; ++yy) {
-                float2 c1 = make_float2(0.f, 0.f);  // (c11, c12)
-                float c22 = 0.f;
-#pragma unroll
-                for (int d = 0; d <= 2 * RAD; ++d) {
-                    c1 = fma2(make_float2(g[yy + d].x, g[yy + d].x), g[yy + d], c1);
-                    c22 = fmaf(g[yy + d].y, g[yy + d].y, c22);
-                }
-                const int o = (half * HC + yy) * RW + rx;
-                PANO_AT(sCSA, o, NCH, 136) = c1;
-                PANO_AT(sCSB, o, NCH, 137) = c22;
-            }
+        for (int j = 0; j < R; ++j) {
+            const int o = (srow + j) * NP + px;
+            PANO_AT(sGA, o, NG, 120) = make_float4(c11[j].x, c11[j].y, c12[j].x, c12[j].y);
+            PANO_AT(sGB, o, NG, 121) = c22[j];
         }
-        __syncthreads();
+        named_barrier<32 * WX>(1 + wy);
+        const bool hl = px > 0, hr = px + 1 < NP;                     // neighbouring pairs inside the region
+        const bool hl2 = px > 1 && RAD == 3, hr2 = px + 2 < NP && RAD == 3;
 #pragma unroll
-        for (int k = 1; k <= K; ++k) {
-            const int c0 = k * RAD;            // columns [c0, RW - c0)
-            if (k == K) {
-                // target rows that the next chunk's products reach for the
-                // first time: asynchronous copies, issued first so that they
-                // overlap this phase (no products are sampled in it)
-                const int yj = a0 + CH + box.fref_y + kMY + 1 + ty;
-                const long long jso = (long long)min(max(yj, 0), h - 1) * box.pitchJ;  // source row
-                const long long NJG = (long long)h * box.pitchJ;
-                (void)NJG;
-                if constexpr (kAsyncT) {
-                    const int jdo = ring_slot(yj) * JW;
-                    for (int bc = tx; bc < JW; bc += TX)
-                        copy_async4(&PANO_AT(sJ, jdo + bc, NJ, 138),
-                                    &PANO_AT(box.J, jso + min(max(jx0 + bc, 0), w - 1), NJG, 139));
-                    copy_async_commit();
-                } else {
-#pragma unroll
-                    for (int q = 0; q < kJPT; ++q) {
-                        const int bc = tx + q * TX;
-                        jnext[q] = bc < JW ? ld_f32(&PANO_AT(box.J, jso + min(max(jx0 + bc, 0), w - 1), NJG, 139)) : 0.f;
-                    }
-                }
+        for (int j = 0; j < R; ++j) {
+            const int o = (srow + j) * NP + px;
+            const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float2 z2 = make_float2(0.f, 0.f);
+            const float4 l = hl ? PANO_AT(sGA, o - 1, NG, 122) : z4, r = hr ? PANO_AT(sGA, o + 1, NG, 123) : z4;
+            const float2 lb = hl ? PANO_AT(sGB, o - 1, NG, 124) : z2, rb = hr ? PANO_AT(sGB, o + 1, NG, 125) : z2;
+            float4 l2 = z4, r2 = z4;
+            float2 lb2 = z2, rb2 = z2;
+            if constexpr (RAD == 3) {
+                if (hl2) l2 = PANO_AT(sGA, o - 2, NG, 126), lb2 = PANO_AT(sGB, o - 2, NG, 127);
+                if (hr2) r2 = PANO_AT(sGA, o + 2, NG, 128), rb2 = PANO_AT(sGB, o + 2, NG, 129);
             }
-            // ---- X_k: row sums, solve, update; products of stage k+1
-            if (k < K) {
-                const int hko = k * 2 * RAD * RW;  // this stage's history in sH
-                const int width = RW - 2 * c0;
-                for (int i = tid; i < 2 * RAD * width; i += kStreamThreads) {
-                    const int yy = i / width, rx = c0 + (i - yy * width);
-                    PANO_AT(sP, yy * RW + rx, NP, 140) = PANO_AT(sH, hko + yy * RW + rx, NHIST, 141);
-                }
-            }
-            {
-                // this thread: row ty of stage k, the column pair (xp, xp + 1)
-                constexpr int HR = (RAD + 1) / 2 * 2;      // even halo >= RAD
-                constexpr int NPAIR = (2 * HR + 2) / 2;     // float4 loads for the row sums
-                const int c0e = c0 & ~1;
-                const int xp = c0e + 2 * tx;
-                const int y = a0 - k * RAD + ty;
-                const bool row_in = y >= 0 && y < h;
-                const bool on0 = xp >= c0 && xp < RW - c0, on1 = xp + 1 >= c0 && xp + 1 < RW - c0;
-                if (xp < RW - c0) {
-                    const int srow = ring_slot(y) * RW;
-                    const bool in0 = on0 && row_in && xp >= cmin && xp < cmax;
-                    const bool in1 = on1 && row_in && xp + 1 >= cmin && xp + 1 < cmax;
-                    // row sums of the column sums for both pixels
-                    const int vqo = ty * RW + xp - HR;  // first column pair at sV[vqo]
-                    float2 vv[2 * HR + 2];
+            c11[j] = row_sums<RAD>(l2.y, make_float2(l.x, l.y), c11[j], make_float2(r.x, r.y), r2.x);
+            c12[j] = row_sums<RAD>(l2.w, make_float2(l.z, l.w), c12[j], make_float2(r.z, r.w), r2.z);
+            c22[j] = row_sums<RAD>(lb2.y, lb, c22[j], rb, rb2.x);
+        }
+        named_barrier<32 * WX>(1 + wy);
+        const float2 lam2 = dup2(a.lambda);
 #pragma unroll
-                    for (int q = 0; q < NPAIR; ++q) {
-                        const float4 t4 = PANO_VEC(const float4, sV - Geo::kPad, vqo + 2 * q + Geo::kPad, 2,
-                                                   NCH + 2 * Geo::kPad, 142);
-                        vv[2 * q] = make_float2(t4.x, t4.y);
-                        vv[2 * q + 1] = make_float2(t4.z, t4.w);
-                    }
-                    float2 m0 = vv[HR - RAD], m1 = vv[HR - RAD + 1];
-#pragma unroll
-                    for (int d = 1; d <= 2 * RAD; ++d) {
-                        m0 = add2(m0, vv[HR - RAD + d]);
-                        m1 = add2(m1, vv[HR - RAD + d + 1]);
-                    }
-                    float2 ga0, ga1;
-                    float gb0, gb1;
-                    if (k == 1) {
-                        const int co = ty * RW + xp;  // column sums of column xp at sCSA[co], sCSB[co]
-                        float2 a1 = make_float2(0.f, 0.f), b1 = make_float2(0.f, 0.f);  // (x11, x12)
-                        float a22 = 0.f, b22 = 0.f;
-#pragma unroll
-                        for (int d = -RAD; d <= RAD; ++d) {
-                            constexpr int NCP = NCH + 2 * Geo::kPad, PD = Geo::kPad;
-                            a1 = add2(a1, PANO_AT(sCSA - PD, co + d + PD, NCP, 143));
-                            a22 += PANO_AT(sCSB - PD, co + d + PD, NCP, 144);
-                            b1 = add2(b1, PANO_AT(sCSA - PD, co + d + 1 + PD, NCP, 145));
-                            b22 += PANO_AT(sCSB - PD, co + d + 1 + PD, NCP, 146);
-                        }
-                        const float a11 = a1.x, a12 = a1.y, b11 = b1.x, b12 = b1.y;
-                        const float p11 = a11 + lam, p22 = a22 + lam;
-                        const float ip = 1.0f / (p11 * p22 - a12 * a12);
-                        const float q11 = b11 + lam, q22 = b22 + lam;
-                        const float iq = 1.0f / (q11 * q22 - b12 * b12);
-                        ga0 = make_float2(p22 * ip, -a12 * ip);
-                        gb0 = p11 * ip;
-                        ga1 = make_float2(q22 * iq, -b12 * iq);
-                        gb1 = q11 * iq;
-                        PANO_VEC(float4, sGiA, srow + xp, 2, NR, 147) = make_float4(ga0.x, ga0.y, ga1.x, ga1.y);
-                        PANO_VEC(float2, sGiB, srow + xp, 2, NR, 148) = make_float2(gb0, gb1);
-                    } else {
-                        const float4 a4 = PANO_VEC(const float4, sGiA, srow + xp, 2, NR, 149);
-                        const float2 b2 = PANO_VEC(const float2, sGiB, srow + xp, 2, NR, 150);
-                        ga0 = make_float2(a4.x, a4.y);
-                        ga1 = make_float2(a4.z, a4.w);
-                        gb0 = b2.x;
-                        gb1 = b2.y;
-                    }
-                    const float4 u4 = PANO_VEC(const float4, sU, srow + xp, 2, NR, 151);
-                    float2 v0 = make_float2(u4.x, u4.y), v1 = make_float2(u4.z, u4.w);
-                    const float2 lam2 = make_float2(lam, lam);
-                    if (in0) {
-                        const float2 r = fma2(lam2, v0, m0);
-                        v0 = fma2(ga0, make_float2(r.x, r.x), mul2(make_float2(ga0.y, gb0), make_float2(r.y, r.y)));
-                    }
-                    if (in1) {
-                        const float2 r = fma2(lam2, v1, m1);
-                        v1 = fma2(ga1, make_float2(r.x, r.x), mul2(make_float2(ga1.y, gb1), make_float2(r.y, r.y)));
-                    }
-                    PANO_VEC(float4, sU, srow + xp, 2, NR, 152) = make_float4(v0.x, v0.y, v1.x, v1.y);
-                    if (k == K) {
-                        if (row_in && y >= Y0 && y < Y1) {
-                            float2* uo = reinterpret_cast<float2*>(D.uout);
-                            const long long uoo = (long long)y * D.uout_pitch + ox + xp;
-                            const long long NUO = (long long)h * D.uout_pitch;
-                            (void)NUO;
-                            if (in0 && xp >= K * RAD && xp < K * RAD + BW) PANO_AT(uo, uoo, NUO, 153) = add2(v0, ref);
-                            if (in1 && xp + 1 >= K * RAD && xp + 1 < K * RAD + BW)
-                                PANO_AT(uo, uoo + 1, NUO, 154) = add2(v1, ref);
-                        }
-                    } else {
-                        // products of stage k+1 at the same two pixels
-                        const float4 g4 = PANO_VEC(const float4, sG, srow + xp, 2, NR, 155);
-                        const float2 t2 = PANO_VEC(const float2, sT, srow + xp, 2, NR, 156);
-                        float2 P0 = make_float2(0.f, 0.f), P1 = make_float2(0.f, 0.f);
-                        if (in0) P0 = residual_product<JW, Ts>(box, ox + xp, y, xp, ref, v0, make_float2(g4.x, g4.y), t2.x);
-                        if (in1) P1 = residual_product<JW, Ts>(box, ox + xp + 1, y, xp + 1, ref, v1, make_float2(g4.z, g4.w), t2.y);
-                        PANO_VEC(float4, sP, (2 * RAD + ty) * RW + xp, 2, NP, 157) = make_float4(P0.x, P0.y, P1.x, P1.y);
-                    }
-                }
+        for (int j = 0; j < R; ++j) {
+            const int o = (srow + j) * NP + px;
+            const float2 p11 = add2(c11[j], lam2), p22 = add2(c22[j], lam2);
+            const float2 det = fma2(p11, p22, mul2(c12[j], make_float2(-c12[j].x, -c12[j].y)));
+            float2 iv = make_float2(1.0f / det.x, 1.0f / det.y);
+            float2 i11 = mul2(p22, iv), i12 = mul2(c12[j], make_float2(-iv.x, -iv.y)), i22 = mul2(p11, iv);
+            if (edge) {
+                // pixels outside the image keep a zero (relative) flow
+                const bool in = row_in(j);
+                if (!(in && cin0)) i11.x = i12.x = i22.x = 0.f;
+                if (!(in && cin1)) i11.y = i12.y = i22.y = 0.f;
             }
-            if (k == K) {
-                // the coarse-flow rows (and for float planes the template and
-                // target rows) copied asynchronously since B_1
-                copy_async_wait_all();
-                if constexpr (!kAsyncT) {
-                    // the target loads issued before X_K land in the ring now
-                    const int yj = a0 + CH + box.fref_y + kMY + 1 + ty;
-                    const int jdo = ring_slot(yj) * JW;
-#pragma unroll
-                    for (int q = 0; q < kJPT; ++q) {
-                        const int bc = tx + q * TX;
-                        if (bc < JW) PANO_AT(sJ, jdo + bc, NJ, 158) = jnext[q];
-                    }
-                }
-            }
-            __syncthreads();
-            if (k < K) {
-                // ---- B_{k+1}: column sums of stage k+1 and its history (two
-                //      threads per column)
-                const int ncol = RW - 2 * c0;
-                if (tid < 2 * ncol) {
-                    const int part = tid >= ncol;
-                    column_sums<RAD, CH, RW, 2>(sP, sV, sH + (size_t)k * 2 * RAD * RW, c0 + tid - part * ncol, part);
-                }
-                __syncthreads();
-            }
+            PANO_AT(sGA, o, NG, 130) = make_float4(i11.x, i11.y, i12.x, i12.y);
+            PANO_AT(sGB, o, NG, 131) = i22;
         }
     }
-}
 
-template <int RAD, int K, int BW, int CH, class Ts>
-__global__ void __launch_bounds__(kStreamThreads, 1) lk_stream_kernel(const __grid_constant__ LkArgs a, int seg) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    lk_stream_item<RAD, K, BW, CH, Ts>(a, blockIdx.z, blockIdx.x, blockIdx.y, seg, smem);
-}
-
-// Persistent form over several strip pairs at once: a fixed grid of CTAs
-// takes (pair, direction, band, segment) items from an atomic counter until
-// none are left. The counter only hands out indices; nothing waits on it.
-template <int RAD, int K, int BW, int CH, class Ts>
-__global__ void __launch_bounds__(kStreamThreads, 1) lk_stream_batch_kernel(const __grid_constant__ LkBatch b) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int s_item;
-    for (;;) {
-        if (threadIdx.x == 0) s_item = (int)atomicAdd(b.counter, 1u);
-        __syncthreads();
-        const int item = s_item;
-        __syncthreads();
-        if (item >= b.start[b.n]) break;
-        int p = 0;
-        while (p + 1 < b.n && item >= b.start[p + 1]) ++p;
-        const int local = item - b.start[p];
-        const int per_dir = b.nb[p] * b.nseg[p];
-        const int dir = local / per_dir, rem = local - dir * per_dir;
-        const int by = rem / b.nb[p], bx = rem - by * b.nb[p];
-        lk_stream_item<RAD, K, BW, CH, Ts>(b.pair[p], dir, bx, by, b.seg[p], smem);
-        __syncthreads();
-    }
-}
-
-// Segment height and count for one level: about 256+ rows per segment (the
-// first chunks of a segment are discarded work), in whole waves of one CTA
-// per SM; seg_rows > 0 overrides the target height. (On the 4000 x 1500
-// pair's level 0 that is 3 waves of 286-row segments; 4 waves of 211 rows
-// measured 0.8% slower for the step, 2 waves of 445 rows 1.6% slower.)
-template <int CH>
-void stream_segments(int h, int per_row, int seg_rows, int* seg_out, int* nseg_out) {
-    const int sms = 152;
-    int seg;
-    if (seg_rows > 0) {
-        seg = seg_rows;
+    // ---- starting flow, relative to the reference
+    float2 ux[R], uy[R];
+    if (a.mode == 1 && D.uin != nullptr) {
+        // x and y of the run's first pixel pair (in image order) are even: the
+        // fine rows lie on or between NE coarse rows, e[i] in run order
+        // (downwards in the upper half, upwards in the lower one)
+        constexpr int NE = (R - 1) / 2 + 2;
+        const float2* __restrict__ uc = reinterpret_cast<const float2*>(D.uin);
+        const int xa = min(x0 >> 1, a.in_w - 1), xb = min((x0 >> 1) + 1, a.in_w - 1);
+        const int cy = (oy + wy * 2 * R) / 2 + (half ? R : 0);
+        const long long NUI = (long long)(a.in_h - 1) * D.uin_pitch + a.in_w;
+        (void)NUI;
+        float2 ex[NE], ey[NE];
+#pragma unroll
+        for (int i = 0; i < NE; ++i) {
+            const long long ro = (long long)min(cy + dr * i, a.in_h - 1) * D.uin_pitch;
+            const float2 ua = PANO_AT(uc, ro + xa, NUI, 132), ub = PANO_AT(uc, ro + xb, NUI, 133);
+            ex[i] = fma2(make_float2(0.f, 0.5f), dup2(ub.x - ua.x), dup2(ua.x));
+            ey[i] = fma2(make_float2(0.f, 0.5f), dup2(ub.y - ua.y), dup2(ua.y));
+        }
+        const float2 rx2 = dup2(-ref.x), ry2 = dup2(-ref.y);
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            const float2 fy = dup2(((j ^ half) & 1) ? 0.5f : 0.f);
+            const float2 px_ = ex[j >> 1], qx = ex[(j >> 1) + 1], py_ = ey[j >> 1], qy = ey[(j >> 1) + 1];
+            const float2 tx = half ? qx : px_, bx = half ? px_ : qx, ty = half ? qy : py_, by = half ? py_ : qy;
+            ux[j] = fma2(dup2(2.f), fma2(fy, sub2(bx, tx), tx), rx2);
+            uy[j] = fma2(dup2(2.f), fma2(fy, sub2(by, ty), ty), ry2);
+        }
     } else {
-        long long waves = (long long)per_row * h / (256LL * sms);
-        if (waves < 1) waves = 1;
-        int nseg = (int)(waves * sms / per_row);
-        if (nseg < 1) nseg = 1;
-        seg = (h + nseg - 1) / nseg;
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            const int y = min(y0 + dr * j, h - 1);
+            const float2 s0 = start_flow_s(a, D, min(x0, w - 1), y), s1 = start_flow_s(a, D, min(x0 + 1, w - 1), y);
+            ux[j] = make_float2(s0.x - ref.x, s1.x - ref.x);
+            uy[j] = make_float2(s0.y - ref.y, s1.y - ref.y);
+        }
     }
-    if (seg < 2 * CH) seg = 2 * CH;
-    *seg_out = seg;
-    *nseg_out = (h + seg - 1) / seg;
+    if (edge) {
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            const bool in = row_in(j);
+            if (!(in && cin0)) ux[j].x = uy[j].x = 0.f;
+            if (!(in && cin1)) ux[j].y = uy[j].y = 0.f;
+        }
+    }
+
+    // Where this run's outer rows go: the run above (upper half) or below
+    // (lower half), in this CTA or its neighbour; none at the cluster's ends.
+    // Every halo has a barrier that counts its bytes, one per parity of the
+    // step: a run goes on as soon as its own two neighbours have sent. A halo
+    // is overwritten two steps later, when the sender has received what its
+    // reader sent after reading it.
+    const int nwy = half ? wy + 1 : wy - 1;
+    const int nrank = nwy < 0 ? rank - 1 : nwy >= WY ? rank + 1 : rank;
+    const bool send = nrank >= 0 && nrank < csize;
+    const int nslot = ((nwy + WY) % WY) * 2 + (half ^ 1);
+    const unsigned so = (unsigned)__cvta_generic_to_shared(sO), sb = (unsigned)__cvta_generic_to_shared(smem + Geo::kB);
+    const unsigned odst = cluster_map(so + (nslot * RAD * NP + px) * (unsigned)sizeof(float4), (unsigned)(send ? nrank : rank));
+    const unsigned bdst = cluster_map(sb + nslot * 8, (unsigned)(send ? nrank : rank));
+    const int oslot = ((wy * 2 + half) * RAD) * NP + px;  // this run's outer halo
+    const bool from_above = wy > 0 || rank > 0, from_below = wy + 1 < WY || rank + 1 < csize;
+    const unsigned bown = sb + wy * 16;  // this warp's barriers: above, below
+    constexpr unsigned kHaloBytes = RAD * NP * sizeof(float4);
+    bool lost = false;
+    // Sample position: 1.5 * 2^23 + position, rounded down, holds the tap's
+    // column / row of the box in its low mantissa bits (its bits are those of
+    // 1.5 * 2^23 plus the integer, exact while |o| < 2^21).
+    constexpr float kMagic = 12582912.0f;
+    const float2 mgx = make_float2(kMagic + (float)(rx + kMX), kMagic + (float)(rx + 1 + kMX));
+    const float mgy0 = kMagic + (float)(r0 + kMY), mgd = (float)dr;
+    const unsigned sj = (unsigned)__cvta_generic_to_shared(sJ);
+    const unsigned jbase = sj - 4u * (0x4B400000u * (unsigned)(JP + 1)), jnone = sj + 4u * (JP - 1);
+    const float2 offx = dup2(off.x), offy = dup2(off.y), lam2 = dup2(a.lambda);
+    const int vo = srow * VP + 2 + px, go = srow * NP + px;
+
+    copy_async_wait<0>();
+    if (wx == 0 && lane == 0) {
+        // the barriers were initialised before the __syncthreads above
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            if (from_above) bar_expect(bown + q * (WY * 16), kHaloBytes);
+            if (from_below) bar_expect(bown + q * (WY * 16) + 8, kHaloBytes);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+    cluster_arrive();  // the staged target and the barriers are visible, the zeroed halos come before a neighbour's rows
+    cluster_wait();
+
+#pragma unroll 1
+    for (int k = 0; k < a.iters; ++k) {
+        float2 Px[R], Py[R];
+        // ---- A: residual products of rows [JB, JE)
+        auto products = [&](auto jb, auto je) {
+            constexpr int JB = decltype(jb)::value, JE = decltype(je)::value;
+            float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int j = JB; j < JE; ++j) {
+                // J at the pixel + ref + u
+                const float2 o_x = add2(offx, ux[j]), o_y = add2(offy, uy[j]);
+                const float my = fmaf((float)j, mgd, mgy0);
+                const float2 tx = make_float2(__fadd_rd(o_x.x, mgx.x), __fadd_rd(o_x.y, mgx.y));
+                const float2 ty = make_float2(__fadd_rd(o_y.x, my), __fadd_rd(o_y.y, my));
+                const float2 ax = sub2(o_x, sub2(tx, mgx)), ay = sub2(o_y, sub2(ty, dup2(my)));
+                unsigned p0 = (__float_as_uint(ty.x) * (unsigned)JP + __float_as_uint(tx.x)) * 4u + jbase;
+                unsigned p1 = (__float_as_uint(ty.y) * (unsigned)JP + __float_as_uint(tx.y)) * 4u + jbase;
+                // a sample outside the box reads the marker instead
+                p0 = fabsf(o_x.x) < (float)kMX && fabsf(o_y.x) < (float)kMY ? p0 : jnone;
+                p1 = fabsf(o_x.y) < (float)kMX && fabsf(o_y.y) < (float)kMY ? p1 : jnone;
+                PANO_FLAG(p0 - sj > 4u * (NJ - JP - 2) || p1 - sj > 4u * (NJ - JP - 2), 140);
+                const float2 i00 = make_float2(ld_shared<0>(p0), ld_shared<0>(p1));
+                const float2 i10 = make_float2(ld_shared<4>(p0), ld_shared<4>(p1));
+                const float2 i01 = make_float2(ld_shared<4 * JP>(p0), ld_shared<4 * JP>(p1));
+                const float2 i11 = make_float2(ld_shared<4 * JP + 4>(p0), ld_shared<4 * JP + 4>(p1));
+                const float2 top = fma2(ax, sub2(i10, i00), i00), bot = fma2(ax, sub2(i11, i01), i01);
+                const float2 jw = fma2(ay, sub2(bot, top), top);
+                float2 s = fma2(gx[j], ux[j], fma2(gy[j], uy[j], sub2(t[j], jw)));
+                if (edge) {  // nothing from outside the image
+                    const bool in = row_in(j);
+                    if (!(in && cin0)) s.x = 0.f;
+                    if (!(in && cin1)) s.y = 0.f;
+                }
+                acc = add2(acc, s);
+                Px[j] = mul2(gx[j], s);
+                Py[j] = mul2(gy[j], s);
+            }
+            if (__builtin_expect(!(acc.x + acc.y == acc.x + acc.y), 0)) {
+                // some samples (or their inputs) are not numbers: those outside
+                // the box are taken from the global plane
+#pragma unroll
+                for (int j = JB; j < JE; ++j)
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        const float vx = c ? ux[j].y : ux[j].x, vy = c ? uy[j].y : uy[j].x;
+                        const float o_x = off.x + vx, o_y = off.y + vy;
+                        if ((fabsf(o_x) < (float)kMX && fabsf(o_y) < (float)kMY) || !row_in(j) || !(c ? cin1 : cin0)) continue;
+                        const float jw = far_sample(J, D.pitchJ, w, h, x0 + c, y0 + dr * j, ref.x + vx, ref.y + vy);
+                        const float hx = c ? gx[j].y : gx[j].x, hy = c ? gy[j].y : gy[j].x;
+                        const float s = fmaf(hx, vx, fmaf(hy, vy, (c ? t[j].y : t[j].x) - jw));
+                        (c ? Px[j].y : Px[j].x) = hx * s;
+                        (c ? Py[j].y : Py[j].x) = hy * s;
+                    }
+            }
+        };
+        // ---- C: row sums, solve, update of row j with column sums (vx, vy)
+        auto update = [&](int j, float2 vx, float2 vy) {
+            const float4 l = PANO_AT(sV, vo + j * VP - 1, NV, 146), r = PANO_AT(sV, vo + j * VP + 1, NV, 147);
+            float4 l2 = make_float4(0.f, 0.f, 0.f, 0.f), r2 = l2;
+            if constexpr (RAD == 3) {
+                l2 = PANO_AT(sV, vo + j * VP - 2, NV, 148);
+                r2 = PANO_AT(sV, vo + j * VP + 2, NV, 149);
+            }
+            const float2 mx = row_sums<RAD>(l2.y, make_float2(l.x, l.y), vx, make_float2(r.x, r.y), r2.x);
+            const float2 my = row_sums<RAD>(l2.w, make_float2(l.z, l.w), vy, make_float2(r.z, r.w), r2.z);
+            const float4 ga = PANO_AT(sGA, go + j * NP, NG, 152);
+            const float2 gb = PANO_AT(sGB, go + j * NP, NG, 153), g11 = make_float2(ga.x, ga.y), g12 = make_float2(ga.z, ga.w);
+            const float2 qx = fma2(lam2, ux[j], mx), qy = fma2(lam2, uy[j], my);
+            ux[j] = fma2(g11, qx, mul2(g12, qy));
+            uy[j] = fma2(g12, qx, mul2(gb, qy));
+        };
+
+        // the outer rows first: they are on their way while the others are formed
+        products(std::integral_constant<int, 0>{}, std::integral_constant<int, RAD>{});
+        if (send) {
+#pragma unroll
+            for (int j = 0; j < RAD; ++j)
+                cluster_send(odst + ((k & 1) * (NO / 2) + j * NP) * (unsigned)sizeof(float4), bdst + (k & 1) * (WY * 16), Px[j], Py[j]);
+        }
+        __syncwarp();
+        // nobody sends any more: no CTA ends before its neighbours are here
+        if (k + 1 == a.iters) cluster_arrive_relaxed();
+        products(std::integral_constant<int, RAD>{}, std::integral_constant<int, R>{});
+        __syncwarp();
+        // ---- B: column sums of the rows that need no outer halo
+        float2 hx[RAD], hy[RAD];  // sums of rows 0 .. i + RAD
+        {
+            float2 e[R + RAD], f[R + RAD];
+#pragma unroll
+            for (int j = 0; j < R; ++j) e[j] = Px[j], f[j] = Py[j];
+#pragma unroll
+            for (int i = 0; i < RAD; ++i) {
+                // the other half's inner rows
+                e[R + i].x = __shfl_xor_sync(0xffffffffu, Px[R - 1 - i].x, 16);
+                e[R + i].y = __shfl_xor_sync(0xffffffffu, Px[R - 1 - i].y, 16);
+                f[R + i].x = __shfl_xor_sync(0xffffffffu, Py[R - 1 - i].x, 16);
+                f[R + i].y = __shfl_xor_sync(0xffffffffu, Py[R - 1 - i].y, 16);
+            }
+            hx[0] = e[0], hy[0] = f[0];
+#pragma unroll
+            for (int i = 1; i <= RAD; ++i) hx[0] = add2(hx[0], e[i]), hy[0] = add2(hy[0], f[i]);
+#pragma unroll
+            for (int i = 1; i < RAD; ++i) hx[i] = add2(hx[i - 1], e[RAD + i]), hy[i] = add2(hy[i - 1], f[RAD + i]);
+            float2 vx[R - RAD], vy[R - RAD];
+            window_sums<RAD, R - RAD>(e, vx);
+            window_sums<RAD, R - RAD>(f, vy);
+#pragma unroll
+            for (int j = RAD; j < R; ++j) {
+                Px[j] = vx[j - RAD], Py[j] = vy[j - RAD];
+                PANO_AT(sV, vo + j * VP, NV, 145) = make_float4(Px[j].x, Px[j].y, Py[j].x, Py[j].y);
+            }
+        }
+        named_barrier<32 * WX>(1 + wy);
+#pragma unroll
+        for (int j = RAD; j < R; ++j) update(j, Px[j], Py[j]);
+        // ---- and of the outer rows, when the neighbours' rows are here
+        {
+            const unsigned bar = bown + (k & 1) * (WY * 16);
+            const unsigned ph = (unsigned)(k >> 1) & 1;
+            if (from_above) lost |= !bar_wait(bar, ph);
+            if (from_below) lost |= !bar_wait(bar + 8, ph);
+            if (wx == 0 && lane == 0 && k + 2 < a.iters) {
+                if (from_above) bar_expect(bar, kHaloBytes);
+                if (from_below) bar_expect(bar + 8, kHaloBytes);
+            }
+            __syncwarp();
+            float2 ex = make_float2(0.f, 0.f), ey = ex;
+#pragma unroll
+            for (int i = RAD - 1; i >= 0; --i) {
+                // row i lacks the halo's first RAD - i rows
+                const float4 o = PANO_AT(sO, (k & 1) * (NO / 2) + oslot + (RAD - 1 - i) * NP, NO, 144);
+                ex = i == RAD - 1 ? make_float2(o.x, o.y) : add2(ex, make_float2(o.x, o.y));
+                ey = i == RAD - 1 ? make_float2(o.z, o.w) : add2(ey, make_float2(o.z, o.w));
+                hx[i] = add2(hx[i], ex), hy[i] = add2(hy[i], ey);
+                PANO_AT(sV, vo + i * VP, NV, 145) = make_float4(hx[i].x, hx[i].y, hy[i].x, hy[i].y);
+            }
+        }
+        named_barrier<32 * WX>(1 + wy);
+#pragma unroll
+        for (int i = 0; i < RAD; ++i) update(i, hx[i], hy[i]);
+    }
+
+    cluster_wait();
+    // ---- the result (not a number where a neighbour's rows never came)
+    float2* uo = reinterpret_cast<float2*>(D.uout);
+    const float2 end = lost ? dup2(__int_as_float(0x7fffffff)) : ref;
+    const bool c0 = x0 >= x_lo && x0 < x_hi, c1 = x0 + 1 >= x_lo && x0 + 1 < x_hi;
+    const long long NUO = (long long)(h - 1) * D.uout_pitch + w;
+    (void)NUO;
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        const int y = y0 + dr * j;
+        if (y < y_lo || y >= y_hi) continue;
+        const long long o = (long long)y * D.uout_pitch + x0;
+        if (c0) PANO_AT(uo, o, NUO, 154) = make_float2(ux[j].x + end.x, uy[j].x + end.y);
+        if (c1) PANO_AT(uo, o + 1, NUO, 155) = make_float2(ux[j].y + end.x, uy[j].y + end.y);
+    }
 }
 
-template <int RAD, int K, int BW, int CH, class Ts>
-cudaError_t launch_one(const LkArgs& a, int ndirs, cudaStream_t s) {
-    using Geo = StreamGeom<RAD, K, BW, CH>;
-    const int nb = (a.w + BW - 1) / BW;
-    int seg = 0, nseg = 0;
-    stream_segments<CH>(a.h, nb * ndirs, a.seg_rows, &seg, &nseg);
-    dim3 grid(nb, nseg, ndirs);
-    lk_stream_kernel<RAD, K, BW, CH, Ts><<<grid, kStreamThreads, Geo::bytes, s>>>(a, seg);
-    return cudaGetLastError();
-}
+// How a level is cut: nb bands, ns segments (clusters) per band of csize CTAs
+// each; `small` selects the CTA shape.
+struct StreamPlan {
+    int nb, ns, csize, small;
+};
 
-template <int RAD, int K, int BW, int CH, class Ts>
-cudaError_t prepare_one(int max_smem) {
-    using Geo = StreamGeom<RAD, K, BW, CH>;
-    if (Geo::bytes > (size_t)max_smem) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(lk_stream_kernel<RAD, K, BW, CH, Ts>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo::bytes);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(lk_stream_batch_kernel<RAD, K, BW, CH, Ts>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo::bytes);
-}
-
-constexpr int kBW = 96;
-
+// Rows per run and warps across and down of a CTA. Large levels: the largest
+// run whose two CTAs per SM fit in registers (128 a thread) and shared memory
+// (103 to 110 KB a CTA). Small levels: narrow, short regions, so that a level
+// spreads over more SMs and each has fewer pixels to work through.
+template <int RAD, bool SMALL>
+struct StreamCfg { static constexpr int R = RAD == 3 ? 6 : 7, WX = 4, WY = 2; };
 template <int RAD>
-struct RadCfg;
-template <>
-struct RadCfg<1> { static constexpr int CH = 12; };
-template <>
-struct RadCfg<2> { static constexpr int CH = 12; };
-template <>
-struct RadCfg<3> { static constexpr int CH = 8; };
+struct StreamCfg<RAD, true> { static constexpr int R = RAD == 3 ? 6 : 4, WX = 2, WY = 2; };
 
-template <int RAD, int K, int BW, int CH, class Ts>
-cudaError_t launch_batch_one(LkBatch b, int n_ctas, cudaStream_t s) {
-    using Geo = StreamGeom<RAD, K, BW, CH>;
-    b.start[0] = 0;
-    for (int p = 0; p < b.n; ++p) {
-        b.nb[p] = (b.pair[p].w + BW - 1) / BW;
-        stream_segments<CH>(b.pair[p].h, b.nb[p] * 2, b.pair[p].seg_rows, &b.seg[p], &b.nseg[p]);
-        b.start[p + 1] = b.start[p] + 2 * b.nb[p] * b.nseg[p];
-    }
-    int grid = n_ctas > 0 ? n_ctas : 152;
-    if (grid > b.start[b.n]) grid = b.start[b.n];
-    cudaError_t e = cudaMemsetAsync(b.counter, 0, sizeof(unsigned), s);
-    if (e != cudaSuccess) return e;
-    lk_stream_batch_kernel<RAD, K, BW, CH, Ts><<<grid, kStreamThreads, Geo::bytes, s>>>(b);
-    return cudaGetLastError();
+template <int RAD, bool SMALL>
+struct CfgGeom : StreamGeom<RAD, StreamCfg<RAD, SMALL>::R, StreamCfg<RAD, SMALL>::WX, StreamCfg<RAD, SMALL>::WY> {
+    static constexpr int min_ctas = 512 / StreamGeom<RAD, StreamCfg<RAD, SMALL>::R, StreamCfg<RAD, SMALL>::WX,
+                                                     StreamCfg<RAD, SMALL>::WY>::threads;
+};
+
+// The region of band bx and segment sy, and the pixels it writes: neighbouring
+// regions overlap by twice the halo, and the first and last ones reach the
+// image's border, where no halo is needed.
+template <int RAD, bool SMALL, class Ts>
+__device__ __forceinline__ void lk_stream_cta(const LkArgs& a, int dir, int bx, int sy, int nb, int ns, int csize,
+                                              unsigned char* smem) {
+    using C = StreamCfg<RAD, SMALL>;
+    using Geo = CfgGeom<RAD, SMALL>;
+    const int halo = stream_halo(a.iters, RAD);
+    const int ox = bx * (Geo::RW - 2 * halo), oy = sy * (csize * Geo::RH - 2 * halo);
+    const int x_lo = bx ? ox + halo : 0, x_hi = bx + 1 < nb ? ox + Geo::RW - halo : a.w;
+    const int y_lo = sy ? oy + halo : 0, y_hi = sy + 1 < ns ? oy + csize * Geo::RH - halo : a.h;
+    lk_stream_item<RAD, C::R, C::WX, C::WY, Ts>(a, dir, ox, oy, csize, x_lo, x_hi, y_lo, y_hi, smem);
 }
 
-template <int RAD, class Ts>
-cudaError_t launch_rad_batch(const LkBatch& b, int n_ctas, cudaStream_t s) {
-    constexpr int CH = RadCfg<RAD>::CH;
-    switch (b.pair[0].iters) {
-        case 1: return launch_batch_one<RAD, 1, kBW, CH, Ts>(b, n_ctas, s);
-        case 2: return launch_batch_one<RAD, 2, kBW, CH, Ts>(b, n_ctas, s);
-        case 3: return launch_batch_one<RAD, 3, kBW, CH, Ts>(b, n_ctas, s);
-        case 4: return launch_batch_one<RAD, 4, kBW, CH, Ts>(b, n_ctas, s);
-        case 5: return launch_batch_one<RAD, 5, kBW, CH, Ts>(b, n_ctas, s);
-        default: return cudaErrorInvalidValue;
+template <int RAD, bool SMALL, class Ts>
+__global__ void __launch_bounds__(CfgGeom<RAD, SMALL>::threads, CfgGeom<RAD, SMALL>::min_ctas)
+    lk_stream_kernel(const __grid_constant__ LkArgs a, StreamPlan p) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int item = blockIdx.x / p.csize;
+    const int per_dir = p.nb * p.ns;
+    const int dir = item / per_dir, rem = item - dir * per_dir;
+    lk_stream_cta<RAD, SMALL, Ts>(a, dir, rem % p.nb, rem / p.nb, p.nb, p.ns, p.csize, smem);
+}
+
+// The same level of several strip pairs in one launch.
+template <int RAD, bool SMALL, class Ts>
+__global__ void __launch_bounds__(CfgGeom<RAD, SMALL>::threads, CfgGeom<RAD, SMALL>::min_ctas)
+    lk_stream_batch_kernel(const __grid_constant__ LkBatch b, int csize) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int item = blockIdx.x / csize;
+    int p = 0;
+    while (p + 1 < b.n && item >= b.start[p + 1]) ++p;
+    const int local = item - b.start[p];
+    const int per_dir = b.nb[p] * b.nseg[p];
+    const int dir = local / per_dir, rem = local - dir * per_dir;
+    lk_stream_cta<RAD, SMALL, Ts>(b.pair[p], dir, rem % b.nb[p], rem / b.nb[p], b.nb[p], b.nseg[p], csize, smem);
+}
+
+// Bands and segments of one level, from its size alone (a pair of a rig is cut
+// as it is by itself). The number of CTAs on top of each other is made as
+// small as possible (each row of a region is computed whether it is halo or
+// not), then the clusters; seg_rows > 0 asks for segments of about that many
+// rows instead.
+template <int RAD>
+StreamPlan stream_plan(int w, int h, int iters, int seg_rows) {
+    const int halo = stream_halo(iters, RAD);
+    StreamPlan p;
+    p.small = (long long)w * h * halo < kStreamSmallWork && halo <= kStreamSmallHalo;
+    const int RW = p.small ? CfgGeom<RAD, true>::RW : CfgGeom<RAD, false>::RW;
+    const int RH = p.small ? CfgGeom<RAD, true>::RH : CfgGeom<RAD, false>::RH;
+    auto parts = [halo](int n, int region) {
+        return n <= region ? 1 : (n - 2 * halo + region - 2 * halo - 1) / (region - 2 * halo);
+    };
+    p.nb = parts(w, RW);
+    const int c_min = 2 * halo / RH + 1;  // a region must be larger than its halo
+    if (seg_rows > 0) {
+        const long long c = ((long long)seg_rows + 2 * halo + RH - 1) / RH;
+        p.csize = c < c_min ? c_min : c > kMaxCluster ? kMaxCluster : (int)c;
+    } else {
+        p.csize = c_min;
+        long long best = -1;
+        for (int c = c_min; c <= kMaxCluster; ++c) {
+            const long long n = (long long)parts(h, c * RH) * c;
+            if (best < 0 || n < best) {
+                best = n;
+                p.csize = c;
+            }
+        }
     }
+    p.ns = parts(h, p.csize * RH);
+    return p;
+}
+
+template <class K, class... A>
+cudaError_t launch_clusters(K kernel, int items, int csize, int threads, size_t smem, cudaStream_t s, const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(items * csize));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)csize;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+    const cudaError_t l = cudaGetLastError();
+    return e != cudaSuccess ? e : l;
 }
 
 template <int RAD, class Ts>
 cudaError_t launch_rad_stream(const LkArgs& a, int ndirs, cudaStream_t s) {
-    constexpr int CH = RadCfg<RAD>::CH;
-    switch (a.iters) {
-        case 1: return launch_one<RAD, 1, kBW, CH, Ts>(a, ndirs, s);
-        case 2: return launch_one<RAD, 2, kBW, CH, Ts>(a, ndirs, s);
-        case 3: return launch_one<RAD, 3, kBW, CH, Ts>(a, ndirs, s);
-        case 4: return launch_one<RAD, 4, kBW, CH, Ts>(a, ndirs, s);
-        case 5: return launch_one<RAD, 5, kBW, CH, Ts>(a, ndirs, s);
-        default: return cudaErrorInvalidValue;
+    const StreamPlan p = stream_plan<RAD>(a.w, a.h, a.iters, a.seg_rows);
+    const int items = p.nb * p.ns * ndirs;
+    if (p.small) {
+        using Geo = CfgGeom<RAD, true>;
+        return launch_clusters(lk_stream_kernel<RAD, true, Ts>, items, p.csize, Geo::threads, Geo::bytes, s, a, p);
     }
+    using Geo = CfgGeom<RAD, false>;
+    return launch_clusters(lk_stream_kernel<RAD, false, Ts>, items, p.csize, Geo::threads, Geo::bytes, s, a, p);
+}
+
+// One launch for the pairs that are cut with the same CTA shape and cluster
+// size; adds the launches to *kernels.
+template <int RAD, class Ts>
+cudaError_t launch_rad_batch(const LkBatch& in, cudaStream_t s, int* kernels) {
+    StreamPlan plan[kMaxBatch];
+    for (int p = 0; p < in.n; ++p)
+        plan[p] = stream_plan<RAD>(in.pair[p].w, in.pair[p].h, in.pair[p].iters, in.pair[p].seg_rows);
+    bool done[kMaxBatch] = {};
+    for (int first = 0; first < in.n; ++first) {
+        if (done[first]) continue;
+        LkBatch b;
+        b.n = 0;
+        b.start[0] = 0;
+        for (int p = first; p < in.n; ++p) {
+            if (done[p] || plan[p].small != plan[first].small || plan[p].csize != plan[first].csize) continue;
+            done[p] = true;
+            b.pair[b.n] = in.pair[p];
+            b.nb[b.n] = plan[p].nb;
+            b.nseg[b.n] = plan[p].ns;
+            b.start[b.n + 1] = b.start[b.n] + 2 * plan[p].nb * plan[p].ns;
+            ++b.n;
+        }
+        const int items = b.start[b.n], csize = plan[first].csize;
+        cudaError_t e;
+        if (plan[first].small) {
+            using Geo = CfgGeom<RAD, true>;
+            e = launch_clusters(lk_stream_batch_kernel<RAD, true, Ts>, items, csize, Geo::threads, Geo::bytes, s, b, csize);
+        } else {
+            using Geo = CfgGeom<RAD, false>;
+            e = launch_clusters(lk_stream_batch_kernel<RAD, false, Ts>, items, csize, Geo::threads, Geo::bytes, s, b, csize);
+        }
+        if (e != cudaSuccess) return e;
+        ++*kernels;
+    }
+    return cudaSuccess;
+}
+
+template <int RAD, bool SMALL, class Ts>
+cudaError_t prepare_cfg(int max_smem) {
+    using Geo = CfgGeom<RAD, SMALL>;
+    if (Geo::bytes > (size_t)max_smem) return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute(lk_stream_kernel<RAD, SMALL, Ts>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)Geo::bytes);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(lk_stream_batch_kernel<RAD, SMALL, Ts>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)Geo::bytes);
 }
 
 template <int RAD, class Ts>
 cudaError_t prepare_rad_stream(int max_smem) {
-    constexpr int CH = RadCfg<RAD>::CH;
-    cudaError_t e;
-    if ((e = prepare_one<RAD, 1, kBW, CH, Ts>(max_smem)) != cudaSuccess) return e;
-    if ((e = prepare_one<RAD, 2, kBW, CH, Ts>(max_smem)) != cudaSuccess) return e;
-    if ((e = prepare_one<RAD, 3, kBW, CH, Ts>(max_smem)) != cudaSuccess) return e;
-    if ((e = prepare_one<RAD, 4, kBW, CH, Ts>(max_smem)) != cudaSuccess) return e;
-    return prepare_one<RAD, 5, kBW, CH, Ts>(max_smem);
+    const cudaError_t e = prepare_cfg<RAD, true, Ts>(max_smem);
+    return e != cudaSuccess ? e : prepare_cfg<RAD, false, Ts>(max_smem);
 }
 
 // Entry points for one storage type (instantiated by exactly one .cu file).
@@ -703,11 +810,11 @@ cudaError_t stream_launch(const LkArgs& a, int ndirs, cudaStream_t s) {
 }
 
 template <class Ts>
-cudaError_t stream_launch_batch(const LkBatch& b, int n_ctas, cudaStream_t s) {
+cudaError_t stream_launch_batch(const LkBatch& b, cudaStream_t s, int* kernels) {
     switch (b.pair[0].radius) {
-        case 1: return launch_rad_batch<1, Ts>(b, n_ctas, s);
-        case 2: return launch_rad_batch<2, Ts>(b, n_ctas, s);
-        case 3: return launch_rad_batch<3, Ts>(b, n_ctas, s);
+        case 1: return launch_rad_batch<1, Ts>(b, s, kernels);
+        case 2: return launch_rad_batch<2, Ts>(b, s, kernels);
+        case 3: return launch_rad_batch<3, Ts>(b, s, kernels);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -720,14 +827,14 @@ cudaError_t stream_prepare(int max_smem_bytes) {
     return prepare_rad_stream<3, Ts>(max_smem_bytes);
 }
 
-#define PANO_LKS_INSTANTIATE(Ts)                                                          \
-    template cudaError_t stream_launch<Ts>(const LkArgs&, int, cudaStream_t);            \
-    template cudaError_t stream_launch_batch<Ts>(const LkBatch&, int, cudaStream_t);     \
+#define PANO_LKS_INSTANTIATE(Ts)                                                      \
+    template cudaError_t stream_launch<Ts>(const LkArgs&, int, cudaStream_t);        \
+    template cudaError_t stream_launch_batch<Ts>(const LkBatch&, cudaStream_t, int*);    \
     template cudaError_t stream_prepare<Ts>(int);
 
-#define PANO_LKS_EXTERN(Ts)                                                                  \
-    extern template cudaError_t stream_launch<Ts>(const LkArgs&, int, cudaStream_t);        \
-    extern template cudaError_t stream_launch_batch<Ts>(const LkBatch&, int, cudaStream_t); \
+#define PANO_LKS_EXTERN(Ts)                                                              \
+    extern template cudaError_t stream_launch<Ts>(const LkArgs&, int, cudaStream_t);    \
+    extern template cudaError_t stream_launch_batch<Ts>(const LkBatch&, cudaStream_t, int*);\
     extern template cudaError_t stream_prepare<Ts>(int);
 
 }  // namespace lks

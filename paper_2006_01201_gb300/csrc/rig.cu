@@ -58,7 +58,6 @@ struct pano_rig {
     int device;
     int nlev;
     int max_smem;
-    int n_ctas;                    // persistent grid of the streamed kernel
     int def_tile_w, def_tile_h;    // default tile of the tiled kernel
     int hs[kMaxLevels];            // level heights (shared by all pairs)
     int ws[kMaxBatch][kMaxLevels]; // level widths per pair
@@ -66,7 +65,6 @@ struct pano_rig {
     int flow_pitch[kMaxBatch][kMaxLevels];  // float2 elements
     void* pyr[kMaxBatch][2][kMaxLevels];    // luma pyramids of L and R (pyr_dtype elements)
     float* flw[kMaxBatch][2][kMaxLevels];   // flows per direction; level 0 = the rig's own output flows
-    unsigned* counters;                     // work counters of the persistent launches, one per level
     void* buf;
     size_t buf_bytes;
     pano_rig_tuning tune[kMaxLevels];
@@ -210,16 +208,15 @@ LkArgs pair_level_args(const pano_rig* r, const RunCall& c, int k, int l, const 
     return a;
 }
 
-bool uses_stream(const pano_rig* r, const LkArgs& a, int kernel) {
-    if (!lk_stream_supports(r->p.iters, r->p.radius)) return false;
-    if (kernel == PANO_LK_STREAM) return true;
+bool uses_stream(const pano_rig* r, int kernel) {
+    if (kernel == PANO_LK_STREAM) return true;  // check_tuning has looked at the steps
     if (kernel == PANO_LK_TILE) return false;
-    return (long long)a.w * a.h >= kStreamMinPixels;  // the rule of launch_lk_level
+    return lk_auto_streams(r->p.iters, r->p.radius);  // the rule of launch_lk_level
 }
 
-// LK level l of every pair with tuning t: one persistent launch of the
-// streamed kernel for the pairs that use it, then one tiled launch per tile
-// shape (in the order of the first pair with that shape). Returns the first
+// LK level l of every pair with tuning t: the pairs that use the streamed
+// kernel (one launch per CTA shape and cluster size of its plans, traced as
+// one), then one tiled launch per tile shape (in the order of the first pair with that shape). Returns the first
 // launch error and adds the kernels launched to *kernels.
 cudaError_t enqueue_lk_level(pano_rig* r, const RunCall& c, int l, const pano_rig_tuning& t, cudaStream_t s,
                              bool trace, int* kernels) {
@@ -229,7 +226,7 @@ cudaError_t enqueue_lk_level(pano_rig* r, const RunCall& c, int l, const pano_ri
     int ntb = 0;
     for (int k = 0; k < r->d.n_pairs; ++k) {
         LkArgs a = pair_level_args(r, c, k, l, t);
-        if (uses_stream(r, a, t.kernel)) {
+        if (uses_stream(r, t.kernel)) {
             sb.pair[sb.n++] = a;
             continue;
         }
@@ -243,11 +240,9 @@ cudaError_t enqueue_lk_level(pano_rig* r, const RunCall& c, int l, const pano_ri
     }
     cudaError_t e;
     if (sb.n) {
-        sb.counter = r->counters + l;
         int slot = trace ? trace_begin(r->tr, PANO_TRACE_LK, l, s) : -1;
-        if ((e = launch_lk_stream_batch(sb, r->n_ctas, s)) != cudaSuccess) return e;
+        if ((e = launch_lk_stream_batch(sb, s, kernels)) != cudaSuccess) return e;
         if (slot >= 0) trace_end(r->tr, slot, s);
-        ++*kernels;
     }
     for (int g = 0; g < ntb; ++g) {
         int slot = trace ? trace_begin(r->tr, PANO_TRACE_LK, l, s) : -1;
@@ -262,8 +257,6 @@ cudaError_t enqueue_lk_level(pano_rig* r, const RunCall& c, int l, const pano_ri
 cudaError_t enqueue_all(pano_rig* r, const RunCall& c, cudaStream_t s, bool trace, int* kernels) {
     const int n = r->d.n_pairs;
     cudaError_t e;
-    // work counters of the persistent launches start at zero
-    if ((e = cudaMemsetAsync(r->counters, 0, sizeof(unsigned) * kMaxLevels, s)) != cudaSuccess) return e;
     // luma of every strip that is not its own level 0
     LumaArgs la;
     memset(&la, 0, sizeof(la));
@@ -475,16 +468,13 @@ pano_status pano_rig_create(const pano_flow_params* p, const pano_rig_desc* d, p
     r->def_tile_w = tw;
     r->def_tile_h = th;
     cudaError_t e = cudaGetDevice(&r->device);
-    int sms = 0;
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, r->device);
     if (e != cudaSuccess) {
         free_rig(r);
         return cuda_fail(e, "device query");
     }
-    r->n_ctas = sms;  // the streamed kernel runs one 768-thread CTA per SM
     const int n = d->n_pairs;
     for (int l = 0; l < r->nlev; ++l) r->hs[l] = l == 0 ? d->h : (r->hs[l - 1] + 1) / 2;
-    size_t total = align_up(sizeof(unsigned) * kMaxLevels, 256);
+    size_t total = 0;
     std::vector<size_t> offs;
     for (int k = 0; k < n; ++k)
         for (int l = 0; l < r->nlev; ++l) {
@@ -509,7 +499,6 @@ pano_status pano_rig_create(const pano_flow_params* p, const pano_rig_desc* d, p
     }
     r->buf_bytes = total;
     char* b = static_cast<char*>(r->buf);
-    r->counters = reinterpret_cast<unsigned*>(b);
     size_t i = 0;
     for (int k = 0; k < n; ++k)
         for (int l = 0; l < r->nlev; ++l) {
@@ -618,15 +607,12 @@ pano_status pano_rig_autotune(pano_rig* r, const pano_image* L, const pano_image
         pano_rig_tuning pick = cand[0];
         for (const pano_rig_tuning& ct : cand) {
             int dummy = 0;
-            // the counter of this level is reset before every launch
-            if ((e = cudaMemsetAsync(r->counters + l, 0, sizeof(unsigned), s)) != cudaSuccess ||
-                (e = enqueue_lk_level(r, c, l, ct, s, false, &dummy)) != cudaSuccess) {
+            if ((e = enqueue_lk_level(r, c, l, ct, s, false, &dummy)) != cudaSuccess) {
                 out = cuda_fail(e, "autotune launch");
                 break;
             }
             for (int i = 0; i < reps && out == PANO_OK; ++i) {
-                if ((e = cudaMemsetAsync(r->counters + l, 0, sizeof(unsigned), s)) != cudaSuccess ||
-                    (e = cudaEventRecord(ev[0], s)) != cudaSuccess ||
+                if ((e = cudaEventRecord(ev[0], s)) != cudaSuccess ||
                     (e = enqueue_lk_level(r, c, l, ct, s, false, &dummy)) != cudaSuccess ||
                     (e = cudaEventRecord(ev[1], s)) != cudaSuccess || (e = cudaEventSynchronize(ev[1])) != cudaSuccess ||
                     (e = cudaEventElapsedTime(&times[i], ev[0], ev[1])) != cudaSuccess)

@@ -173,6 +173,56 @@ def test_each_lk_kernel_matches_oracle(kernel, h, w, iters, radius, start):
     assert np.abs(got - ref).max() <= 1e-3
 
 
+# the streamed kernel cuts a level into regions of 64 columns and 16 rows (24 at
+# radius 3) per CTA, or of 128 columns and 28 rows (24 at radius 3) for large
+# levels, up to 8 CTAs on top of each other, that overlap by twice the halo:
+# sizes on either side of one region, of one CTA and of one segment, and of the
+# line between the two
+@pytest.mark.parametrize("h,w,iters,radius,start", [
+    (16, 64, 5, 2, "coarse"), (17, 65, 5, 2, "coarse"), (33, 108, 5, 2, "zero"), (128, 109, 5, 2, "coarse"),
+    (129, 63, 5, 2, "coarse"), (27, 1, 1, 1, "zero"), (1, 255, 3, 1, "coarse"), (223, 117, 1, 1, "given"),
+    (192, 97, 5, 3, "coarse"), (193, 61, 4, 3, "zero"), (25, 129, 5, 3, "given"),
+    (400, 399, 5, 2, "coarse"), (400, 400, 5, 2, "coarse"), (408, 452, 5, 2, "zero"), (429, 453, 5, 2, "given"),
+    (224, 893, 4, 2, "coarse"), (225, 894, 4, 2, "coarse"), (350, 291, 5, 3, "coarse"), (1601, 100, 3, 3, "given"),
+    (517, 521, 5, 1, "coarse")])
+def test_streamed_kernel_at_the_edges_of_its_regions(h, w, iters, radius, start):
+    # a reference of 64 bits; the bounds are those of the test above
+    T = texture(h, w, 14).astype(np.float32)
+    J = (0.8 * np.roll(T, (1, -1), axis=(0, 1)) + 0.2 * texture(h, w, 15)).astype(np.float32)
+    g = rng(16)
+    uin, ref = None, np.zeros((h, w, 2))
+    if start == "coarse":
+        uin = g.normal(0, 1.0, size=((h + 1) // 2, (w + 1) // 2, 2)).astype(np.float32)
+        ref = oracle.upsample_flow(uin, h, w)
+    elif start == "given":
+        uin = g.normal(0, 1.5, size=(h, w, 2)).astype(np.float32)
+        ref = uin.astype(np.float64)
+    for _ in range(iters):
+        ref = oracle.lk_step(T, J, ref, radius, 1e-2)
+    got = host(binding.stage_lk(cuda(T), cuda(J), None if uin is None else cuda(uin), upsample=start == "coarse",
+                                iters=iters, radius=radius, lam=1e-2, kernel=binding.PANO_LK_STREAM))
+    assert np.isfinite(got).all()
+    assert epe(got, ref).mean() <= 1e-5
+    assert np.abs(got - ref).max() <= 1e-3
+
+
+@pytest.mark.parametrize("y,x", [(0, 0), (59, 139), (30, 127), (28, 128), (13, 64)])
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+@pytest.mark.parametrize("where", ["T", "J"])
+def test_streamed_kernel_spreads_non_numbers_like_the_tiled_one(y, x, value, where):
+    T = texture(60, 140, 17).astype(np.float32)
+    J = np.roll(T, 1, axis=1).astype(np.float32)
+    (T if where == "T" else J)[y, x] = value
+    u = np.zeros((60, 140, 2), np.float32)
+    u[..., 0] = 0.25
+    u[20:25, 20:25] = 40.0   # samples outside the staged box
+    a, b = (host(binding.stage_lk(cuda(T), cuda(J), cuda(u), iters=1, radius=2, lam=1e-2, kernel=k))
+            for k in (binding.PANO_LK_STREAM, binding.PANO_LK_TILE))
+    assert np.array_equal(np.isfinite(a), np.isfinite(b))
+    ok = np.isfinite(a)
+    assert ok.any() and not ok.all() and np.abs(a[ok] - b[ok]).max() <= 1e-4
+
+
 @pytest.mark.parametrize("kernel", [binding.PANO_LK_AUTO, binding.PANO_LK_TILE])
 @pytest.mark.parametrize("h,w,iters,radius,start", [(70, 90, 8, 2, "zero"), (40, 60, 16, 1, "given")])
 def test_lk_kernels_beyond_five_steps_match_oracle(kernel, h, w, iters, radius, start):
@@ -186,6 +236,22 @@ def test_lk_kernels_beyond_five_steps_match_oracle(kernel, h, w, iters, radius, 
         ref = oracle.lk_step(T, J, ref, radius, 1e-2)
     got = host(binding.stage_lk(cuda(T), cuda(J), None if uin is None else cuda(uin), iters=iters, radius=radius,
                                 lam=1e-2, kernel=kernel))
+    assert np.isfinite(got).all()
+    assert epe(got, ref).mean() <= 1e-5
+    assert np.abs(got - ref).max() <= 1e-3
+
+
+@pytest.mark.parametrize("h,w,iters,radius", [(300, 260, 8, 2), (150, 300, 8, 3), (90, 200, 9, 3), (260, 300, 12, 2),
+                                              (200, 230, 16, 1), (60, 70, 13, 2)])
+def test_auto_beyond_five_steps_on_either_side_of_its_lines(h, w, iters, radius):
+    # iters * radius up to 24 runs the streamed kernel (small regions up to 16), more the tiled one
+    T = texture(h, w, 24).astype(np.float32)
+    J = np.roll(T, (1, 1), axis=(0, 1)).astype(np.float32)
+    ref = np.zeros((h, w, 2))
+    for _ in range(iters):
+        ref = oracle.lk_step(T, J, ref, radius, 1e-2)
+    got = host(binding.stage_lk(cuda(T), cuda(J), None, iters=iters, radius=radius, lam=1e-2,
+                                kernel=binding.PANO_LK_AUTO))
     assert np.isfinite(got).all()
     assert epe(got, ref).mean() <= 1e-5
     assert np.abs(got - ref).max() <= 1e-3
