@@ -12,8 +12,12 @@
 // Distances are computed exactly, as integers, in two separable passes:
 //   columns: g(x, y) = |y - y'| to the nearest feature pixel (x, y') of the
 //            same column, or "none";
-//   rows:    d2(x, y) = min over columns x' of (x - x')^2 + g(x', y)^2, the
-//            lower envelope of one parabola per column that has a feature
+//   rows:    d2(x, y) = min over columns x' of (x - x')^2 + g(x', y)^2. The
+//            leftmost column that attains the minimum never moves left as x
+//            grows, so the columns of a few pixels bound those of the pixels
+//            between them (edt_near_kernel). Canvases with a side above
+//            kNearMaxSide, whose squared distances leave 32 bits, take the
+//            lower envelope of one parabola per column instead
 //            (edt_row.cuh: banded envelopes merged in a tree).
 // Only the final ratio is rounded (FP32 square roots and one division).
 #include <stdio.h>
@@ -32,23 +36,38 @@ namespace pano {
 namespace {
 
 // ---------------------------------------------------------------------------
-// Column pass. A CTA of 32 x 32 threads owns 32 columns and walks down them
-// in blocks of 1024 rows; thread (tx, ty) holds rows ty*32 .. ty*32+31 of a
+// Column pass. A CTA of 32 x 16 threads owns 32 columns and walks down them
+// in blocks of 512 rows; thread (tx, ty) holds rows ty*32 .. ty*32+31 of a
 // block of column tx as two 32-bit masks (Area1, Area2 pixels). A first pass
 // over the labels finds, per column and block, the first feature row; a
 // suffix minimum gives the first feature row at or after each block. The
-// second pass finds each row's nearest feature above and below from the
-// bits of its own mask, the masks of the other threads of its block (shared
-// memory), the last feature row of the blocks above and the first of the
-// blocks below. g of each area goes to a plane of 16-bit values (coalesced
-// 2-byte stores; edt::kNoSite where the column has no feature pixel).
+// second pass finds the nearest features above and below the thread's rows
+// from the masks of the other threads of its block (shared memory), the last
+// feature row of the blocks above and the first of the blocks below, and walks
+// its rows down and up with the last feature row seen. The masks of the first
+// kKeptBlocks blocks stay in shared memory between the two passes, so canvases
+// of up to 4096 rows are read once.
+// kPacked: g of both areas in one 32-bit element (Area1 low, Area2 high), one
+// coalesced 4-byte store a pixel; otherwise a plane of 16-bit values each.
+// 99 us on a 4000 x 9000 canvas (0.18 GB: 27 us at the memory's rate), bound by
+// instructions (67 M); labels read twice, distances from shifted masks and two
+// 16-bit stores a pixel took 131 us (102 M).
+// edt::kNoSite where the column has no feature pixel. gp: elements per row.
 // ---------------------------------------------------------------------------
 constexpr int kColW = 32;                     // columns per CTA
-constexpr int kColTY = 32;                    // threads along y, 32 rows each
+constexpr int kColTY = 16;                    // threads along y, 32 rows each
 constexpr int kColBlock = 32 * kColTY;        // rows per block
 constexpr int kMaxBlocks = (65535 + kColBlock - 1) / kColBlock;
+constexpr int kKeptBlocks = 8;
 constexpr int kAboveNone = -(1 << 20);        // y - kAboveNone > any distance
 constexpr int kBelowNone = INT_MAX;
+
+struct ColSmem {
+    uint32_t mask[kKeptBlocks][2][kColTY][kColW];
+    int next[2][kMaxBlocks + 1][kColW];       // first feature row at or after block rb's first row
+    int above[2][kColW];                      // last feature row above the current block
+    uint32_t some[kKeptBlocks][2][kColW];     // bit k: thread row k of the block has a feature pixel
+};
 
 __device__ __forceinline__ void col_masks(const unsigned char* __restrict__ label, long long pitch, long long nl,
                                           int h, int x, int y0, uint32_t* m1, uint32_t* m2) {
@@ -67,96 +86,384 @@ __device__ __forceinline__ void col_masks(const unsigned char* __restrict__ labe
     *m2 = b;
 }
 
+template <bool kPacked>
 __global__ void __launch_bounds__(kColW * kColTY, 2) edt_cols_kernel(const unsigned char* __restrict__ label, int h,
-                                                                    int w, long long pitch, uint16_t* __restrict__ g1,
-                                                                    uint16_t* __restrict__ g2) {
-    __shared__ int s_next[2][kMaxBlocks + 1][kColW];  // first feature row at or after block rb's first row
-    __shared__ uint32_t s_mask[2][kColTY][kColW];
-    __shared__ int s_above[2][kColW];                 // last feature row above the current block
+                                                                    int w, long long pitch, uint32_t* __restrict__ gb,
+                                                                    uint16_t* __restrict__ g1,
+                                                                    uint16_t* __restrict__ g2, int gp) {
+    extern __shared__ __align__(16) unsigned char s_col[];
+    ColSmem& S = *reinterpret_cast<ColSmem*>(s_col);
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kColW + tx;
     const int x = blockIdx.x * kColW + tx;
     const bool col_in = x < w;
     const int nblk = (h + kColBlock - 1) / kColBlock;
-    const long long nl = (long long)(h - 1) * pitch + w, ng = (long long)h * w;  // label and g elements
+    const long long nl = (long long)(h - 1) * pitch + w, ng = (long long)h * gp;  // label and g elements
     (void)nl;
     (void)ng;
-    constexpr int NN = 2 * (kMaxBlocks + 1) * kColW;
-    for (int i = tid; i < NN; i += kColW * kColTY) PANO_AT(&s_next[0][0][0], i, NN, 502) = kBelowNone;
-    if (tid < 2 * kColW) PANO_AT(&s_above[0][0], tid, 2 * kColW, 503) = kAboveNone;
+    const int nn = 2 * (kMaxBlocks + 1) * kColW;
+    for (int i = tid; i < nn; i += kColW * kColTY) PANO_AT(&S.next[0][0][0], i, nn, 502) = kBelowNone;
+    if (tid < 2 * kColW) PANO_AT(&S.above[0][0], tid, 2 * kColW, 503) = kAboveNone;
+    for (int i = tid; i < kKeptBlocks * 2 * kColW; i += kColW * kColTY) (&S.some[0][0][0])[i] = 0;
     __syncthreads();
     for (int rb = 0; rb < nblk; ++rb) {
         const int y0 = rb * kColBlock + ty * 32;
         uint32_t m1 = 0, m2 = 0;
         if (col_in && y0 < h) col_masks(label, pitch, nl, h, x, y0, &m1, &m2);
-        if (m1) atomicMin(&s_next[0][rb][tx], y0 + __ffs(m1) - 1);
-        if (m2) atomicMin(&s_next[1][rb][tx], y0 + __ffs(m2) - 1);
+        if (m1) atomicMin(&S.next[0][rb][tx], y0 + __ffs(m1) - 1);
+        if (m2) atomicMin(&S.next[1][rb][tx], y0 + __ffs(m2) - 1);
+        if (rb < kKeptBlocks) {
+            S.mask[rb][0][ty][tx] = m1, S.mask[rb][1][ty][tx] = m2;
+            if (m1) atomicOr(&S.some[rb][0][tx], 1u << ty);
+            if (m2) atomicOr(&S.some[rb][1][tx], 1u << ty);
+        }
     }
     __syncthreads();
     if (ty < 2)
-        for (int rb = nblk - 1; rb >= 0; --rb) s_next[ty][rb][tx] = min(s_next[ty][rb][tx], s_next[ty][rb + 1][tx]);
+        for (int rb = nblk - 1; rb >= 0; --rb) S.next[ty][rb][tx] = min(S.next[ty][rb][tx], S.next[ty][rb + 1][tx]);
     __syncthreads();
     for (int rb = 0; rb < nblk; ++rb) {
         const int yb = rb * kColBlock, y0 = yb + ty * 32;
+        const int slot = rb < kKeptBlocks ? rb : 0;
         uint32_t m[2] = {0, 0};
-        if (col_in && y0 < h) col_masks(label, pitch, nl, h, x, y0, &m[0], &m[1]);
-        s_mask[0][ty][tx] = m[0];
-        s_mask[1][ty][tx] = m[1];
-        __syncthreads();
+        if (rb < kKeptBlocks) {
+            m[0] = S.mask[slot][0][ty][tx];
+            m[1] = S.mask[slot][1][ty][tx];
+        } else {
+            if (col_in && y0 < h) col_masks(label, pitch, nl, h, x, y0, &m[0], &m[1]);
+            if (tid < 2 * kColW) (&S.some[slot][0][0])[tid] = 0;
+            S.mask[slot][0][ty][tx] = m[0];
+            S.mask[slot][1][ty][tx] = m[1];
+            __syncthreads();
+            if (m[0]) atomicOr(&S.some[slot][0][tx], 1u << ty);
+            if (m[1]) atomicOr(&S.some[slot][1][tx], 1u << ty);
+            __syncthreads();
+        }
         int above[2], below[2];  // nearest feature rows above and below this thread's 32 rows
 #pragma unroll
         for (int a = 0; a < 2; ++a) {
-            int p = s_above[a][tx];
-            for (int k = ty - 1; k >= 0; --k) {
-                const uint32_t v = s_mask[a][k][tx];
-                if (v) {
-                    p = yb + k * 32 + 31 - __clz(v);
-                    break;
-                }
+            const uint32_t some = S.some[slot][a][tx], lo = some & ((1u << ty) - 1u), hi = some & ~((2u << ty) - 1u);
+            int p = S.above[a][tx], n = S.next[a][rb + 1][tx];
+            if (lo) {
+                const int k = 31 - __clz(lo);
+                p = yb + k * 32 + 31 - __clz(S.mask[slot][a][k][tx]);
             }
-            int n = s_next[a][rb + 1][tx];
-            for (int k = ty + 1; k < kColTY; ++k) {
-                const uint32_t v = s_mask[a][k][tx];
-                if (v) {
-                    n = yb + k * 32 + __ffs(v) - 1;
-                    break;
-                }
+            if (hi) {
+                const int k = __ffs(hi) - 1;
+                n = yb + k * 32 + __ffs(S.mask[slot][a][k][tx]) - 1;
             }
             above[a] = p;
             below[a] = n;
         }
         if (col_in && y0 < h) {
             const int n = min(32, h - y0);
-#pragma unroll 8
-            for (int i = 0; i < 32; ++i) {
-                if (i >= n) break;
-                const int yy = y0 + i;
-                uint32_t g[2];
+            const unsigned kNone = edt::kNoSite;
+#pragma unroll 1
+            for (int i0 = 0; i0 < 32; i0 += 16) {
+                // 16 rows at a time (their distances upwards stay in registers)
+                const uint32_t before[2] = {m[0] & ((1u << i0) - 1u), m[1] & ((1u << i0) - 1u)};
+                const uint32_t after[2] = {i0 ? 0u : m[0] & 0xFFFF0000u, i0 ? 0u : m[1] & 0xFFFF0000u};
+                uint32_t d[16];  // both areas in 16 bits each
+                int p1 = before[0] ? y0 + 31 - __clz(before[0]) : above[0], p2 = before[1] ? y0 + 31 - __clz(before[1]) : above[1];
+                const uint32_t k1 = m[0] >> i0, k2 = m[1] >> i0;
 #pragma unroll
-                for (int a = 0; a < 2; ++a) {
-                    const uint32_t up = m[a] << (31 - i);  // rows y0 .. yy, row yy in bit 31
-                    const uint32_t dn = m[a] >> i;         // rows yy .. y0 + 31, row yy in bit 0
-                    // distances above and below (ints: rows < 2^16, the no-feature
-                    // values keep both differences below 2^31)
-                    const int da = up ? __clz(up) : yy - above[a];
-                    const int db = dn ? __ffs(dn) - 1 : below[a] - yy;
-                    const int d = min(da, db);
-                    g[a] = d >= (int)edt::kNoSite ? edt::kNoSite : (uint32_t)d;
+                for (int i = 0; i < 16; ++i) {
+                    const int yy = y0 + i0 + i;
+                    if (k1 >> i & 1) p1 = yy;
+                    if (k2 >> i & 1) p2 = yy;
+                    d[i] = min((unsigned)(yy - p1), kNone) | min((unsigned)(yy - p2), kNone) << 16;
                 }
-                PANO_AT(g1, (long long)yy * w + x, ng, 504) = (uint16_t)g[0];
-                PANO_AT(g2, (long long)yy * w + x, ng, 504) = (uint16_t)g[1];
+                p1 = after[0] ? y0 + __ffs(after[0]) - 1 : below[0];
+                p2 = after[1] ? y0 + __ffs(after[1]) - 1 : below[1];
+#pragma unroll
+                for (int i = 15; i >= 0; --i) {
+                    const int yy = y0 + i0 + i;
+                    if (k1 >> i & 1) p1 = yy;
+                    if (k2 >> i & 1) p2 = yy;
+                    // ints: rows < 2^16, the no-feature values keep both differences below 2^31
+                    const uint32_t v = __vminu2(d[i], min((unsigned)(p1 - yy), kNone) | min((unsigned)(p2 - yy), kNone) << 16);
+                    if (i0 + i < n) {
+                        const long long o = (long long)yy * gp + x;
+                        if constexpr (kPacked) {
+                            PANO_AT(gb, o, ng, 504) = v;
+                        } else {
+                            PANO_AT(g1, o, ng, 504) = (uint16_t)(v & 0xFFFFu);
+                            PANO_AT(g2, o, ng, 504) = (uint16_t)(v >> 16);
+                        }
+                    }
+                }
             }
         }
-        __syncthreads();  // the masks and s_above are read
+        __syncthreads();  // the masks and S.above are read
         if (ty == kColTY - 1) {
-            s_above[0][tx] = m[0] ? y0 + 31 - __clz(m[0]) : above[0];
-            s_above[1][tx] = m[1] ? y0 + 31 - __clz(m[1]) : above[1];
+            S.above[0][tx] = m[0] ? y0 + 31 - __clz(m[0]) : above[0];
+            S.above[1][tx] = m[1] ? y0 + 31 - __clz(m[1]) : above[1];
         }
         __syncthreads();
     }
 }
 
 // ---------------------------------------------------------------------------
-// Row pass: one CTA of kRowThreads per row and area, one band of
+// Row pass, sides up to kNearMaxSide: one CTA per row, both areas. The row's
+// columns are cut into groups of 64; only groups with an Area3 pixel matter.
+//   1  g of both areas to shared memory, with the least g of every block of 32
+//      columns; pixels of the other groups are written at once;
+//   2  the nearest column (leftmost of equals) for the first pixel of every
+//      group and the last pixel of the last one, by bisection over the groups:
+//      a warp searches between the columns of the two neighbours already
+//      known. A long range is searched by blocks: the least g bounds every
+//      distance to a block from both sides, and only the blocks whose lower
+//      bound does not exceed the least upper bound are looked through;
+//   3  a lane per two pixels: the least distance over the columns between those of
+//      its group and of the next one, and Eq. (1). Where that range is long
+//      (the nearest column jumps from one seam to another), the bisection goes
+//      on over the group's lanes.
+// Distances are 32-bit integers (kNearMaxSide: the bound of step 2 adds 31
+// columns to the largest distance and still stays below 2^32).
+// What bounds it: the instructions of steps 2 and 3 (195 M warp instructions on
+// a 4000 x 9000 canvas, 64% of the issue rate); the g plane is read once.
+// 254 us there, against 457 + 505 us of the envelopes' two launches. Groups of
+// 32: 284 us; steps 2 and 3 alone without the bisection in step 3: a row whose
+// overlaps lie far apart looks through the columns between them, 935 us.
+// ---------------------------------------------------------------------------
+constexpr int kNearThreads = 256;
+constexpr int kNearWarps = kNearThreads / 32;
+constexpr int kNearMaxSide = 46000;
+constexpr int kNearScan = 64;  // columns that a lane looks through one by one
+constexpr int kNearFew = 4;    // a shorter range is left for step 3
+
+struct NearSmem {
+    int w4, nb, ng;  // columns rounded up to 4, blocks of 32 columns, groups of 64
+    __host__ __device__ explicit NearSmem(int w) : w4((w + 3) / 4 * 4), nb((w + 31) / 32), ng((w + 63) / 64) {}
+    __host__ __device__ size_t bytes() const { return 4 * ((size_t)w4 + nb) + 2 * (4 * ((size_t)ng + 1) + ng); }
+};
+
+__device__ __forceinline__ unsigned near_cost(unsigned g, int dx) {
+    return g == edt::kNoSite ? 0xFFFFFFFFu : (unsigned)(dx * dx) + g * g;
+}
+
+// Leftmost nearest column of pixel x among [lo, hi], by one warp; some column
+// of [lo, hi] is a nearest one of the whole row. gs and bm hold both areas'
+// values, sh (0 or 16) selects the area.
+__device__ __forceinline__ int near_search(const uint32_t* __restrict__ gs, const uint32_t* __restrict__ bm, int sh, int w,
+                                           int nb, int x, int lo, int hi) {
+    (void)w, (void)nb;
+    const int lane = threadIdx.x & 31;
+    constexpr unsigned kAll = 0xffffffffu;
+    unsigned best = 0xFFFFFFFFu;
+    int bq = hi;
+    if (hi - lo < 128) {
+        for (int q = lo + lane; q <= hi; q += 32) {
+            const unsigned c = near_cost(PANO_AT(gs, q, w, 516) >> sh & 0xFFFFu, x - q);
+            if (c < best) best = c, bq = q;
+        }
+        const unsigned m = __reduce_min_sync(kAll, best);
+        return (int)__reduce_min_sync(kAll, best == m ? (unsigned)bq : 0xFFFFFFFFu);
+    }
+    const int b0 = lo >> 5, b1 = hi >> 5;
+    unsigned ub = 0xFFFFFFFFu;
+    for (int b = b0 + lane; b <= b1; b += 32)
+        ub = min(ub, near_cost(PANO_AT(bm, b, nb, 517) >> sh & 0xFFFFu, max(abs(x - 32 * b), abs(x - 32 * b - 31))));
+    ub = __reduce_min_sync(kAll, ub);
+    for (int base = b0; base <= b1; base += 32) {
+        const int b = base + lane;
+        unsigned lb = 0xFFFFFFFFu;
+        if (b <= b1) lb = near_cost(PANO_AT(bm, b, nb, 518) >> sh & 0xFFFFu, max(0, max(32 * b - x, x - 32 * b - 31)));
+        unsigned todo = __ballot_sync(kAll, lb <= ub && lb != 0xFFFFFFFFu);
+        while (todo) {
+            const int k = __ffs(todo) - 1;
+            const int q = 32 * (base + k) + lane;
+            unsigned c = 0xFFFFFFFFu;
+            if (q >= lo && q <= hi) c = near_cost(PANO_AT(gs, q, w, 519) >> sh & 0xFFFFu, x - q);
+            const unsigned m = __reduce_min_sync(kAll, c);
+            if (m < best) {
+                best = m;
+                bq = (int)__reduce_min_sync(kAll, c == m ? (unsigned)q : 0xFFFFFFFFu);
+                ub = min(ub, m);
+            }
+            todo &= __ballot_sync(kAll, lb <= ub && lb != 0xFFFFFFFFu) & ~((2u << k) - 1u);
+        }
+    }
+    return bq;
+}
+
+__global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const unsigned char* __restrict__ label, int h, int w,
+                                                               long long pitch, const uint32_t* __restrict__ gb, int gp,
+                                                               float* __restrict__ blend, int blend_pitch) {
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    __shared__ int s_n;
+    __shared__ unsigned s_any[2];
+    const NearSmem L(w);
+    const int w4 = L.w4, nb = L.nb, ng = L.ng;
+    uint32_t* gs = reinterpret_cast<uint32_t*>(s_dyn);      // [w4] g of both areas
+    uint32_t* bm = gs + w4;                                  // [nb] least g of a block, both areas
+    uint16_t* ql = reinterpret_cast<uint16_t*>(bm + nb);     // [2][ng + 1] the nearest column of point i lies
+    uint16_t* qh = ql + 2 * (ng + 1);                        // [2][ng + 1] between these two
+    uint16_t* list = qh + 2 * (ng + 1);                      // [ng] groups with an Area3 pixel
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, y = blockIdx.x;
+    constexpr unsigned kAll = 0xffffffffu;
+    const unsigned char* lab = label + (long long)y * pitch;
+    float* out = blend + (long long)y * blend_pitch;
+
+    // ---- 1: g, and the least g of each block (eight threads of four columns)
+    if (tid < 2) s_any[tid] = 0;
+    __syncthreads();
+    {
+        const uint32_t* row = gb + (long long)y * gp;
+        const bool vec = (((uintptr_t)row) & 15) == 0;
+        unsigned all = kAll;
+        for (int v0 = 0; v0 < w4 / 4; v0 += kNearThreads) {
+            const int v = v0 + tid;
+            uint4 k = make_uint4(kAll, kAll, kAll, kAll);
+            if (v < w4 / 4) {
+                if (vec && 4 * v + 4 <= w) {
+                    k = __ldg(reinterpret_cast<const uint4*>(&PANO_VEC(const uint32_t, row, 4 * v, 4, w, 505)));
+                } else {
+                    uint32_t e[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) e[i] = 4 * v + i < w ? PANO_AT(row, 4 * v + i, w, 506) : kAll;
+                    k = make_uint4(e[0], e[1], e[2], e[3]);
+                }
+                *reinterpret_cast<uint4*>(&PANO_VEC(uint32_t, gs, 4 * v, 4, w4, 507)) = k;
+            }
+            unsigned m = __vminu2(__vminu2(k.x, k.y), __vminu2(k.z, k.w));
+            m = __vminu2(m, __shfl_xor_sync(kAll, m, 1));
+            m = __vminu2(m, __shfl_xor_sync(kAll, m, 2));
+            m = __vminu2(m, __shfl_xor_sync(kAll, m, 4));
+            if (v < w4 / 4 && (v & 7) == 0) PANO_AT(bm, v / 8, nb, 508) = m;
+            all = __vminu2(all, m);
+        }
+        if ((all & 0xFFFFu) != edt::kNoSite) s_any[0] = 1;
+        if (all >> 16 != edt::kNoSite) s_any[1] = 1;
+    }
+    // groups without an Area3 pixel are written now; the others are listed
+    const bool lvec = (((uintptr_t)lab) & 3) == 0, ovec = (((uintptr_t)out) & 15) == 0;
+    for (int x0 = 128 * wid; x0 < w; x0 += 128 * kNearWarps) {
+        // two groups, four columns a lane
+        const int x = x0 + 4 * lane;
+        unsigned c = 0;
+        if (lvec && x + 4 <= w) {
+            c = __ldg(reinterpret_cast<const unsigned*>(&PANO_VEC(const unsigned char, lab, x, 4, w, 509)));
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (x + i < w) c |= (unsigned)PANO_AT(lab, x + i, w, 509) << (8 * i);
+        }
+        const unsigned three = __ballot_sync(kAll, __vcmpeq4(c, 0x03030303u) != 0u);
+        const bool act = (lane < 16 ? three & 0xFFFFu : three >> 16) != 0u;
+        if ((lane & 15) == 0 && x < w) PANO_AT(list, x / 64, ng, 510) = act;
+        if (act || x >= w) continue;
+        float b[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const unsigned e = c >> (8 * i) & 0xFFu;
+            b[i] = e == 1 ? 0.f : e == 2 ? 1.f : 0.5f;
+        }
+        if (ovec && x + 4 <= w) {
+            PANO_VEC(float4, out, x, 4, w, 511) = make_float4(b[0], b[1], b[2], b[3]);
+        } else {
+            for (int i = 0; i < 4 && x + i < w; ++i) PANO_AT(out, x + i, w, 511) = b[i];
+        }
+    }
+    __syncthreads();
+    if (wid == 0) {
+        int n = 0;
+        for (int g0 = 0; g0 < ng; g0 += 32) {
+            const bool act = g0 + lane < ng && list[g0 + lane];
+            const unsigned m = __ballot_sync(kAll, act);
+            __syncwarp();
+            // written at or before the entries read so far
+            if (act) PANO_AT(list, n + __popc(m & ((1u << lane) - 1u)), ng, 512) = (uint16_t)(g0 + lane);
+            n += __popc(m);
+        }
+        if (lane == 0) s_n = n;
+    }
+    __syncthreads();
+    const int n = s_n;
+    if (n == 0) return;
+    const bool any0 = s_any[0] != 0, any1 = s_any[1] != 0;
+
+    // ---- 2: nearest columns of points 0 .. n
+    auto point_x = [&](int i) { return i < n ? 64 * (int)list[i] : min(w - 1, 64 * (int)list[n - 1] + 63); };
+    if (wid < 4) {
+        const int a = wid & 1, i = wid < 2 ? 0 : n;
+        const int q = (a ? any1 : any0) ? near_search(gs, bm, 16 * a, w, nb, point_x(i), 0, w - 1) : 0;
+        if (lane == 0) PANO_AT(ql, a * (ng + 1) + i, 2 * (ng + 1), 513) = PANO_AT(qh, a * (ng + 1) + i, 2 * (ng + 1), 513) = (uint16_t)q;
+    }
+    __syncthreads();
+    int s = 1;
+    while (2 * s < n) s *= 2;
+    for (; s >= 1; s >>= 1) {
+        const int cnt = (n - 1 + s) / (2 * s);  // odd multiples of s below n
+        // a lane per point and area; the warp searches the long ranges together
+        for (int t0 = 0; t0 < 2 * cnt; t0 += kNearThreads) {
+            const int t = t0 + wid + kNearWarps * lane;
+            const int a = t & 1, i = s * (2 * (t >> 1) + 1), o = a * (ng + 1);
+            int lo = 0, hi = 0;
+            if (t < 2 * cnt) {
+                lo = PANO_AT(ql, o + i - s, 2 * (ng + 1), 514);
+                hi = PANO_AT(qh, o + min(i + s, n), 2 * (ng + 1), 515);
+            }
+            for (unsigned todo = __ballot_sync(kAll, hi - lo > kNearFew); todo; todo &= todo - 1) {
+                const int k = __ffs(todo) - 1;
+                const int l = __shfl_sync(kAll, lo, k), u = __shfl_sync(kAll, hi, k), j = __shfl_sync(kAll, i, k);
+                const int q = near_search(gs, bm, 16 * __shfl_sync(kAll, a, k), w, nb, point_x(j), l, u);
+                if (lane == k) lo = hi = q;
+            }
+            if (t < 2 * cnt) ql[o + i] = (uint16_t)lo, qh[o + i] = (uint16_t)hi;
+        }
+        __syncthreads();
+    }
+
+    // ---- 3: distances and Eq. (1)
+    for (int i = wid; i < n; i += kNearWarps) {
+        const int X = 64 * (int)list[i], x = X + 2 * lane;
+        const unsigned c0 = x < w ? PANO_AT(lab, x, w, 545) : 0, c1 = x + 1 < w ? PANO_AT(lab, x + 1, w, 545) : 0;
+        unsigned d0[2], d1[2];
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            unsigned b0 = 0xFFFFFFFFu, b1 = 0xFFFFFFFFu;
+            if (a ? any1 : any0) {
+                int lo = ql[a * (ng + 1) + i], hi = qh[a * (ng + 1) + i + 1];
+                if (hi - lo > kNearScan) {
+                    // the nearest column jumps in this group, or before the next
+                    // one: bisect on, over the lanes, where the range is long
+                    hi = near_search(gs, bm, 16 * a, w, nb, min(X + 63, w - 1), lo, hi);
+                    for (int st = 16; st >= 1; st >>= 1)
+                        for (int b = 0; b < 32; b += 2 * st) {
+                            const int l = __shfl_sync(kAll, lo, b), u = __shfl_sync(kAll, hi, b), xm = X + 2 * (b + st);
+                            if (u - l <= kNearScan || xm >= w) continue;
+                            const int m = near_search(gs, bm, 16 * a, w, nb, xm, l, u);
+                            if (lane >= b && lane < b + st) hi = m;
+                            if (lane >= b + st && lane < b + 2 * st) lo = m;
+                        }
+                }
+#pragma unroll 1
+                for (int q = lo; q <= hi; ++q) {
+                    const unsigned g = PANO_AT(gs, q, w, 546) >> (16 * a) & 0xFFFFu;
+                    b0 = min(b0, near_cost(g, x - q));
+                    b1 = min(b1, near_cost(g, x + 1 - q));
+                }
+            }
+            d0[a] = b0, d1[a] = b1;
+        }
+        auto eq1 = [&](unsigned c, unsigned e0, unsigned e1) {
+            if (c != 3) return c == 1 ? 0.f : c == 2 ? 1.f : 0.5f;
+            if (!any0 || !any1) return any1 ? 1.f : any0 ? 0.f : 0.5f;
+            const float dl = sqrtf((float)e0), dr = sqrtf((float)e1);
+            return dl / (dl + dr);
+        };
+        const float v0 = eq1(c0, d0[0], d0[1]), v1 = eq1(c1, d1[0], d1[1]);
+        if (ovec && x + 2 <= w) {
+            PANO_VEC(float2, out, x, 2, w, 547) = make_float2(v0, v1);
+        } else {
+            if (x < w) PANO_AT(out, x, w, 547) = v0;
+            if (x + 1 < w) PANO_AT(out, x + 1, w, 547) = v1;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Row pass of larger canvases: one CTA of kRowThreads per row and area, one band of
 // ceil(w / kRowThreads) columns per thread (edt_row.cuh for the steps).
 // The Area1 launch writes the distances to Area1 (FP32 square roots of the
 // exact squared distances, +inf with no Area1 pixel on the canvas) of the
@@ -371,20 +678,37 @@ size_t blend_coeff_scratch_bytes(int h, int w) {
 size_t blend_coeff_row_smem(int w) { return (size_t)4 * w + (size_t)(5 * kRowThreads + 33) * sizeof(int); }
 
 cudaError_t blend_coeff_prepare(int max_smem_bytes) {
-    cudaError_t e = cudaFuncSetAttribute(edt_row_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         max_smem_bytes);
+    cudaError_t e = cudaFuncSetAttribute(edt_near_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)NearSmem(kNearMaxSide).bytes());
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(edt_cols_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ColSmem));
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(edt_cols_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ColSmem));
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(edt_row_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem_bytes);
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(edt_row_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem_bytes);
 }
 
 cudaError_t launch_blend_coeff(const unsigned char* label, int h, int w, long long pitch, float* blend,
                                int blend_pitch, void* scratch, cudaStream_t s) {
+    const bool near = h <= kNearMaxSide && w <= kNearMaxSide;
+    const dim3 grid((w + kColW - 1) / kColW), block(kColW, kColTY);
+    cudaError_t e;
+    if (near) {
+        // rows of whole 16 bytes where the scratch (8 bytes a pixel) has the room for it
+        const int gp = w >= 4 ? (w + 3) / 4 * 4 : w;
+        uint32_t* gb = static_cast<uint32_t*>(scratch);
+        edt_cols_kernel<true><<<grid, block, sizeof(ColSmem), s>>>(label, h, w, pitch, gb, nullptr, nullptr, gp);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        edt_near_kernel<<<h, kNearThreads, NearSmem(w).bytes(), s>>>(label, h, w, pitch, gb, gp, blend, blend_pitch);
+        return cudaGetLastError();
+    }
     uint16_t* g1 = static_cast<uint16_t*>(scratch);
     uint16_t* g2 = g1 + (size_t)h * w;
+    edt_cols_kernel<false><<<grid, block, sizeof(ColSmem), s>>>(label, h, w, pitch, nullptr, g1, g2, w);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     float* dist1 = reinterpret_cast<float*>(g2 + (size_t)h * w);
-    edt_cols_kernel<<<(w + kColW - 1) / kColW, dim3(kColW, kColTY), 0, s>>>(label, h, w, pitch, g1, g2);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
     const size_t smem = blend_coeff_row_smem(w);
     edt_row_kernel<false><<<h, kRowThreads, smem, s>>>(label, h, w, pitch, g1, dist1, blend, blend_pitch);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -172,3 +172,29 @@ def test_bad_arguments_raise():
         binding.blend_coeff(lab, scratch=torch.empty(16, dtype=torch.uint8, device=DEV))
     with pytest.raises(binding.PanoError):
         binding.blend_coeff(lab.float())
+
+
+# The row pass works on groups of 32 columns (loads of 8) and bisects over the
+# groups with Area3; sides above 46000 take the other row pass. Sizes on either
+# side of each, areas that miss from whole columns, and one-group rows.
+@pytest.mark.parametrize("shape,p", [((9, 31), 0.5), ((9, 32), 0.5), ((9, 33), 0.5), ((7, 64), 0.02), ((7, 65), 0.02),
+                                     ((5, 255), 0.01), ((5, 257), 0.003), ((3, 1025), 0.002), ((40, 700), 0.0004),
+                                     ((1, 7), 0.3), ((2, 8), 0.3), ((300, 40), 0.001)])
+def test_sparse_areas_around_the_group_sizes(shape, p):
+    g = np.random.default_rng(shape[1])
+    label = g.choice([1, 2, 3], p=[p, p, 1 - 2 * p], size=shape).astype(np.uint8)
+    label[:, shape[1] // 3: shape[1] // 2] = 0    # columns without a site
+    np.testing.assert_allclose(gpu_blend(label), oracle.blend_coeff(label), rtol=0, atol=TOL)
+
+
+@pytest.mark.parametrize("shape", [(3, 46000), (3, 46001), (46000, 3), (46001, 3)])
+def test_sides_around_the_32_bit_distances(shape):
+    # few sites, so that distances near the largest ones occur
+    label = np.full(shape, 3, dtype=np.uint8)
+    label[0, 0] = 1
+    label[-1, -1] = 2
+    if shape[1] > 3:
+        label[1, shape[1] // 2] = 1
+    ys, xs = (np.random.default_rng(9).integers(0, n, 200) for n in shape)
+    ys[:4], xs[:4] = [0, shape[0] - 1, shape[0] - 1, 0], [shape[1] - 1, 0, 1, 1]
+    np.testing.assert_allclose(gpu_blend(label)[ys, xs], oracle.blend_coeff_at(label, ys, xs), rtol=0, atol=TOL)
