@@ -428,6 +428,7 @@ void pair_lk_args(const pano_flow_ctx* c, const PairPlanes& pp, int l, float* fl
     ka->lambda = c->p.lambda;
     lk_level_tile(ka->w, ka->h, c->tile_w, c->tile_h, &ka->tile_w, &ka->tile_h);
     ka->pyr = pyr_type(c->p.pyr_dtype);
+    ka->early = l < nlev - 1;  // the previous kernel is a coarser level's
 }
 
 }  // namespace pano

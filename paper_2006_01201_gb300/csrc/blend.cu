@@ -88,6 +88,7 @@ __device__ __forceinline__ void blend_pixel(const BlendArgs& a, int x, int y, in
 
 template <typename Tv, int C>
 __global__ void __launch_bounds__(256, 8) blend_kernel(BlendArgs a) {
+    grid_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= a.L.w || y >= a.L.h) return;
@@ -101,6 +102,7 @@ __global__ void __launch_bounds__(256, 8) blend_kernel(BlendArgs a) {
 // every canvas pixel has one writer and the result is deterministic.
 template <typename Tv, int C>
 __global__ void __launch_bounds__(256, 8) rig_blend_kernel(const __grid_constant__ RigBlendArgs r) {
+    grid_begin();
     const int p = blockIdx.z;
     const BlendArgs& a = r.pair[p];
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -122,6 +124,7 @@ __global__ void __launch_bounds__(256, 8) rig_blend_kernel(const __grid_constant
 // crop (zero outside it), any other label writes 0.
 template <typename Tv, int C>
 __global__ void __launch_bounds__(256, 8) compose_kernel(ComposeArgs a) {
+    grid_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int w = a.L.w, h = a.L.h;
@@ -157,6 +160,7 @@ __global__ void __launch_bounds__(256, 8) compose_kernel(ComposeArgs a) {
 
 template <typename Tv>
 __global__ void __launch_bounds__(256) warp_kernel(WarpArgs a) {
+    grid_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int w = a.src.w, h = a.src.h, C = a.src.c;
@@ -178,13 +182,12 @@ cudaError_t launch_blend(const BlendArgs& args, cudaStream_t s) {
     dim3 block(32, 8);
     dim3 grid((a.L.w + 31) / 32, (a.L.h + 7) / 8);
     if (a.L.dtype == 0) {
-        if (a.L.c == 3) blend_kernel<uint8_t, 3><<<grid, block, 0, s>>>(a);
-        else blend_kernel<uint8_t, 1><<<grid, block, 0, s>>>(a);
+        if (a.L.c == 3) return launch_dependent(blend_kernel<uint8_t, 3>, grid, block, 0, s, 0, a);
+        return launch_dependent(blend_kernel<uint8_t, 1>, grid, block, 0, s, 0, a);
     } else {
-        if (a.L.c == 3) blend_kernel<float, 3><<<grid, block, 0, s>>>(a);
-        else blend_kernel<float, 1><<<grid, block, 0, s>>>(a);
+        if (a.L.c == 3) return launch_dependent(blend_kernel<float, 3>, grid, block, 0, s, 0, a);
+        return launch_dependent(blend_kernel<float, 1>, grid, block, 0, s, 0, a);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_rig_blend(const RigBlendArgs& args, cudaStream_t s) {
@@ -200,13 +203,12 @@ cudaError_t launch_rig_blend(const RigBlendArgs& args, cudaStream_t s) {
     dim3 grid((w + 31) / 32, (h + 7) / 8, r.n);
     const ImageDesc& d = r.pair[0].L;
     if (d.dtype == 0) {
-        if (d.c == 3) rig_blend_kernel<uint8_t, 3><<<grid, block, 0, s>>>(r);
-        else rig_blend_kernel<uint8_t, 1><<<grid, block, 0, s>>>(r);
+        if (d.c == 3) return launch_dependent(rig_blend_kernel<uint8_t, 3>, grid, block, 0, s, 0, r);
+        return launch_dependent(rig_blend_kernel<uint8_t, 1>, grid, block, 0, s, 0, r);
     } else {
-        if (d.c == 3) rig_blend_kernel<float, 3><<<grid, block, 0, s>>>(r);
-        else rig_blend_kernel<float, 1><<<grid, block, 0, s>>>(r);
+        if (d.c == 3) return launch_dependent(rig_blend_kernel<float, 3>, grid, block, 0, s, 0, r);
+        return launch_dependent(rig_blend_kernel<float, 1>, grid, block, 0, s, 0, r);
     }
-    return cudaGetLastError();
 }
 
 PANO_BOUNDS_READER(bounds_read_blend)
@@ -215,21 +217,19 @@ cudaError_t launch_compose(const ComposeArgs& a, cudaStream_t s) {
     dim3 block(32, 8);
     dim3 grid((a.L.w + 31) / 32, (a.L.h + 7) / 8);
     if (a.L.dtype == 0) {
-        if (a.L.c == 3) compose_kernel<uint8_t, 3><<<grid, block, 0, s>>>(a);
-        else compose_kernel<uint8_t, 1><<<grid, block, 0, s>>>(a);
+        if (a.L.c == 3) return launch_dependent(compose_kernel<uint8_t, 3>, grid, block, 0, s, 0, a);
+        return launch_dependent(compose_kernel<uint8_t, 1>, grid, block, 0, s, 0, a);
     } else {
-        if (a.L.c == 3) compose_kernel<float, 3><<<grid, block, 0, s>>>(a);
-        else compose_kernel<float, 1><<<grid, block, 0, s>>>(a);
+        if (a.L.c == 3) return launch_dependent(compose_kernel<float, 3>, grid, block, 0, s, 0, a);
+        return launch_dependent(compose_kernel<float, 1>, grid, block, 0, s, 0, a);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_warp(const WarpArgs& a, cudaStream_t s) {
     dim3 block(32, 8);
     dim3 grid((a.src.w + 31) / 32, (a.src.h + 7) / 8);
-    if (a.src.dtype == 0) warp_kernel<uint8_t><<<grid, block, 0, s>>>(a);
-    else warp_kernel<float><<<grid, block, 0, s>>>(a);
-    return cudaGetLastError();
+    if (a.src.dtype == 0) return launch_dependent(warp_kernel<uint8_t>, grid, block, 0, s, 0, a);
+    return launch_dependent(warp_kernel<float>, grid, block, 0, s, 0, a);
 }
 
 }  // namespace pano

@@ -69,7 +69,7 @@ struct ColSmem {
     uint32_t some[kKeptBlocks][2][kColW];     // bit k: thread row k of the block has a feature pixel
 };
 
-__device__ __forceinline__ void col_masks(const unsigned char* __restrict__ label, long long pitch, long long nl,
+__device__ __forceinline__ void col_masks(const unsigned char* label, long long pitch, long long nl,
                                           int h, int x, int y0, uint32_t* m1, uint32_t* m2) {
     uint32_t a = 0, b = 0;
     const int n = min(32, h - y0);
@@ -77,7 +77,7 @@ __device__ __forceinline__ void col_masks(const unsigned char* __restrict__ labe
 #pragma unroll 8
     for (int i = 0; i < 32; ++i) {
         if (i < n) {
-            const unsigned char c = __ldg(&PANO_AT(p, (long long)i * pitch, nl - ((long long)y0 * pitch + x), 501));
+            const unsigned char c = PANO_AT(p, (long long)i * pitch, nl - ((long long)y0 * pitch + x), 501);
             a |= (uint32_t)(c == 1) << i;
             b |= (uint32_t)(c == 2) << i;
         }
@@ -87,11 +87,12 @@ __device__ __forceinline__ void col_masks(const unsigned char* __restrict__ labe
 }
 
 template <bool kPacked>
-__global__ void __launch_bounds__(kColW * kColTY, 2) edt_cols_kernel(const unsigned char* __restrict__ label, int h,
-                                                                    int w, long long pitch, uint32_t* __restrict__ gb,
-                                                                    uint16_t* __restrict__ g1,
-                                                                    uint16_t* __restrict__ g2, int gp) {
+__global__ void __launch_bounds__(kColW * kColTY, 2) edt_cols_kernel(const unsigned char* label, int h,
+                                                                    int w, long long pitch, uint32_t* gb,
+                                                                    uint16_t* g1,
+                                                                    uint16_t* g2, int gp) {
     extern __shared__ __align__(16) unsigned char s_col[];
+    grid_begin();
     ColSmem& S = *reinterpret_cast<ColSmem*>(s_col);
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kColW + tx;
     const int x = blockIdx.x * kColW + tx;
@@ -244,7 +245,7 @@ __device__ __forceinline__ unsigned near_cost(unsigned g, int dx) {
 // Leftmost nearest column of pixel x among [lo, hi], by one warp; some column
 // of [lo, hi] is a nearest one of the whole row. gs and bm hold both areas'
 // values, sh (0 or 16) selects the area.
-__device__ __forceinline__ int near_search(const uint32_t* __restrict__ gs, const uint32_t* __restrict__ bm, int sh, int w,
+__device__ __forceinline__ int near_search(const uint32_t* gs, const uint32_t* bm, int sh, int w,
                                            int nb, int x, int lo, int hi) {
     (void)w, (void)nb;
     const int lane = threadIdx.x & 31;
@@ -286,12 +287,13 @@ __device__ __forceinline__ int near_search(const uint32_t* __restrict__ gs, cons
     return bq;
 }
 
-__global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const unsigned char* __restrict__ label, int h, int w,
-                                                               long long pitch, const uint32_t* __restrict__ gb, int gp,
-                                                               float* __restrict__ blend, int blend_pitch) {
+__global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const unsigned char* label, int h, int w,
+                                                               long long pitch, const uint32_t* gb, int gp, float* blend,
+                                                               int blend_pitch) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     __shared__ int s_n;
     __shared__ unsigned s_any[2];
+    grid_begin();
     const NearSmem L(w);
     const int w4 = L.w4, nb = L.nb, ng = L.ng;
     uint32_t* gs = reinterpret_cast<uint32_t*>(s_dyn);      // [w4] g of both areas
@@ -316,14 +318,14 @@ __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const unsigned c
             uint4 k = make_uint4(kAll, kAll, kAll, kAll);
             if (v < w4 / 4) {
                 if (vec && 4 * v + 4 <= w) {
-                    k = __ldg(reinterpret_cast<const uint4*>(&PANO_VEC(const uint32_t, row, 4 * v, 4, w, 505)));
+                    k = PANO_VEC(const uint4, row, 4 * v, 4, w, 505);
                 } else {
                     uint32_t e[4];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) e[i] = 4 * v + i < w ? PANO_AT(row, 4 * v + i, w, 506) : kAll;
                     k = make_uint4(e[0], e[1], e[2], e[3]);
                 }
-                *reinterpret_cast<uint4*>(&PANO_VEC(uint32_t, gs, 4 * v, 4, w4, 507)) = k;
+                PANO_VEC(uint4, gs, 4 * v, 4, w4, 507) = k;
             }
             unsigned m = __vminu2(__vminu2(k.x, k.y), __vminu2(k.z, k.w));
             m = __vminu2(m, __shfl_xor_sync(kAll, m, 1));
@@ -342,7 +344,7 @@ __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const unsigned c
         const int x = x0 + 4 * lane;
         unsigned c = 0;
         if (lvec && x + 4 <= w) {
-            c = __ldg(reinterpret_cast<const unsigned*>(&PANO_VEC(const unsigned char, lab, x, 4, w, 509)));
+            c = PANO_VEC(const unsigned, lab, x, 4, w, 509);
         } else {
 #pragma unroll
             for (int i = 0; i < 4; ++i)
@@ -699,10 +701,11 @@ cudaError_t launch_blend_coeff(const unsigned char* label, int h, int w, long lo
         // rows of whole 16 bytes where the scratch (8 bytes a pixel) has the room for it
         const int gp = w >= 4 ? (w + 3) / 4 * 4 : w;
         uint32_t* gb = static_cast<uint32_t*>(scratch);
-        edt_cols_kernel<true><<<grid, block, sizeof(ColSmem), s>>>(label, h, w, pitch, gb, nullptr, nullptr, gp);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        edt_near_kernel<<<h, kNearThreads, NearSmem(w).bytes(), s>>>(label, h, w, pitch, gb, gp, blend, blend_pitch);
-        return cudaGetLastError();
+        e = launch_dependent(edt_cols_kernel<true>, grid, block, sizeof(ColSmem), s, 0, label, h, w, pitch, gb, (uint16_t*)nullptr,
+                             (uint16_t*)nullptr, gp);
+        if (e != cudaSuccess) return e;
+        return launch_dependent(edt_near_kernel, dim3(h), dim3(kNearThreads), NearSmem(w).bytes(), s, 0, label, h, w, pitch,
+                                (const uint32_t*)gb, gp, blend, blend_pitch);
     }
     uint16_t* g1 = static_cast<uint16_t*>(scratch);
     uint16_t* g2 = g1 + (size_t)h * w;

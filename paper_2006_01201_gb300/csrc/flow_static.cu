@@ -216,6 +216,7 @@ pano_status pano_flow_pair_static(const pano_flow_params* p, const pano_image* L
         ka.radius = p->radius;
         ka.lambda = p->lambda;
         ka.pyr = kPyrF32;
+        ka.early = l < nlev - 1;  // the previous kernel is a coarser level's
         lk_level_tile(ka.w, ka.h, tw, th, &ka.tile_w, &ka.tile_h);  // as pano_flow_pair
         if ((e = launch_lk_level(ka, 2, s)) != cudaSuccess) return cuda_fail(e, "LK launch");
         if ((e = debug_check(s)) != cudaSuccess) return cuda_fail(e, "LK level (PANO_DEBUG=sync)");

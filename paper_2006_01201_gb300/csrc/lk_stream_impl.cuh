@@ -218,8 +218,9 @@ __device__ __forceinline__ float2 row_sums(float ll, float2 l, float2 c, float2 
 // [ox, ox + RW), the cluster's region rows from oyc on; the pixels
 // [x_lo, x_hi) x [y_lo, y_hi) of the result are written. ox and oyc are even
 // and not negative. A float2 holds the same quantity of the thread's two
-// columns.
-template <int RAD, int R, int WX, int WY, class Ts>
+// columns. LATE: with a.early, what does not depend on the starting flow is done
+// before the previous kernel (the coarser level) has ended.
+template <int RAD, int R, int WX, int WY, bool LATE, class Ts>
 __device__ __forceinline__ void lk_stream_item(const LkArgs& a, int dir, int ox, int oyc, int csize, int x_lo, int x_hi,
                                                int y_lo, int y_hi, unsigned char* smem) {
     using Geo = StreamGeom<RAD, R, WX, WY>;
@@ -268,12 +269,23 @@ __device__ __forceinline__ void lk_stream_item(const LkArgs& a, int dir, int ox,
         }
         copy_async_commit();
     };
+    if (!(LATE && a.early)) {
+        grid_wait();
+        // large levels: the successor's CTAs would only take slots (released
+        // here, a 960 x 1000 pair takes 5% longer, a 4000 x 1500 one 1%)
+        if (LATE) grid_release();
+    }
     stage(T, D.pitchT, ox - 1, oy - (RAD + 1), sT + 1, TP, RW + 3, TH, 110);
-    // reference flow of the cluster; box shift of the CTA
-    const float2 ref = start_flow_s(a, D, min(ox + RW / 2, w - 1), min(oyc + csize * RH / 2, h - 1));
-    const float2 sh = floor_clamped(start_flow_s(a, D, min(ox + RW / 2, w - 1), min(oy + RH / 2, h - 1)), w, h);
-    const float2 off = make_float2(ref.x - sh.x, ref.y - sh.y);
-    stage(J, D.pitchJ, ox + (int)sh.x - kMX, oy + (int)sh.y - kMY, sJ, JP, RW + 2 * kMX, JH, 111);
+    // reference flow of the cluster; the target box, shifted by the flow at the CTA's centre
+    float2 ref, off;
+    auto stage_target = [&]() {
+        ref = start_flow_s(a, D, min(ox + RW / 2, w - 1), min(oyc + csize * RH / 2, h - 1));
+        const float2 sh = floor_clamped(start_flow_s(a, D, min(ox + RW / 2, w - 1), min(oy + RH / 2, h - 1)), w, h);
+        off = make_float2(ref.x - sh.x, ref.y - sh.y);
+        stage(J, D.pitchJ, ox + (int)sh.x - kMX, oy + (int)sh.y - kMY, sJ, JP, RW + 2 * kMX, JH, 111);
+    };
+    const bool late = LATE && a.early;
+    if (!late) stage_target();
     // the box's unused last column marks samples that fall outside the box
     if (tid < 4 * WY) bar_init((unsigned)__cvta_generic_to_shared(smem + Geo::kB) + 8 * tid);
     if (tid < JH) PANO_AT(sJ, tid * JP + JP - 1, NJ, 112) = __int_as_float(0x7fffffff);
@@ -288,7 +300,8 @@ __device__ __forceinline__ void lk_stream_item(const LkArgs& a, int dir, int ox,
     const bool cin0 = x0 < w, cin1 = x0 + 1 < w;
     auto row_in = [&](int j) { return (unsigned)(y0 + dr * j) < (unsigned)h; };
 
-    copy_async_wait<1>();
+    if (late) copy_async_wait<0>();
+    else copy_async_wait<1>();
     __syncthreads();
 
     // ---- template, gradient and the normal matrices
@@ -367,6 +380,11 @@ __device__ __forceinline__ void lk_stream_item(const LkArgs& a, int dir, int ox,
             PANO_AT(sGA, o, NG, 130) = make_float4(i11.x, i11.y, i12.x, i12.y);
             PANO_AT(sGB, o, NG, 131) = i22;
         }
+    }
+
+    if (late) {
+        grid_begin();
+        stage_target();
     }
 
     // ---- starting flow, relative to the reference
@@ -651,7 +669,7 @@ __device__ __forceinline__ void lk_stream_cta(const LkArgs& a, int dir, int bx, 
     const int ox = bx * (Geo::RW - 2 * halo), oy = sy * (csize * Geo::RH - 2 * halo);
     const int x_lo = bx ? ox + halo : 0, x_hi = bx + 1 < nb ? ox + Geo::RW - halo : a.w;
     const int y_lo = sy ? oy + halo : 0, y_hi = sy + 1 < ns ? oy + csize * Geo::RH - halo : a.h;
-    lk_stream_item<RAD, C::R, C::WX, C::WY, Ts>(a, dir, ox, oy, csize, x_lo, x_hi, y_lo, y_hi, smem);
+    lk_stream_item<RAD, C::R, C::WX, C::WY, SMALL, Ts>(a, dir, ox, oy, csize, x_lo, x_hi, y_lo, y_hi, smem);
 }
 
 template <int RAD, bool SMALL, class Ts>
@@ -713,35 +731,16 @@ StreamPlan stream_plan(int w, int h, int iters, int seg_rows) {
     return p;
 }
 
-template <class K, class... A>
-cudaError_t launch_clusters(K kernel, int items, int csize, int threads, size_t smem, cudaStream_t s, const A&... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(items * csize));
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)csize;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
-    const cudaError_t l = cudaGetLastError();
-    return e != cudaSuccess ? e : l;
-}
-
 template <int RAD, class Ts>
 cudaError_t launch_rad_stream(const LkArgs& a, int ndirs, cudaStream_t s) {
     const StreamPlan p = stream_plan<RAD>(a.w, a.h, a.iters, a.seg_rows);
     const int items = p.nb * p.ns * ndirs;
     if (p.small) {
         using Geo = CfgGeom<RAD, true>;
-        return launch_clusters(lk_stream_kernel<RAD, true, Ts>, items, p.csize, Geo::threads, Geo::bytes, s, a, p);
+        return launch_dependent(lk_stream_kernel<RAD, true, Ts>, dim3(items * p.csize), dim3(Geo::threads), Geo::bytes, s, p.csize, a, p);
     }
     using Geo = CfgGeom<RAD, false>;
-    return launch_clusters(lk_stream_kernel<RAD, false, Ts>, items, p.csize, Geo::threads, Geo::bytes, s, a, p);
+    return launch_dependent(lk_stream_kernel<RAD, false, Ts>, dim3(items * p.csize), dim3(Geo::threads), Geo::bytes, s, p.csize, a, p);
 }
 
 // One launch for the pairs that are cut with the same CTA shape and cluster
@@ -770,10 +769,10 @@ cudaError_t launch_rad_batch(const LkBatch& in, cudaStream_t s, int* kernels) {
         cudaError_t e;
         if (plan[first].small) {
             using Geo = CfgGeom<RAD, true>;
-            e = launch_clusters(lk_stream_batch_kernel<RAD, true, Ts>, items, csize, Geo::threads, Geo::bytes, s, b, csize);
+            e = launch_dependent(lk_stream_batch_kernel<RAD, true, Ts>, dim3(items * csize), dim3(Geo::threads), Geo::bytes, s, csize, b, csize);
         } else {
             using Geo = CfgGeom<RAD, false>;
-            e = launch_clusters(lk_stream_batch_kernel<RAD, false, Ts>, items, csize, Geo::threads, Geo::bytes, s, b, csize);
+            e = launch_dependent(lk_stream_batch_kernel<RAD, false, Ts>, dim3(items * csize), dim3(Geo::threads), Geo::bytes, s, csize, b, csize);
         }
         if (e != cudaSuccess) return e;
         ++*kernels;

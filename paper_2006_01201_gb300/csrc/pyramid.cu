@@ -49,7 +49,7 @@ __device__ __forceinline__ void luma4(const ImageDesc& in, const unsigned char* 
     x = PANO_IDX(x, in.w - 3, 316);  // pixels x .. x+3
     if (in.dtype == 0 && in.c == 3 && ((((uintptr_t)row) + 3 * x) & 3) == 0) {
         const uint32_t* p = reinterpret_cast<const uint32_t*>(row + 3 * x);
-        const uint32_t w0 = __ldg(p), w1 = __ldg(p + 1), w2 = __ldg(p + 2);
+        const uint32_t w0 = p[0], w1 = p[1], w2 = p[2];
         const uint32_t b[12] = {w0 & 255, (w0 >> 8) & 255, (w0 >> 16) & 255, w0 >> 24,
                                 w1 & 255, (w1 >> 8) & 255, (w1 >> 16) & 255, w1 >> 24,
                                 w2 & 255, (w2 >> 8) & 255, (w2 >> 16) & 255, w2 >> 24};
@@ -86,6 +86,7 @@ __device__ __forceinline__ void store4(To* o, const float (&v)[4]) {
 
 template <class To>
 __global__ void __launch_bounds__(256) luma_kernel(const __grid_constant__ LumaArgs a) {
+    grid_begin();
     const ImageDesc& in = a.in[blockIdx.z];
     To* out = static_cast<To*>(a.out[blockIdx.z]);
     const int out_pitch = a.out_pitch[blockIdx.z];
@@ -181,6 +182,7 @@ __device__ __forceinline__ void reduce_staged(const float (*s_src)[kPdSW], float
 
 template <class Ts>
 __global__ void __launch_bounds__(256) pyr_down_kernel(const __grid_constant__ PyrDownArgs a) {
+    grid_begin();
     __shared__ __align__(16) float s_src[kPdSH][kPdSW];
     __shared__ float s_v[kPdTH][kPdSW + 1];
     const int z = blockIdx.z;
@@ -205,7 +207,7 @@ __global__ void __launch_bounds__(256) pyr_down_kernel(const __grid_constant__ P
         float* o = &PANO_VEC(float, &s_src[0][0], r * kPdSW + 4 * q, 4, kPdSH * kPdSW, 318);
         if (vec && sx >= 0 && sx + 3 < w) {
             using V = typename Vec4Of<Ts>::type;
-            const V v = __ldg(&PANO_VEC(const V, src, ro + sx, 4, ns, 319));
+            const V v = PANO_VEC(const V, src, ro + sx, 4, ns, 319);
             if constexpr (sizeof(Ts) == 4) widen4(v, o);
             else widen4<Ts>(v, o);
         } else {
@@ -226,6 +228,7 @@ __global__ void __launch_bounds__(256) pyr_down_kernel(const __grid_constant__ P
 // luma_kernel followed by pyr_down_kernel.
 template <class Ts>
 __global__ void __launch_bounds__(256) luma_reduce_kernel(const __grid_constant__ LumaReduceArgs a) {
+    grid_begin();
     __shared__ __align__(16) float s_src[kPdSH][kPdSW];
     __shared__ float s_v[kPdTH][kPdSW + 1];
     const int z = blockIdx.z;
@@ -306,6 +309,7 @@ struct TailSmem {
 
 template <class Ts, int M>
 __global__ void __launch_bounds__(256) pyr_tail_kernel(const __grid_constant__ PyrTailArgs a) {
+    grid_begin();
     extern __shared__ float tsm[];
     const int z = blockIdx.z;
     // level sizes at distance d from the coarsest (ceil of repeated halving
@@ -395,8 +399,7 @@ cudaError_t launch_tail_m(const PyrTailArgs& a, cudaStream_t s) {
         wc = max(wc, w);
     }
     dim3 grid((wc + kTailTC - 1) / kTailTC, (hc + kTailTC - 1) / kTailTC, a.count);
-    pyr_tail_kernel<Ts, M><<<grid, 256, TailSmem<M>::bytes, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(pyr_tail_kernel<Ts, M>, grid, dim3(256), TailSmem<M>::bytes, s, 0, a);
 }
 
 template <class Ts>
@@ -452,12 +455,11 @@ cudaError_t launch_luma_reduce(const LumaReduceArgs& a, cudaStream_t s) {
     dim3 block(256);
     dim3 grid((wd + kPdTW - 1) / kPdTW, (hd + kPdTH - 1) / kPdTH, a.count);
     switch (a.pyr) {
-        case kPyrF32: luma_reduce_kernel<float><<<grid, block, 0, s>>>(a); break;
-        case kPyrBF16: luma_reduce_kernel<__nv_bfloat16><<<grid, block, 0, s>>>(a); break;
-        case kPyrF16: luma_reduce_kernel<__half><<<grid, block, 0, s>>>(a); break;
+        case kPyrF32: return launch_dependent(luma_reduce_kernel<float>, grid, block, 0, s, 0, a);
+        case kPyrBF16: return launch_dependent(luma_reduce_kernel<__nv_bfloat16>, grid, block, 0, s, 0, a);
+        case kPyrF16: return launch_dependent(luma_reduce_kernel<__half>, grid, block, 0, s, 0, a);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 PANO_BOUNDS_READER(bounds_read_pyramid)
@@ -473,12 +475,11 @@ cudaError_t launch_luma(const LumaArgs& a, cudaStream_t s) {
     dim3 block(64, 4);
     dim3 grid((w + 4 * 64 - 1) / (4 * 64), (h + 3) / 4, a.count);
     switch (a.pyr) {
-        case kPyrF32: luma_kernel<float><<<grid, block, 0, s>>>(a); break;
-        case kPyrBF16: luma_kernel<__nv_bfloat16><<<grid, block, 0, s>>>(a); break;
-        case kPyrF16: luma_kernel<__half><<<grid, block, 0, s>>>(a); break;
+        case kPyrF32: return launch_dependent(luma_kernel<float>, grid, block, 0, s, 0, a);
+        case kPyrBF16: return launch_dependent(luma_kernel<__nv_bfloat16>, grid, block, 0, s, 0, a);
+        case kPyrF16: return launch_dependent(luma_kernel<__half>, grid, block, 0, s, 0, a);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_pyr_down(const PyrDownArgs& a, cudaStream_t s) {
@@ -491,12 +492,11 @@ cudaError_t launch_pyr_down(const PyrDownArgs& a, cudaStream_t s) {
     dim3 block(256);
     dim3 grid((wd + kPdTW - 1) / kPdTW, (hd + kPdTH - 1) / kPdTH, a.count);
     switch (a.pyr) {
-        case kPyrF32: pyr_down_kernel<float><<<grid, block, 0, s>>>(a); break;
-        case kPyrBF16: pyr_down_kernel<__nv_bfloat16><<<grid, block, 0, s>>>(a); break;
-        case kPyrF16: pyr_down_kernel<__half><<<grid, block, 0, s>>>(a); break;
+        case kPyrF32: return launch_dependent(pyr_down_kernel<float>, grid, block, 0, s, 0, a);
+        case kPyrBF16: return launch_dependent(pyr_down_kernel<__nv_bfloat16>, grid, block, 0, s, 0, a);
+        case kPyrF16: return launch_dependent(pyr_down_kernel<__half>, grid, block, 0, s, 0, a);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 }  // namespace pano

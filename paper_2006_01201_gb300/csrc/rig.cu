@@ -205,6 +205,7 @@ LkArgs pair_level_args(const pano_rig* r, const RunCall& c, int k, int l, const 
     }
     a.seg_rows = t.seg_rows;
     a.pyr = pyr_type(r->p.pyr_dtype);
+    a.early = l < nlev - 1;  // the previous kernel is a coarser level's (or another launch of this level)
     return a;
 }
 
