@@ -210,13 +210,35 @@ PANO_API pano_status pano_blend_coeff(const unsigned char* label, int h, int w, 
 
 /* E and its gradients for template T and target J (h x w float32, row pitch
  * `pitch` floats) and flow u ((h, w, 2) float32 contiguous).
- * energy: device pointer to one double that receives E (reduced in FP64), or
- * NULL. grad_u ((h, w, 2)), grad_T ((h, w)) and grad_J ((h, w)), all float32
+ * energy: device pointer to one double that receives E (summed per thread in
+ * pairs of floats, exact to about 2^-46, then in FP64), or NULL. grad_u ((h, w, 2)), grad_T ((h, w)) and grad_J ((h, w)), all float32
  * contiguous, receive dE/du, dE/dT and dE/dJ; any may be NULL. dE/dJ is
  * accumulated with atomic additions, so its last bits vary between runs.
  * Errors: INVALID_ARG, CUDA. */
 PANO_API pano_status pano_energy_grad(const float* T, const float* J, int h, int w, int pitch, const float* u,
                                       float alpha, double* energy, float* grad_u, float* grad_T, float* grad_J,
+                                      void* cuda_stream);
+
+/* E and its gradients at pyramid level `level` (0..11) of two full-resolution
+ * planes T0 and J0 (h x w float32, row pitches in floats): T and J of
+ * pano_energy_grad are their level-`level` REDUCE images (the values of
+ * repeated pano_stage_pyr_down calls), u lives on that level, and the
+ * gradients with respect to T0 and J0 are carried back by the transposes.
+ * pano_refine_energy: *energy (device) receives E.
+ * pano_refine_grad: grad_u ((h_l, w_l, 2)), grad_T0 and grad_J0 ((h, w)), all
+ * float32 contiguous, receive the gradients times *scale (a double in device
+ * memory; NULL: 1); any may be NULL. The pyramid is rebuilt, not kept from an
+ * earlier call.
+ * scratch: device memory of at least pano_refine_scratch_bytes(h, w, level)
+ * bytes, 16-byte aligned (may be NULL at level 0). Errors: INVALID_ARG,
+ * UNSUPPORTED, CUDA. */
+PANO_API size_t pano_refine_scratch_bytes(int h, int w, int level);
+PANO_API pano_status pano_refine_energy(const float* T0, const float* J0, int h, int w, int pitch_T, int pitch_J,
+                                        int level, const float* u, float alpha, double* energy, void* scratch,
+                                        size_t scratch_bytes, void* cuda_stream);
+PANO_API pano_status pano_refine_grad(const float* T0, const float* J0, int h, int w, int pitch_T, int pitch_J,
+                                      int level, const float* u, float alpha, const double* scale, float* grad_u,
+                                      float* grad_T0, float* grad_J0, void* scratch, size_t scratch_bytes,
                                       void* cuda_stream);
 
 /* Transpose of pano_stage_pyr_down: given the gradient gdst of the

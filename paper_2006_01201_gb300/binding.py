@@ -86,6 +86,9 @@ SIGNATURES = {
     "pano_flow_launches": ([_VP], ctypes.c_ulonglong),
     "pano_flow_pair_static": ([_PAR, _IMG, _IMG, _VP, _VP, _VP], _I),
     "pano_energy_grad": ([_VP, _VP, _I, _I, _I, _VP, _F, _VP, _VP, _VP, _VP, _VP], _I),
+    "pano_refine_scratch_bytes": ([_I, _I, _I], ctypes.c_size_t),
+    "pano_refine_energy": ([_VP, _VP, _I, _I, _I, _I, _I, _VP, _F, _VP, _VP, ctypes.c_size_t, _VP], _I),
+    "pano_refine_grad": ([_VP, _VP, _I, _I, _I, _I, _I, _VP, _F, _VP, _VP, _VP, _VP, _VP, ctypes.c_size_t, _VP], _I),
     "pano_stage_pyr_down_adjoint": ([_VP, _I, _I, _I, _VP, _I, _VP], _I),
     "pano_stage_luma": ([_IMG, _VP, _I, _VP], _I),
     "pano_stage_pyr_down": ([_VP, _I, _I, _I, _VP, _I, _VP], _I),
@@ -794,6 +797,53 @@ def energy_grad(T, J, u, alpha: float, want_energy=True, want_u=True, want_T=Tru
     _check(load_library().pano_energy_grad(T.data_ptr(), J.data_ptr(), h, w, w, uptr, float(alpha), ptr(E),
                                            ptr(gu), ptr(gt), ptr(gj), _stream_ptr(stream)))
     return E, gu, gt, gj
+
+
+def _refine_args(T0, J0, u, level: int):
+    """(tensors to keep, leading C arguments, scratch) of the refinement calls."""
+    torch = _torch()
+    if level == 0:
+        T0, J0 = T0.contiguous(), J0.contiguous()
+    for t, n in ((T0, "T0"), (J0, "J0")):
+        if t.dtype != torch.float32 or t.dim() != 2 or t.stride(1) != 1 or not t.is_cuda:
+            raise PanoError(PANO_ERR_INVALID_ARG, f"{n} must be a float32 (H, W) CUDA tensor with contiguous rows")
+    h, w = T0.shape
+    hl, wl = h, w
+    for _ in range(level):
+        hl, wl = (hl + 1) // 2, (wl + 1) // 2
+    u = u.contiguous()
+    uptr = _flow_ptr(u, hl, wl, "u")
+    need = int(load_library().pano_refine_scratch_bytes(h, w, level))
+    scratch = torch.empty(need, dtype=torch.uint8, device=T0.device) if need else None
+    return (T0, J0, u), (T0.data_ptr(), J0.data_ptr(), h, w, T0.stride(0), J0.stride(0), level, uptr), scratch
+
+
+def refine_energy(T0, J0, u, level: int, alpha: float, stream=None):
+    """E (float64 0-d tensor) at pyramid level `level` of T0 and J0 (pano_refine_energy)."""
+    torch = _torch()
+    keep, args, scratch = _refine_args(T0, J0, u, level)
+    E = torch.empty((), dtype=torch.float64, device=T0.device)
+    sp, sn = (scratch.data_ptr(), scratch.numel()) if scratch is not None else (None, 0)
+    _check(load_library().pano_refine_energy(*args, float(alpha), E.data_ptr(), sp, sn, _stream_ptr(stream)))
+    return E
+
+
+def refine_grad(T0, J0, u, level: int, alpha: float, scale=None, want_u=True, want_T=True, want_J=True, stream=None):
+    """(dE/du, dE/dT0, dE/dJ0) times `scale`, a float64 0-d CUDA tensor or None
+    (pano_refine_grad); None in the place of a gradient that is not wanted."""
+    torch = _torch()
+    keep, args, scratch = _refine_args(T0, J0, u, level)
+    dev = T0.device
+    gu = torch.empty(keep[2].shape, dtype=torch.float32, device=dev) if want_u else None
+    gt = torch.empty(T0.shape, dtype=torch.float32, device=dev) if want_T else None
+    gj = torch.empty(T0.shape, dtype=torch.float32, device=dev) if want_J else None
+    if scale is not None and (scale.dtype != torch.float64 or scale.numel() != 1 or not scale.is_cuda):
+        raise PanoError(PANO_ERR_INVALID_ARG, "scale must be a float64 CUDA tensor of one element")
+    ptr = lambda t: None if t is None else t.data_ptr()
+    sp, sn = (scratch.data_ptr(), scratch.numel()) if scratch is not None else (None, 0)
+    _check(load_library().pano_refine_grad(*args, float(alpha), ptr(scale), ptr(gu), ptr(gt), ptr(gj), sp, sn,
+                                           _stream_ptr(stream)))
+    return gu, gt, gj
 
 
 def stage_pyr_down_adjoint(gdst, h: int, w: int, stream=None):

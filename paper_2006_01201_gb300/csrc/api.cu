@@ -855,8 +855,9 @@ pano_status pano_energy_grad(const float* T, const float* J, int h, int w, int p
     a.u = u;
     a.h = h;
     a.w = w;
-    a.pitch = pitch;
+    a.pitch = a.pitchJ = pitch;
     a.alpha = alpha;
+    a.scale = nullptr;
     a.energy = energy;
     a.grad_u = grad_u;
     a.grad_T = grad_T;
@@ -871,8 +872,161 @@ pano_status pano_stage_pyr_down_adjoint(const float* gdst, int h, int w, int dst
         return fail(PANO_ERR_INVALID_ARG, "gdst or gsrc NULL or misaligned");
     if (h < 1 || w < 1 || src_pitch < w || dst_pitch < (w + 1) / 2)
         return fail(PANO_ERR_INVALID_ARG, "bad size or pitch");
-    cudaError_t e = launch_pyr_down_adjoint(gdst, h, w, dst_pitch, gsrc, src_pitch, static_cast<cudaStream_t>(cuda_stream));
+    AdjointArgs a;
+    memset(&a, 0, sizeof(a));
+    a.gdst[0] = gdst;
+    a.gsrc[0] = gsrc;
+    a.count = 1;
+    a.h = h;
+    a.w = w;
+    a.dst_pitch = dst_pitch;
+    a.src_pitch = src_pitch;
+    cudaError_t e = launch_pyr_down_adjoint(a, static_cast<cudaStream_t>(cuda_stream));
     return e == cudaSuccess ? PANO_OK : cuda_fail(e, "REDUCE adjoint launch");
+}
+
+// ---------------------------------------------------------------------------
+// The refinement energy at a pyramid level of two full-resolution planes
+// ---------------------------------------------------------------------------
+
+namespace {
+
+// Levels 1 .. level of both planes and of both gradients, in the caller's scratch.
+struct RefineScratch {
+    int h[kMaxLevels], w[kMaxLevels];
+    float* plane[2][kMaxLevels];
+    float* grad[2][kMaxLevels];
+    size_t bytes;
+    RefineScratch(int h0, int w0, int level, void* base) {
+        char* b = static_cast<char*>(base);
+        bytes = 0;
+        h[0] = h0;
+        w[0] = w0;
+        for (int l = 1; l <= level; ++l) {
+            h[l] = (h[l - 1] + 1) / 2;
+            w[l] = (w[l - 1] + 1) / 2;
+            const size_t n = align_up((size_t)h[l] * w[l] * sizeof(float), 256);
+            for (int i = 0; i < 2; ++i, bytes += n) plane[i][l] = b ? reinterpret_cast<float*>(b + bytes) : nullptr;
+            for (int i = 0; i < 2; ++i, bytes += n) grad[i][l] = b ? reinterpret_cast<float*>(b + bytes) : nullptr;
+        }
+    }
+};
+
+pano_status check_refine(const float* T0, const float* J0, int h, int w, int pitch_T, int pitch_J, int level, const float* u,
+                         float alpha, const void* scratch, size_t scratch_bytes) {
+    if (!T0 || !J0 || !u) return fail(PANO_ERR_INVALID_ARG, "T0, J0 or u is NULL");
+    if (h < 1 || w < 1 || pitch_T < w || pitch_J < w) return fail(PANO_ERR_INVALID_ARG, "bad size or pitch");
+    if (level < 0 || level >= kMaxLevels) return fail(PANO_ERR_INVALID_ARG, "level %d not in 0..%d", level, kMaxLevels - 1);
+    if (((uintptr_t)T0) % 4 || ((uintptr_t)J0) % 4 || ((uintptr_t)u) % 8)
+        return fail(PANO_ERR_INVALID_ARG, "T0, J0 or u misaligned");
+    if (!(alpha >= 0.f) || !(alpha < 1e30f)) return fail(PANO_ERR_INVALID_ARG, "alpha must be finite and >= 0");
+    if ((double)h * (double)(pitch_T > pitch_J ? pitch_T : pitch_J) > (double)INT_MAX)
+        return fail(PANO_ERR_UNSUPPORTED, "more than 2^31 elements");
+    const size_t need = RefineScratch(h, w, level, nullptr).bytes;
+    if (need && (!scratch || ((uintptr_t)scratch) % 16 || scratch_bytes < need))
+        return fail(PANO_ERR_INVALID_ARG, "scratch is NULL, not 16-byte aligned or of less than %zu bytes", need);
+    return PANO_OK;
+}
+
+// Levels 1 .. level of both planes, then the energy's arguments at the level.
+cudaError_t refine_level(const float* T0, const float* J0, int pitch_T, int pitch_J, int level, const float* u, float alpha,
+                         const RefineScratch& r, EnergyArgs* a, cudaStream_t s) {
+    PyrSet ps;
+    memset(&ps, 0, sizeof(ps));
+    const float* p0[2] = {T0, J0};
+    const int pitch0[2] = {pitch_T, pitch_J};
+    for (int i = 0; i < 2; ++i) {
+        for (int l = 0; l <= level; ++l) {
+            ps.plane[i][l] = l ? r.plane[i][l] : p0[i];
+            ps.pitch[i][l] = l ? r.w[l] : pitch0[i];
+        }
+        ps.h0[i] = r.h[0];
+        ps.w0[i] = r.w[0];
+    }
+    ps.count = 2;
+    ps.nlev = level + 1;
+    ps.pyr = kPyrF32;
+    int kernels = 0;
+    const cudaError_t e = launch_pyramid_rest(ps, 1, nullptr, s, &kernels);
+    memset(a, 0, sizeof(*a));
+    a->T = static_cast<const float*>(ps.plane[0][level]);
+    a->J = static_cast<const float*>(ps.plane[1][level]);
+    a->pitch = ps.pitch[0][level];
+    a->pitchJ = ps.pitch[1][level];
+    a->h = r.h[level];
+    a->w = r.w[level];
+    a->u = u;
+    a->alpha = alpha;
+    return e;
+}
+
+}  // namespace
+
+size_t pano_refine_scratch_bytes(int h, int w, int level) {
+    if (h < 1 || w < 1 || level < 0 || level >= kMaxLevels) return 0;
+    return RefineScratch(h, w, level, nullptr).bytes;
+}
+
+pano_status pano_refine_energy(const float* T0, const float* J0, int h, int w, int pitch_T, int pitch_J, int level,
+                               const float* u, float alpha, double* energy, void* scratch, size_t scratch_bytes,
+                               void* cuda_stream) {
+    pano_status st = check_refine(T0, J0, h, w, pitch_T, pitch_J, level, u, alpha, scratch, scratch_bytes);
+    if (st != PANO_OK) return st;
+    if (!energy || ((uintptr_t)energy) % 8) return fail(PANO_ERR_INVALID_ARG, "energy is NULL or misaligned");
+    int max_smem = 0;
+    if ((st = ensure_lk_ready(&max_smem)) != PANO_OK) return st;
+    NvtxRange range("pano_refine_energy");
+    cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+    const RefineScratch r(h, w, level, scratch);
+    EnergyArgs a;
+    cudaError_t e = refine_level(T0, J0, pitch_T, pitch_J, level, u, alpha, r, &a, s);
+    a.energy = energy;
+    if (e == cudaSuccess) e = launch_energy_grad(a, s);
+    if (e == cudaSuccess) e = debug_check(s);
+    return e == cudaSuccess ? PANO_OK : cuda_fail(e, "refinement energy launch");
+}
+
+pano_status pano_refine_grad(const float* T0, const float* J0, int h, int w, int pitch_T, int pitch_J, int level,
+                             const float* u, float alpha, const double* scale, float* grad_u, float* grad_T0,
+                             float* grad_J0, void* scratch, size_t scratch_bytes, void* cuda_stream) {
+    pano_status st = check_refine(T0, J0, h, w, pitch_T, pitch_J, level, u, alpha, scratch, scratch_bytes);
+    if (st != PANO_OK) return st;
+    if ((scale && ((uintptr_t)scale) % 8) || (grad_u && ((uintptr_t)grad_u) % 8) || (grad_T0 && ((uintptr_t)grad_T0) % 4) ||
+        (grad_J0 && ((uintptr_t)grad_J0) % 4))
+        return fail(PANO_ERR_INVALID_ARG, "scale or an output misaligned");
+    if (!grad_u && !grad_T0 && !grad_J0) return PANO_OK;
+    int max_smem = 0;
+    if ((st = ensure_lk_ready(&max_smem)) != PANO_OK) return st;
+    NvtxRange range("pano_refine_grad");
+    cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+    const RefineScratch r(h, w, level, scratch);
+    EnergyArgs a;
+    cudaError_t e = refine_level(T0, J0, pitch_T, pitch_J, level, u, alpha, r, &a, s);
+    float* out[2] = {grad_T0, grad_J0};
+    a.scale = scale;
+    a.grad_u = grad_u;
+    a.grad_T = level && grad_T0 ? r.grad[0][level] : grad_T0;
+    a.grad_J = level && grad_J0 ? r.grad[1][level] : grad_J0;
+    if (e == cudaSuccess) e = launch_energy_grad(a, s);
+    for (int l = level; l > 0 && e == cudaSuccess; --l) {
+        // both planes' gradients one level down
+        AdjointArgs g;
+        memset(&g, 0, sizeof(g));
+        for (int i = 0; i < 2; ++i) {
+            if (!out[i]) continue;
+            g.gdst[g.count] = r.grad[i][l];
+            g.gsrc[g.count] = l > 1 ? r.grad[i][l - 1] : out[i];
+            ++g.count;
+        }
+        if (!g.count) break;
+        g.h = r.h[l - 1];
+        g.w = r.w[l - 1];
+        g.dst_pitch = r.w[l];
+        g.src_pitch = r.w[l - 1];
+        e = launch_pyr_down_adjoint(g, s);
+    }
+    if (e == cudaSuccess) e = debug_check(s);
+    return e == cudaSuccess ? PANO_OK : cuda_fail(e, "refinement gradient launch");
 }
 
 }  // extern "C"

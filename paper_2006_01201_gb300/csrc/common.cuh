@@ -272,12 +272,22 @@ struct EnergyArgs {
     const float* T;
     const float* J;
     const float* u;      // (h, w, 2)
-    int h, w, pitch;     // pitch of T and J in floats
+    int h, w;
+    int pitch, pitchJ;   // pitches of T and J in floats
     float alpha;
+    const double* scale; // one double that the gradients are multiplied by, or null
     double* energy;      // one double, or null
     float* grad_u;       // (h, w, 2) or null
     float* grad_T;       // (h, w) or null
     float* grad_J;       // (h, w) or null (zeroed by the launcher)
+};
+
+// Transpose of one REDUCE of up to two planes (refine.cu).
+struct AdjointArgs {
+    const float* gdst[2];  // gradients of the outputs, ceil(h/2) x ceil(w/2)
+    float* gsrc[2];        // gradients of the h x w inputs
+    int count, h, w;
+    int dst_pitch, src_pitch;  // floats
 };
 
 // Launchers: enqueue on `s`, return the launch error (cudaSuccess if none).
@@ -342,8 +352,7 @@ cudaError_t launch_blend_coeff(const unsigned char* label, int h, int w, long lo
                                int blend_pitch, void* scratch, cudaStream_t s);
 
 cudaError_t launch_energy_grad(const EnergyArgs& a, cudaStream_t s);
-cudaError_t launch_pyr_down_adjoint(const float* gdst, int h, int w, int dst_pitch, float* gsrc, int src_pitch,
-                                    cudaStream_t s);
+cudaError_t launch_pyr_down_adjoint(const AdjointArgs& a, cudaStream_t s);
 
 // Index-check records of the debug build (bounds.cuh), one per translation
 // unit: each adds its record to out[4] and clears it (no-ops in the normal

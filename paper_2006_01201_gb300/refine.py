@@ -8,8 +8,9 @@ u on level l is
 
 with T_l, J_l the level-l REDUCE images of T0, J0 (the LK pyramid of the flow
 path) and J_l sampled by the same bilinear clamp-to-edge sampler. The energy
-and every gradient come from the library's kernels (``pano_energy_grad`` and
-the REDUCE transpose ``pano_stage_pyr_down_adjoint``). ``PyramidEnergy``
+and every gradient come from the library's kernels (``pano_refine_energy`` and
+``pano_refine_grad``: the REDUCE levels, the energy or its gradients, and the
+REDUCE transposes in one call each). ``PyramidEnergy``
 stores only T0, J0 and u: the backward pass rebuilds the pyramid levels
 instead of keeping them.
 """
@@ -42,11 +43,14 @@ class PyramidEnergy(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, T0, J0, u, level: int, alpha: float):
-        T = _levels(T0, level)[-1]
-        J = _levels(J0, level)[-1]
-        E, _, _, _ = binding.energy_grad(T.contiguous(), J.contiguous(), u.contiguous(), alpha,
-                                         want_u=False, want_T=False, want_J=False)
         ctx.save_for_backward(T0, J0, u)
+        if T0.shape == J0.shape:
+            E = binding.refine_energy(T0, J0, u, level, alpha)
+        else:
+            T = _levels(T0, level)[-1]
+            J = _levels(J0, level)[-1]
+            E, _, _, _ = binding.energy_grad(T.contiguous(), J.contiguous(), u.contiguous(), alpha,
+                                             want_u=False, want_T=False, want_J=False)
         ctx.level, ctx.alpha = level, alpha
         return E
 
@@ -54,6 +58,10 @@ class PyramidEnergy(torch.autograd.Function):
     def backward(ctx, gE):
         T0, J0, u = ctx.saved_tensors
         need_T, need_J, need_u = ctx.needs_input_grad[:3]
+        if T0.shape == J0.shape:   # the whole step in one call
+            du, dT, dJ = binding.refine_grad(T0, J0, u, ctx.level, ctx.alpha, gE, want_u=need_u, want_T=need_T,
+                                             want_J=need_J)
+            return dT, dJ, du, None, None
         Tl = _levels(T0, ctx.level)          # rebuilt, not stored
         Jl = _levels(J0, ctx.level)
         shapes = [tuple(t.shape) for t in Tl]

@@ -126,3 +126,68 @@ def test_refinement_lowers_energy_and_recovers_flow():
     err = np.hypot(*(u.cpu().numpy() - p.flow_LtoR).transpose(2, 0, 1))[m:-m, m:-m]
     zero = np.hypot(*p.flow_LtoR.transpose(2, 0, 1))[m:-m, m:-m]
     assert err.mean() < 0.35 * zero.mean(), (err.mean(), zero.mean())
+
+
+def _step_arrays(h, w, level, seed):
+    g = np.random.default_rng(seed)
+    T = g.uniform(0, 1, (h, w)).astype(np.float32)
+    J = (0.7 * T + 0.3 * g.uniform(0, 1, (h, w))).astype(np.float32)
+    for _ in range(level):
+        h, w = (h + 1) // 2, (w + 1) // 2
+    # a smooth flow (neighbouring pixels share taps), some noise, some far out
+    u = np.stack(np.broadcast_arrays(1.3 + 0.01 * np.arange(w)[None, :], -0.6 + 0.02 * np.arange(h)[:, None]), -1)
+    u = u + g.normal(0, 0.2, u.shape)
+    u[:: 7, :: 5] *= 40
+    return cuda(T), cuda(J), cuda(u)
+
+
+@pytest.mark.parametrize("h,w,level", [(1, 1, 0), (1, 40, 0), (33, 31, 0), (64, 65, 0), (9, 257, 1), (37, 53, 1), (2, 3, 1),
+                                       (66, 130, 2), (35, 5, 2), (131, 67, 3), (130, 260, 5)])
+def test_one_call_steps_equal_the_composed_ones(h, w, level):
+    # pano_refine_energy / pano_refine_grad against the same step composed from
+    # pano_stage_pyr_down, pano_energy_grad and pano_stage_pyr_down_adjoint;
+    # sums and the dE/dJ scatter differ in their order only
+    T0, J0, u = _step_arrays(h, w, level, 100 + h)
+    T, J = refine._levels(T0, level), refine._levels(J0, level)
+    E, gu, gt, gj = binding.energy_grad(T[-1].contiguous(), J[-1].contiguous(), u, ALPHA)
+    shapes = [tuple(x.shape) for x in T]
+    gt, gj = refine._reduce_transpose(gt, shapes), refine._reduce_transpose(gj, shapes)
+    scale = torch.tensor(-2.5, dtype=torch.float64, device=DEV)
+    E1 = binding.refine_energy(T0, J0, u, level, ALPHA)
+    du, dT, dJ = binding.refine_grad(T0, J0, u, level, ALPHA, scale)
+    assert float(E1) == pytest.approx(float(E), rel=1e-12)
+    for got, ref in ((du, gu), (dT, gt), (dJ, gj)):
+        assert (got - ref * -2.5).abs().max() <= 4e-6 * max(1.0, float(ref.abs().max()))
+    only = binding.refine_grad(T0, J0, u, level, ALPHA, None, want_u=False, want_T=False)
+    assert only[0] is None and only[1] is None
+    assert (only[2] - gj).abs().max() <= 4e-6 * max(1.0, float(gj.abs().max()))
+
+
+@pytest.mark.parametrize("shape", [(1, 1), (1, 2), (2, 1), (3, 3), (4, 5), (5, 4), (6, 6), (64, 16), (65, 17), (130, 131)])
+def test_adjoint_at_the_border_of_its_interior(shape):
+    h, w = shape
+    g = np.random.default_rng(h * 1000 + w).normal(0, 1, ((h + 1) // 2, (w + 1) // 2)).astype(np.float32)
+    got = binding.stage_pyr_down_adjoint(cuda(g), h, w).cpu().numpy()
+    # sixteen products of weights that are powers of two times 6 or 11 sixteenths
+    np.testing.assert_allclose(got, oracle.pyr_down_adjoint(g, h, w), rtol=0, atol=2e-6)
+
+
+@pytest.mark.parametrize("factor", [1.0, 1e-12, 1e-18, 1e17, 0.0])
+def test_energy_of_very_small_and_large_differences(factor):
+    # beyond 1e-15 .. 1e15 the squares are summed in doubles
+    g = np.random.default_rng(5)
+    T = cuda(np.zeros((70, 90)))
+    J = cuda(g.normal(0, 1, (70, 90)) * factor)
+    u = cuda(np.zeros((70, 90, 2)))
+    E = float(binding.energy_grad(T, J, u, ALPHA, want_u=False, want_T=False, want_J=False)[0])
+    assert E == pytest.approx(float((J.double() ** 2).sum()), rel=1e-12)
+
+
+def test_energy_of_non_numbers():
+    T, u = cuda(np.zeros((40, 40))), cuda(np.zeros((40, 40, 2)))
+    for value, check in ((np.inf, np.isinf), (np.nan, np.isnan)):
+        A = np.zeros((40, 40))
+        A[39, 39] = value
+        # at the corner: every tap of the pixel is the value itself for T; J mixes inf - inf
+        E = float(binding.energy_grad(cuda(A), T, u, ALPHA, want_u=False, want_T=False, want_J=False)[0])
+        assert check(E)
