@@ -28,17 +28,18 @@
 // cluster's top and bottom carry a halo of K r pixels, that the steps eat up
 // from outside (108 x 204 of 128 x 224 pixels are left at K r = 10).
 //
-// What bounds it (level 0 of a 4000 x 1500 pair, both directions): the issue
-// of instructions and the shared-memory pipe, at 128 registers a thread and
-// 16 warps an SM. Before, 768 threads worked through 12-row chunks of a ring
-// in shared memory, eleven CTA-wide barriers a chunk: 352 M warp
-// instructions in 568 us. Registers instead of the ring, and two pixels per
-// paired instruction: 177 M instructions. Measured with the same arithmetic:
-// one barrier.cluster a step in place of the counted halos 375 us (every
-// thread's fence in it); the same, sent before and awaited after the inner
-// rows' work, 3% slower on the whole 4000 x 1500 pair than this form;
-// counted halos without the inner rows in between 408 us. Clusters of at most
-// 4 CTAs: 1 to 3% slower; runs of 6 rows: 2 to 6% slower.
+// What bounds it (level 0 of a 4000 x 1500 pair, both directions, 300 us by
+// itself): the issue of instructions (half of the slots) and the shared-memory
+// pipe (57%), at 128 registers a thread and 16 warps an SM. Before, 768
+// threads worked through 12-row chunks of a ring in shared memory, eleven
+// CTA-wide barriers a chunk: 352 M warp instructions and 494 us. Registers
+// instead of the ring, and two pixels per paired instruction: 200 M. Measured
+// with the same arithmetic, on the whole pair (603 us): one barrier.cluster a
+// step, sent before and awaited after the inner rows' work, 3% slower (every
+// thread's fence in it); counted halos without the inner rows in between 10%;
+// the image's border masked behind a branch per row 2.5%; clusters of at most
+// 4 CTAs 1 to 3%, of up to 12 4%, runs of 6 rows 2 to 6%, of 4 rows with 24
+// warps an SM 6%, 256-column regions 17%.
 //
 // The two halves of a warp own two runs on top of each other, the lower one
 // upside down. "Outer" rows (towards another warp) and "inner" rows (towards
@@ -139,15 +140,22 @@ __device__ __forceinline__ void bar_expect(unsigned bar, unsigned bytes) {
 // Waits until the phase of this parity has ended; false if it has not after
 // a bounded number of tries (some 0.1 s at least), which no launch that the
 // host checks let through reaches.
-__device__ __forceinline__ bool bar_wait(unsigned bar, unsigned parity) {
-    unsigned done = 0;
-    for (int n = 0; n < (1 << 22) && !done; ++n)
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-            : "=r"(done)
-            : "r"(bar), "r"(parity)
-            : "memory");
+__device__ __forceinline__ bool bar_try(unsigned bar, unsigned parity) {
+    unsigned done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
     return done != 0;
+}
+__device__ __forceinline__ bool bar_retry(unsigned bar, unsigned parity) {
+    for (int n = 0; n < (1 << 22); ++n)
+        if (bar_try(bar, parity)) return true;
+    return false;
+}
+__device__ __forceinline__ bool bar_wait(unsigned bar, unsigned parity) {
+    return bar_try(bar, parity) || bar_retry(bar, parity);
 }
 // shared-memory load at a byte address plus a constant
 template <int OFF>
@@ -477,147 +485,153 @@ __device__ __forceinline__ void lk_stream_item(const LkArgs& a, int dir, int ox,
     cluster_arrive();  // the staged target and the barriers are visible, the zeroed halos come before a neighbour's rows
     cluster_wait();
 
+    // The steps, with and without the mask of the pixels outside the image (a
+    // branch per row instead would keep the rows' loads from overlapping).
+    auto steps = [&](auto masked) {
 #pragma unroll 1
-    for (int k = 0; k < a.iters; ++k) {
-        float2 Px[R], Py[R];
-        // ---- A: residual products of rows [JB, JE)
-        auto products = [&](auto jb, auto je) {
-            constexpr int JB = decltype(jb)::value, JE = decltype(je)::value;
-            float2 acc = make_float2(0.f, 0.f);
+        for (int k = 0; k < a.iters; ++k) {
+            float2 Px[R], Py[R];
+            // ---- A: residual products of rows [JB, JE)
+            auto products = [&](auto jb, auto je) {
+                constexpr int JB = decltype(jb)::value, JE = decltype(je)::value;
+                float2 acc = make_float2(0.f, 0.f);
 #pragma unroll
-            for (int j = JB; j < JE; ++j) {
-                // J at the pixel + ref + u
-                const float2 o_x = add2(offx, ux[j]), o_y = add2(offy, uy[j]);
-                const float my = fmaf((float)j, mgd, mgy0);
-                const float2 tx = make_float2(__fadd_rd(o_x.x, mgx.x), __fadd_rd(o_x.y, mgx.y));
-                const float2 ty = make_float2(__fadd_rd(o_y.x, my), __fadd_rd(o_y.y, my));
-                const float2 ax = sub2(o_x, sub2(tx, mgx)), ay = sub2(o_y, sub2(ty, dup2(my)));
-                unsigned p0 = (__float_as_uint(ty.x) * (unsigned)JP + __float_as_uint(tx.x)) * 4u + jbase;
-                unsigned p1 = (__float_as_uint(ty.y) * (unsigned)JP + __float_as_uint(tx.y)) * 4u + jbase;
-                // a sample outside the box reads the marker instead
-                p0 = fabsf(o_x.x) < (float)kMX && fabsf(o_y.x) < (float)kMY ? p0 : jnone;
-                p1 = fabsf(o_x.y) < (float)kMX && fabsf(o_y.y) < (float)kMY ? p1 : jnone;
-                PANO_FLAG(p0 - sj > 4u * (NJ - JP - 2) || p1 - sj > 4u * (NJ - JP - 2), 140);
-                const float2 i00 = make_float2(ld_shared<0>(p0), ld_shared<0>(p1));
-                const float2 i10 = make_float2(ld_shared<4>(p0), ld_shared<4>(p1));
-                const float2 i01 = make_float2(ld_shared<4 * JP>(p0), ld_shared<4 * JP>(p1));
-                const float2 i11 = make_float2(ld_shared<4 * JP + 4>(p0), ld_shared<4 * JP + 4>(p1));
-                const float2 top = fma2(ax, sub2(i10, i00), i00), bot = fma2(ax, sub2(i11, i01), i01);
-                const float2 jw = fma2(ay, sub2(bot, top), top);
-                float2 s = fma2(gx[j], ux[j], fma2(gy[j], uy[j], sub2(t[j], jw)));
-                if (edge) {  // nothing from outside the image
-                    const bool in = row_in(j);
-                    if (!(in && cin0)) s.x = 0.f;
-                    if (!(in && cin1)) s.y = 0.f;
-                }
-                acc = add2(acc, s);
-                Px[j] = mul2(gx[j], s);
-                Py[j] = mul2(gy[j], s);
-            }
-            if (__builtin_expect(!(acc.x + acc.y == acc.x + acc.y), 0)) {
-                // some samples (or their inputs) are not numbers: those outside
-                // the box are taken from the global plane
-#pragma unroll
-                for (int j = JB; j < JE; ++j)
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        const float vx = c ? ux[j].y : ux[j].x, vy = c ? uy[j].y : uy[j].x;
-                        const float o_x = off.x + vx, o_y = off.y + vy;
-                        if ((fabsf(o_x) < (float)kMX && fabsf(o_y) < (float)kMY) || !row_in(j) || !(c ? cin1 : cin0)) continue;
-                        const float jw = far_sample(J, D.pitchJ, w, h, x0 + c, y0 + dr * j, ref.x + vx, ref.y + vy);
-                        const float hx = c ? gx[j].y : gx[j].x, hy = c ? gy[j].y : gy[j].x;
-                        const float s = fmaf(hx, vx, fmaf(hy, vy, (c ? t[j].y : t[j].x) - jw));
-                        (c ? Px[j].y : Px[j].x) = hx * s;
-                        (c ? Py[j].y : Py[j].x) = hy * s;
+                for (int j = JB; j < JE; ++j) {
+                    // J at the pixel + ref + u
+                    const float2 o_x = add2(offx, ux[j]), o_y = add2(offy, uy[j]);
+                    const float my = fmaf((float)j, mgd, mgy0);
+                    const float2 tx = make_float2(__fadd_rd(o_x.x, mgx.x), __fadd_rd(o_x.y, mgx.y));
+                    const float2 ty = make_float2(__fadd_rd(o_y.x, my), __fadd_rd(o_y.y, my));
+                    const float2 ax = sub2(o_x, sub2(tx, mgx)), ay = sub2(o_y, sub2(ty, dup2(my)));
+                    unsigned p0 = (__float_as_uint(ty.x) * (unsigned)JP + __float_as_uint(tx.x)) * 4u + jbase;
+                    unsigned p1 = (__float_as_uint(ty.y) * (unsigned)JP + __float_as_uint(tx.y)) * 4u + jbase;
+                    // a sample outside the box reads the marker instead
+                    p0 = fabsf(o_x.x) < (float)kMX && fabsf(o_y.x) < (float)kMY ? p0 : jnone;
+                    p1 = fabsf(o_x.y) < (float)kMX && fabsf(o_y.y) < (float)kMY ? p1 : jnone;
+                    PANO_FLAG(p0 - sj > 4u * (NJ - JP - 2) || p1 - sj > 4u * (NJ - JP - 2), 140);
+                    const float2 i00 = make_float2(ld_shared<0>(p0), ld_shared<0>(p1));
+                    const float2 i10 = make_float2(ld_shared<4>(p0), ld_shared<4>(p1));
+                    const float2 i01 = make_float2(ld_shared<4 * JP>(p0), ld_shared<4 * JP>(p1));
+                    const float2 i11 = make_float2(ld_shared<4 * JP + 4>(p0), ld_shared<4 * JP + 4>(p1));
+                    const float2 top = fma2(ax, sub2(i10, i00), i00), bot = fma2(ax, sub2(i11, i01), i01);
+                    const float2 jw = fma2(ay, sub2(bot, top), top);
+                    float2 s = fma2(gx[j], ux[j], fma2(gy[j], uy[j], sub2(t[j], jw)));
+                    if constexpr (decltype(masked)::value) {  // nothing from outside the image
+                        const bool in = row_in(j);
+                        if (!(in && cin0)) s.x = 0.f;
+                        if (!(in && cin1)) s.y = 0.f;
                     }
-            }
-        };
-        // ---- C: row sums, solve, update of row j with column sums (vx, vy)
-        auto update = [&](int j, float2 vx, float2 vy) {
-            const float4 l = PANO_AT(sV, vo + j * VP - 1, NV, 146), r = PANO_AT(sV, vo + j * VP + 1, NV, 147);
-            float4 l2 = make_float4(0.f, 0.f, 0.f, 0.f), r2 = l2;
-            if constexpr (RAD == 3) {
-                l2 = PANO_AT(sV, vo + j * VP - 2, NV, 148);
-                r2 = PANO_AT(sV, vo + j * VP + 2, NV, 149);
-            }
-            const float2 mx = row_sums<RAD>(l2.y, make_float2(l.x, l.y), vx, make_float2(r.x, r.y), r2.x);
-            const float2 my = row_sums<RAD>(l2.w, make_float2(l.z, l.w), vy, make_float2(r.z, r.w), r2.z);
-            const float4 ga = PANO_AT(sGA, go + j * NP, NG, 152);
-            const float2 gb = PANO_AT(sGB, go + j * NP, NG, 153), g11 = make_float2(ga.x, ga.y), g12 = make_float2(ga.z, ga.w);
-            const float2 qx = fma2(lam2, ux[j], mx), qy = fma2(lam2, uy[j], my);
-            ux[j] = fma2(g11, qx, mul2(g12, qy));
-            uy[j] = fma2(g12, qx, mul2(gb, qy));
-        };
+                    acc = add2(acc, s);
+                    Px[j] = mul2(gx[j], s);
+                    Py[j] = mul2(gy[j], s);
+                }
+                if (__builtin_expect(!(acc.x + acc.y == acc.x + acc.y), 0)) {
+                    // some samples (or their inputs) are not numbers: those outside
+                    // the box are taken from the global plane
+#pragma unroll
+                    for (int j = JB; j < JE; ++j)
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            const float vx = c ? ux[j].y : ux[j].x, vy = c ? uy[j].y : uy[j].x;
+                            const float o_x = off.x + vx, o_y = off.y + vy;
+                            if ((fabsf(o_x) < (float)kMX && fabsf(o_y) < (float)kMY) || !row_in(j) || !(c ? cin1 : cin0)) continue;
+                            const float jw = far_sample(J, D.pitchJ, w, h, x0 + c, y0 + dr * j, ref.x + vx, ref.y + vy);
+                            const float hx = c ? gx[j].y : gx[j].x, hy = c ? gy[j].y : gy[j].x;
+                            const float s = fmaf(hx, vx, fmaf(hy, vy, (c ? t[j].y : t[j].x) - jw));
+                            (c ? Px[j].y : Px[j].x) = hx * s;
+                            (c ? Py[j].y : Py[j].x) = hy * s;
+                        }
+                }
+            };
+            // ---- C: row sums, solve, update of row j with column sums (vx, vy)
+            auto update = [&](int j, float2 vx, float2 vy) {
+                const float4 l = PANO_AT(sV, vo + j * VP - 1, NV, 146), r = PANO_AT(sV, vo + j * VP + 1, NV, 147);
+                float4 l2 = make_float4(0.f, 0.f, 0.f, 0.f), r2 = l2;
+                if constexpr (RAD == 3) {
+                    l2 = PANO_AT(sV, vo + j * VP - 2, NV, 148);
+                    r2 = PANO_AT(sV, vo + j * VP + 2, NV, 149);
+                }
+                const float2 mx = row_sums<RAD>(l2.y, make_float2(l.x, l.y), vx, make_float2(r.x, r.y), r2.x);
+                const float2 my = row_sums<RAD>(l2.w, make_float2(l.z, l.w), vy, make_float2(r.z, r.w), r2.z);
+                const float4 ga = PANO_AT(sGA, go + j * NP, NG, 152);
+                const float2 gb = PANO_AT(sGB, go + j * NP, NG, 153), g11 = make_float2(ga.x, ga.y), g12 = make_float2(ga.z, ga.w);
+                const float2 qx = fma2(lam2, ux[j], mx), qy = fma2(lam2, uy[j], my);
+                ux[j] = fma2(g11, qx, mul2(g12, qy));
+                uy[j] = fma2(g12, qx, mul2(gb, qy));
+            };
 
-        // the outer rows first: they are on their way while the others are formed
-        products(std::integral_constant<int, 0>{}, std::integral_constant<int, RAD>{});
-        if (send) {
+            // the outer rows first: they are on their way while the others are formed
+            products(std::integral_constant<int, 0>{}, std::integral_constant<int, RAD>{});
+            if (send) {
 #pragma unroll
-            for (int j = 0; j < RAD; ++j)
-                cluster_send(odst + ((k & 1) * (NO / 2) + j * NP) * (unsigned)sizeof(float4), bdst + (k & 1) * (WY * 16), Px[j], Py[j]);
-        }
-        __syncwarp();
-        // nobody sends any more: no CTA ends before its neighbours are here
-        if (k + 1 == a.iters) cluster_arrive_relaxed();
-        products(std::integral_constant<int, RAD>{}, std::integral_constant<int, R>{});
-        __syncwarp();
-        // ---- B: column sums of the rows that need no outer halo
-        float2 hx[RAD], hy[RAD];  // sums of rows 0 .. i + RAD
-        {
-            float2 e[R + RAD], f[R + RAD];
-#pragma unroll
-            for (int j = 0; j < R; ++j) e[j] = Px[j], f[j] = Py[j];
-#pragma unroll
-            for (int i = 0; i < RAD; ++i) {
-                // the other half's inner rows
-                e[R + i].x = __shfl_xor_sync(0xffffffffu, Px[R - 1 - i].x, 16);
-                e[R + i].y = __shfl_xor_sync(0xffffffffu, Px[R - 1 - i].y, 16);
-                f[R + i].x = __shfl_xor_sync(0xffffffffu, Py[R - 1 - i].x, 16);
-                f[R + i].y = __shfl_xor_sync(0xffffffffu, Py[R - 1 - i].y, 16);
-            }
-            hx[0] = e[0], hy[0] = f[0];
-#pragma unroll
-            for (int i = 1; i <= RAD; ++i) hx[0] = add2(hx[0], e[i]), hy[0] = add2(hy[0], f[i]);
-#pragma unroll
-            for (int i = 1; i < RAD; ++i) hx[i] = add2(hx[i - 1], e[RAD + i]), hy[i] = add2(hy[i - 1], f[RAD + i]);
-            float2 vx[R - RAD], vy[R - RAD];
-            window_sums<RAD, R - RAD>(e, vx);
-            window_sums<RAD, R - RAD>(f, vy);
-#pragma unroll
-            for (int j = RAD; j < R; ++j) {
-                Px[j] = vx[j - RAD], Py[j] = vy[j - RAD];
-                PANO_AT(sV, vo + j * VP, NV, 145) = make_float4(Px[j].x, Px[j].y, Py[j].x, Py[j].y);
-            }
-        }
-        named_barrier<32 * WX>(1 + wy);
-#pragma unroll
-        for (int j = RAD; j < R; ++j) update(j, Px[j], Py[j]);
-        // ---- and of the outer rows, when the neighbours' rows are here
-        {
-            const unsigned bar = bown + (k & 1) * (WY * 16);
-            const unsigned ph = (unsigned)(k >> 1) & 1;
-            if (from_above) lost |= !bar_wait(bar, ph);
-            if (from_below) lost |= !bar_wait(bar + 8, ph);
-            if (wx == 0 && lane == 0 && k + 2 < a.iters) {
-                if (from_above) bar_expect(bar, kHaloBytes);
-                if (from_below) bar_expect(bar + 8, kHaloBytes);
+                for (int j = 0; j < RAD; ++j)
+                    cluster_send(odst + ((k & 1) * (NO / 2) + j * NP) * (unsigned)sizeof(float4), bdst + (k & 1) * (WY * 16), Px[j], Py[j]);
             }
             __syncwarp();
-            float2 ex = make_float2(0.f, 0.f), ey = ex;
+            // nobody sends any more: no CTA ends before its neighbours are here
+            if (k + 1 == a.iters) cluster_arrive_relaxed();
+            products(std::integral_constant<int, RAD>{}, std::integral_constant<int, R>{});
+            __syncwarp();
+            // ---- B: column sums of the rows that need no outer halo
+            float2 hx[RAD], hy[RAD];  // sums of rows 0 .. i + RAD
+            {
+                float2 e[R + RAD], f[R + RAD];
 #pragma unroll
-            for (int i = RAD - 1; i >= 0; --i) {
-                // row i lacks the halo's first RAD - i rows
-                const float4 o = PANO_AT(sO, (k & 1) * (NO / 2) + oslot + (RAD - 1 - i) * NP, NO, 144);
-                ex = i == RAD - 1 ? make_float2(o.x, o.y) : add2(ex, make_float2(o.x, o.y));
-                ey = i == RAD - 1 ? make_float2(o.z, o.w) : add2(ey, make_float2(o.z, o.w));
-                hx[i] = add2(hx[i], ex), hy[i] = add2(hy[i], ey);
-                PANO_AT(sV, vo + i * VP, NV, 145) = make_float4(hx[i].x, hx[i].y, hy[i].x, hy[i].y);
+                for (int j = 0; j < R; ++j) e[j] = Px[j], f[j] = Py[j];
+#pragma unroll
+                for (int i = 0; i < RAD; ++i) {
+                    // the other half's inner rows
+                    e[R + i].x = __shfl_xor_sync(0xffffffffu, Px[R - 1 - i].x, 16);
+                    e[R + i].y = __shfl_xor_sync(0xffffffffu, Px[R - 1 - i].y, 16);
+                    f[R + i].x = __shfl_xor_sync(0xffffffffu, Py[R - 1 - i].x, 16);
+                    f[R + i].y = __shfl_xor_sync(0xffffffffu, Py[R - 1 - i].y, 16);
+                }
+                hx[0] = e[0], hy[0] = f[0];
+#pragma unroll
+                for (int i = 1; i <= RAD; ++i) hx[0] = add2(hx[0], e[i]), hy[0] = add2(hy[0], f[i]);
+#pragma unroll
+                for (int i = 1; i < RAD; ++i) hx[i] = add2(hx[i - 1], e[RAD + i]), hy[i] = add2(hy[i - 1], f[RAD + i]);
+                float2 vx[R - RAD], vy[R - RAD];
+                window_sums<RAD, R - RAD>(e, vx);
+                window_sums<RAD, R - RAD>(f, vy);
+#pragma unroll
+                for (int j = RAD; j < R; ++j) {
+                    Px[j] = vx[j - RAD], Py[j] = vy[j - RAD];
+                    PANO_AT(sV, vo + j * VP, NV, 145) = make_float4(Px[j].x, Px[j].y, Py[j].x, Py[j].y);
+                }
             }
-        }
-        named_barrier<32 * WX>(1 + wy);
+            named_barrier<32 * WX>(1 + wy);
 #pragma unroll
-        for (int i = 0; i < RAD; ++i) update(i, hx[i], hy[i]);
-    }
+            for (int j = RAD; j < R; ++j) update(j, Px[j], Py[j]);
+            // ---- and of the outer rows, when the neighbours' rows are here
+            {
+                const unsigned bar = bown + (k & 1) * (WY * 16);
+                const unsigned ph = (unsigned)(k >> 1) & 1;
+                if (from_above) lost |= !bar_wait(bar, ph);
+                if (from_below) lost |= !bar_wait(bar + 8, ph);
+                if (wx == 0 && lane == 0 && k + 2 < a.iters) {
+                    if (from_above) bar_expect(bar, kHaloBytes);
+                    if (from_below) bar_expect(bar + 8, kHaloBytes);
+                }
+                __syncwarp();
+                float2 ex = make_float2(0.f, 0.f), ey = ex;
+#pragma unroll
+                for (int i = RAD - 1; i >= 0; --i) {
+                    // row i lacks the halo's first RAD - i rows
+                    const float4 o = PANO_AT(sO, (k & 1) * (NO / 2) + oslot + (RAD - 1 - i) * NP, NO, 144);
+                    ex = i == RAD - 1 ? make_float2(o.x, o.y) : add2(ex, make_float2(o.x, o.y));
+                    ey = i == RAD - 1 ? make_float2(o.z, o.w) : add2(ey, make_float2(o.z, o.w));
+                    hx[i] = add2(hx[i], ex), hy[i] = add2(hy[i], ey);
+                    PANO_AT(sV, vo + i * VP, NV, 145) = make_float4(hx[i].x, hx[i].y, hy[i].x, hy[i].y);
+                }
+            }
+            named_barrier<32 * WX>(1 + wy);
+#pragma unroll
+            for (int i = 0; i < RAD; ++i) update(i, hx[i], hy[i]);
+        }
+    };
+    if (edge) steps(std::true_type{});
+    else steps(std::false_type{});
 
     cluster_wait();
     // ---- the result (not a number where a neighbour's rows never came)
