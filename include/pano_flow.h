@@ -339,7 +339,8 @@ PANO_API pano_status pano_stage_luma_pyr(const pano_image* in, float* Y, int y_p
 
 /* Levels 1 .. nlev-1 of the pyramid of Y (h x w, row pitch `pitch` floats)
  * with the launch sequence pano_flow_pair uses (one-level REDUCE launches
- * for levels 1 and 2, several levels per launch after that): levels[l - 1]
+ * for levels 1 and 2 and from planes of a million pixels, several levels per
+ * launch after that): levels[l - 1]
  * receives level l, ceil(h / 2^l) x ceil(w / 2^l), row pitch pitches[l - 1]
  * floats. The same values as nlev - 1 pano_stage_pyr_down calls, bit for
  * bit. nlev in 2..12. */

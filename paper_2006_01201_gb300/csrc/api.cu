@@ -313,7 +313,13 @@ cudaError_t launch_pyramid_rest(const PyrSet& ps, int first, Trace* tr, cudaStre
     int l = first;
     while (l < ps.nlev) {
         const int m = ps.nlev - l < kTailMaxLevels ? ps.nlev - l : kTailMaxLevels;
-        if (l >= 3 && m >= 2) {
+        long long most = 0;  // pixels of the largest plane's level l - 1
+        for (int i = 0; i < ps.count; ++i) {
+            int sh, sw;
+            size(i, l - 1, &sh, &sw);
+            most = (long long)sh * sw > most ? (long long)sh * sw : most;
+        }
+        if (l >= 3 && m >= 2 && most < kTailMaxPixels) {
             // levels l .. l+m-1 from level l-1 in one launch
             PyrTailArgs ta;
             memset(&ta, 0, sizeof(ta));

@@ -163,6 +163,10 @@ struct LumaReduceArgs {
 // Several REDUCE steps of up to kMaxPlanes planes in one launch: levels
 // s+1 .. s+levels from level s (pyramid.cu, pyr_tail_kernel).
 constexpr int kTailMaxLevels = 4;
+// One launch per level for larger planes: the tail's blocks stage the whole
+// footprint of their coarsest pixels, one or two blocks an SM. (Four levels
+// from 2000 x 1500 pixels: 83 us as a tail, 23 us with level 3 by itself.)
+constexpr long long kTailMaxPixels = 1000000;
 struct PyrTailArgs {
     const void* src[kMaxPlanes];    // level s, planes of type pyr
     int src_pitch[kMaxPlanes];

@@ -74,7 +74,8 @@ bool pick_tile(int iters, int radius, int max_smem, int* tw, int* th);
 pano_status ensure_lk_ready(int* max_smem_out);
 
 // The pyramid levels below level 1 (or 0): one REDUCE launch per level for
-// levels 1 and 2, then launches of up to four levels each. plane/pitch give
+// levels 1 and 2 and from planes of kTailMaxPixels, then launches of up to four
+// levels each. plane/pitch give
 // every level of every plane (level 0 of a plane may be the strip itself);
 // h0/w0 the level-0 sizes. Launches are traced in *tr (if not null) and
 // added to *kernels.

@@ -29,36 +29,98 @@ __device__ __forceinline__ float byte_f(uint32_t b) { return __uint_as_float(0x4
 // forms level 0 (so that all of them give the same bits).
 __device__ __forceinline__ float luma3(float r, float g, float b) { return fmaf(0.114f, b, fmaf(0.587f, g, 0.299f * r)); }
 
+// Byte k of a word as float: one byte permutation puts it below the exponent.
+template <int K>
+__device__ __forceinline__ float word_byte_f(uint32_t w) {
+    return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440 | K)) - 8388608.0f;
+}
+
+// Sample type and channels of an image, known when the kernel is compiled.
+template <int DTYPE, int C>
+struct ImageKind { static constexpr int dtype = DTYPE, c = C; };
+
+template <class K>
 __device__ __forceinline__ float luma_at(const ImageDesc& in, const unsigned char* row, int x) {
     x = PANO_IDX(x, in.w, 315);
-    if (in.dtype == 0) {
-        if (in.c == 3) {
+    if constexpr (K::dtype == 0) {
+        if constexpr (K::c == 3) {
             const uint8_t* px = row + 3 * x;
             return luma3(byte_f(px[0]), byte_f(px[1]), byte_f(px[2])) * kInv255;
         }
         return byte_f(row[x]) * kInv255;
+    } else {
+        const float* r = reinterpret_cast<const float*>(row);
+        if constexpr (K::c == 3) return luma3(r[3 * x], r[3 * x + 1], r[3 * x + 2]);
+        return r[x];
     }
-    const float* r = reinterpret_cast<const float*>(row);
-    if (in.c == 3) return luma3(r[3 * x], r[3 * x + 1], r[3 * x + 2]);
-    return r[x];
 }
 
-// Luma of the four pixels x .. x+3 of a row (all inside the row): 12 aligned
-// bytes for u8 RGB when the address allows it, else one pixel at a time.
-__device__ __forceinline__ void luma4(const ImageDesc& in, const unsigned char* row, int x, float (&v)[4]) {
-    x = PANO_IDX(x, in.w - 3, 316);  // pixels x .. x+3
-    if (in.dtype == 0 && in.c == 3 && ((((uintptr_t)row) + 3 * x) & 3) == 0) {
-        const uint32_t* p = reinterpret_cast<const uint32_t*>(row + 3 * x);
-        const uint32_t w0 = p[0], w1 = p[1], w2 = p[2];
-        const uint32_t b[12] = {w0 & 255, (w0 >> 8) & 255, (w0 >> 16) & 255, w0 >> 24,
-                                w1 & 255, (w1 >> 8) & 255, (w1 >> 16) & 255, w1 >> 24,
-                                w2 & 255, (w2 >> 8) & 255, (w2 >> 16) & 255, w2 >> 24};
+// The N words from byte address p on, as they would be read from an aligned
+// address: N or N + 1 aligned loads and a funnel shift each. The bytes of the
+// aligned words before and after must belong to the image.
+template <int N>
+__device__ __forceinline__ void load_words(const unsigned char* p, uint32_t (&w)[N]) {
+    const unsigned off = (unsigned)((uintptr_t)p & 3);
+    const uint32_t* q = reinterpret_cast<const uint32_t*>(p - off);
+    if (off == 0) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = luma3(byte_f(b[3 * k]), byte_f(b[3 * k + 1]), byte_f(b[3 * k + 2])) * kInv255;
+        for (int i = 0; i < N; ++i) w[i] = q[i];
         return;
     }
+    uint32_t lo = q[0];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = luma_at(in, row, x + k);
+    for (int i = 0; i < N; ++i) {
+        const uint32_t hi = q[i + 1];
+        w[i] = __funnelshift_r(lo, hi, 8 * off);
+        lo = hi;
+    }
+}
+
+// Luma of the four pixels x .. x+3 of a row (all inside the row). u8: by
+// 32-bit words, where three more bytes on either side belong to the row or the
+// address is aligned (a byte at a time, the 48 M gray pixels of an 8000 x 6000
+// strip pair took 220 us with level 1, by words 156 us). float32: 16-byte
+// loads where the address allows it.
+template <class K>
+__device__ __forceinline__ void luma4(const ImageDesc& in, const unsigned char* row, int x, float (&v)[4]) {
+    x = PANO_IDX(x, in.w - 3, 316);  // pixels x .. x+3
+    constexpr int C = K::c;
+    if constexpr (K::dtype == 0) {
+        const int n = C * in.w, o = C * x;  // bytes of the row, first byte
+        if ((((uintptr_t)(row + o)) & 3) == 0 || (o >= 3 && o + 4 * C + 3 <= n)) {
+            uint32_t w[C];
+            load_words<C>(row + o, w);
+            if constexpr (C == 3) {
+                v[0] = luma3(word_byte_f<0>(w[0]), word_byte_f<1>(w[0]), word_byte_f<2>(w[0])) * kInv255;
+                v[1] = luma3(word_byte_f<3>(w[0]), word_byte_f<0>(w[1]), word_byte_f<1>(w[1])) * kInv255;
+                v[2] = luma3(word_byte_f<2>(w[1]), word_byte_f<3>(w[1]), word_byte_f<0>(w[2])) * kInv255;
+                v[3] = luma3(word_byte_f<1>(w[2]), word_byte_f<2>(w[2]), word_byte_f<3>(w[2])) * kInv255;
+            } else {
+                v[0] = word_byte_f<0>(w[0]) * kInv255;
+                v[1] = word_byte_f<1>(w[0]) * kInv255;
+                v[2] = word_byte_f<2>(w[0]) * kInv255;
+                v[3] = word_byte_f<3>(w[0]) * kInv255;
+            }
+            return;
+        }
+    } else {
+        const float* p = reinterpret_cast<const float*>(row) + C * x;
+        if ((((uintptr_t)p) & 15) == 0) {
+            const float4 a = *reinterpret_cast<const float4*>(p);
+            if constexpr (C == 3) {
+                const float4 b = *reinterpret_cast<const float4*>(p + 4), c = *reinterpret_cast<const float4*>(p + 8);
+                v[0] = luma3(a.x, a.y, a.z);
+                v[1] = luma3(a.w, b.x, b.y);
+                v[2] = luma3(b.z, b.w, c.x);
+                v[3] = luma3(c.y, c.z, c.w);
+            } else {
+                v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+            }
+            return;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = luma_at<K>(in, row, x + k);
 }
 
 // Four consecutive outputs: one 16-byte store for float32 rows, one 8-byte
@@ -84,7 +146,7 @@ __device__ __forceinline__ void store4(To* o, const float (&v)[4]) {
     }
 }
 
-template <class To>
+template <class To, class K>
 __global__ void __launch_bounds__(256) luma_kernel(const __grid_constant__ LumaArgs a) {
     grid_begin();
     const ImageDesc& in = a.in[blockIdx.z];
@@ -97,12 +159,12 @@ __global__ void __launch_bounds__(256) luma_kernel(const __grid_constant__ LumaA
     To* orow = out + (long long)y * out_pitch;
     if (x + 4 <= in.w) {
         float v[4];
-        luma4(in, row, x, v);
+        luma4<K>(in, row, x, v);
         store4(orow + x, v);
         return;
     }
     const int n = min(4, in.w - x);
-    for (int k = 0; k < n; ++k) orow[x + k] = from_f32<To>(luma_at(in, row, x + k));
+    for (int k = 0; k < n; ++k) orow[x + k] = from_f32<To>(luma_at<K>(in, row, x + k));
 }
 
 // ---------------------------------------------------------------------------
@@ -147,20 +209,28 @@ __device__ __forceinline__ void widen4(const uint2& v, float* o) {
 }
 
 // Blur the staged footprint along y at the even rows and along x at the even
-// columns, and store the 64 x 16 destination tile (one barrier inside).
+// columns, and store the 64 x 16 destination tile (one barrier inside). Along
+// y a thread forms two rows of four columns from seven 16-byte loads.
 template <class Ts>
-__device__ __forceinline__ void reduce_staged(const float (*s_src)[kPdSW], float (*s_v)[kPdSW + 1], int xd0, int yd0,
+__device__ __forceinline__ void reduce_staged(const float (*s_src)[kPdSW], float (*s_v)[kPdSW], int xd0, int yd0,
                                               int wd, int hd, Ts* __restrict__ dst, int dst_pitch) {
     const int tid = threadIdx.x;
-    for (int i = tid; i < kPdTH * kPdSW; i += 256) {
-        int r = i / kPdSW, c = i - r * kPdSW;
-        int sr = 2 * r + 2;
-        const float* S = &s_src[0][0];
-        constexpr int NS = kPdSH * kPdSW;
-        PANO_AT(&s_v[0][0], r * (kPdSW + 1) + c, kPdTH * (kPdSW + 1), 311) =
-            reduce5(PANO_AT(S, (sr - 2) * kPdSW + c, NS, 312), PANO_AT(S, (sr - 1) * kPdSW + c, NS, 312),
-                    PANO_AT(S, sr * kPdSW + c, NS, 312), PANO_AT(S, (sr + 1) * kPdSW + c, NS, 312),
-                    PANO_AT(S, (sr + 2) * kPdSW + c, NS, 312));
+    const float* S = &s_src[0][0];
+    float* V = &s_v[0][0];
+    constexpr int NS = kPdSH * kPdSW, NV = kPdTH * kPdSW;
+    (void)NS, (void)NV;
+    for (int i = tid; i < kPdTH / 2 * kPdQ; i += 256) {
+        const int r = i / kPdQ, c = 4 * (i - r * kPdQ);  // destination rows 2 r and 2 r + 1, columns c .. c + 3
+        float4 a[7];
+#pragma unroll
+        for (int k = 0; k < 7; ++k) a[k] = PANO_VEC(const float4, S, (4 * r + k) * kPdSW + c, 4, NS, 312);
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            PANO_VEC(float4, V, (2 * r + k) * kPdSW + c, 4, NV, 311) =
+                make_float4(reduce5(a[2 * k].x, a[2 * k + 1].x, a[2 * k + 2].x, a[2 * k + 3].x, a[2 * k + 4].x),
+                            reduce5(a[2 * k].y, a[2 * k + 1].y, a[2 * k + 2].y, a[2 * k + 3].y, a[2 * k + 4].y),
+                            reduce5(a[2 * k].z, a[2 * k + 1].z, a[2 * k + 2].z, a[2 * k + 3].z, a[2 * k + 4].z),
+                            reduce5(a[2 * k].w, a[2 * k + 1].w, a[2 * k + 2].w, a[2 * k + 3].w, a[2 * k + 4].w));
     }
     __syncthreads();
     const int x = tid & (kPdTW - 1);
@@ -171,11 +241,10 @@ __device__ __forceinline__ void reduce_staged(const float (*s_src)[kPdSW], float
         for (int r = tid / kPdTW; r < kPdTH; r += 256 / kPdTW) {
             const int yd = yd0 + r;
             if (yd >= hd) break;
-            const float* V = &s_v[0][0];
-            const int o = r * (kPdSW + 1) + c, NV = kPdTH * (kPdSW + 1);
-            PANO_AT(dst, (long long)yd * dst_pitch + xd, (long long)hd * dst_pitch, 313) = from_f32<Ts>(
-                reduce5(PANO_AT(V, o - 2, NV, 314), PANO_AT(V, o - 1, NV, 314), PANO_AT(V, o, NV, 314),
-                        PANO_AT(V, o + 1, NV, 314), PANO_AT(V, o + 2, NV, 314)));
+            const int o = r * kPdSW + c;
+            const float2 l = PANO_VEC(const float2, V, o - 2, 2, NV, 314), m = PANO_VEC(const float2, V, o, 2, NV, 314);
+            PANO_AT(dst, (long long)yd * dst_pitch + xd, (long long)hd * dst_pitch, 313) =
+                from_f32<Ts>(reduce5(l.x, l.y, m.x, m.y, PANO_AT(V, o + 2, NV, 314)));
         }
     }
 }
@@ -184,7 +253,7 @@ template <class Ts>
 __global__ void __launch_bounds__(256) pyr_down_kernel(const __grid_constant__ PyrDownArgs a) {
     grid_begin();
     __shared__ __align__(16) float s_src[kPdSH][kPdSW];
-    __shared__ float s_v[kPdTH][kPdSW + 1];
+    __shared__ __align__(16) float s_v[kPdTH][kPdSW];
     const int z = blockIdx.z;
     const Ts* __restrict__ src = static_cast<const Ts*>(a.src[z]);
     Ts* __restrict__ dst = static_cast<Ts*>(a.dst[z]);
@@ -197,25 +266,35 @@ __global__ void __launch_bounds__(256) pyr_down_kernel(const __grid_constant__ P
     const int tid = threadIdx.x;
     // four-element loads need a plane whose rows start on 4-element boundaries
     const bool vec = ((((uintptr_t)src) & (4 * sizeof(Ts) - 1)) == 0) && (src_pitch & 3) == 0;
-    for (int i = tid; i < kPdSH * kPdQ; i += 256) {
+    constexpr int kIts = (kPdSH * kPdQ + 255) / 256;
+    float v[kIts][4];
+#pragma unroll
+    for (int it = 0; it < kIts; ++it) {
+        const int i = min(tid + 256 * it, kPdSH * kPdQ - 1);
         const int r = i / kPdQ, q = i - r * kPdQ;
         const int sy = PANO_IDX(min(max(sy0 + r, 0), h - 1), h, 317);
         const int sx = cx0 + 4 * q;
         const long long ro = (long long)sy * src_pitch;
         const long long ns = (long long)(h - 1) * src_pitch + w;  // elements of the plane
         (void)ns;
-        float* o = &PANO_VEC(float, &s_src[0][0], r * kPdSW + 4 * q, 4, kPdSH * kPdSW, 318);
         if (vec && sx >= 0 && sx + 3 < w) {
             using V = typename Vec4Of<Ts>::type;
-            const V v = PANO_VEC(const V, src, ro + sx, 4, ns, 319);
-            if constexpr (sizeof(Ts) == 4) widen4(v, o);
-            else widen4<Ts>(v, o);
+            const V e = PANO_VEC(const V, src, ro + sx, 4, ns, 319);
+            if constexpr (sizeof(Ts) == 4) widen4(e, v[it]);
+            else widen4<Ts>(e, v[it]);
         } else {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) o[k] = ld_f32(&PANO_AT(src, ro + min(max(sx + k, 0), w - 1), ns, 320));
+            for (int k = 0; k < 4; ++k) v[it][k] = ld_f32(&PANO_AT(src, ro + min(max(sx + k, 0), w - 1), ns, 320));
         }
     }
-    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < kIts; ++it) {
+        const int i = tid + 256 * it;
+        if (i >= kPdSH * kPdQ) break;
+        const int r = i / kPdQ, q = i - r * kPdQ;
+        PANO_VEC(float4, &s_src[0][0], r * kPdSW + 4 * q, 4, kPdSH * kPdSW, 318) =
+            make_float4(v[it][0], v[it][1], v[it][2], v[it][3]);
+    }
     __syncthreads();
     reduce_staged<Ts>(s_src, s_v, xd0, yd0, wd, hd, dst, dst_pitch);
 }
@@ -226,11 +305,11 @@ __global__ void __launch_bounds__(256) pyr_down_kernel(const __grid_constant__ P
 // (rows 2*y0 .. 2*y0+31, columns 2*x0 .. 2*x0+127; the blocks tile level 0
 // exactly) and reduces the footprint to the level-1 tile. Same values as
 // luma_kernel followed by pyr_down_kernel.
-template <class Ts>
+template <class Ts, class K>
 __global__ void __launch_bounds__(256) luma_reduce_kernel(const __grid_constant__ LumaReduceArgs a) {
     grid_begin();
     __shared__ __align__(16) float s_src[kPdSH][kPdSW];
-    __shared__ float s_v[kPdTH][kPdSW + 1];
+    __shared__ __align__(16) float s_v[kPdTH][kPdSW];
     const int z = blockIdx.z;
     const ImageDesc& in = a.in[z];
     const int h = in.h, w = in.w;
@@ -241,33 +320,43 @@ __global__ void __launch_bounds__(256) luma_reduce_kernel(const __grid_constant_
     Ts* __restrict__ l0 = static_cast<Ts*>(a.l0[z]);
     const int p0 = a.l0_pitch[z];
     const int tid = threadIdx.x;
-    for (int i = tid; i < kPdSH * kPdQ; i += 256) {
+    // all loads of a thread first: its stores may alias the image as far as the
+    // compiler knows, and one load at a time leaves the memory waiting
+    constexpr int kIts = (kPdSH * kPdQ + 255) / 256;
+    float v[kIts][4];
+#pragma unroll
+    for (int it = 0; it < kIts; ++it) {
+        const int i = min(tid + 256 * it, kPdSH * kPdQ - 1);
         const int r = i / kPdQ, q = i - r * kPdQ;
-        const int yy = sy0 + r;
-        const int sy = PANO_IDX(min(max(yy, 0), h - 1), h, 321);
+        const int sy = PANO_IDX(min(max(sy0 + r, 0), h - 1), h, 321);
         const int sx = cx0 + 4 * q;
         const unsigned char* row = static_cast<const unsigned char*>(in.data) + (long long)sy * in.pitch_bytes;
-        float v[4];
         if (sx >= 0 && sx + 3 < w) {
-            luma4(in, row, sx, v);
+            luma4<K>(in, row, sx, v[it]);
         } else {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) v[k] = luma_at(in, row, min(max(sx + k, 0), w - 1));
+            for (int k = 0; k < 4; ++k) v[it][k] = luma_at<K>(in, row, min(max(sx + k, 0), w - 1));
         }
+    }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = to_f32(from_f32<Ts>(v[k]));  // the stored level-0 value
-        float* o = &PANO_VEC(float, &s_src[0][0], r * kPdSW + 4 * q, 4, kPdSH * kPdSW, 322);
+    for (int it = 0; it < kIts; ++it) {
+        const int i = tid + 256 * it;
+        if (i >= kPdSH * kPdQ) break;
+        const int r = i / kPdQ, q = i - r * kPdQ;
+        const int yy = sy0 + r, sx = cx0 + 4 * q;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) o[k] = v[k];
+        for (int k = 0; k < 4; ++k) v[it][k] = to_f32(from_f32<Ts>(v[it][k]));  // the stored level-0 value
+        PANO_VEC(float4, &s_src[0][0], r * kPdSW + 4 * q, 4, kPdSH * kPdSW, 322) =
+            make_float4(v[it][0], v[it][1], v[it][2], v[it][3]);
         // level-0 pixels owned by this block
         if (r >= 2 && r < 2 + 2 * kPdTH && yy < h && q >= 1 && q <= kPdTW / 2 && sx < w) {
             const long long ro = (long long)yy * p0;
             const long long n0 = (long long)(h - 1) * p0 + w;  // elements of level 0
             (void)n0;
             if (sx + 3 < w) {
-                store4(&PANO_VEC(Ts, l0, ro + sx, 1, n0 - 3, 323), v);   // elements sx .. sx+3
+                store4(&PANO_VEC(Ts, l0, ro + sx, 1, n0 - 3, 323), v[it]);   // elements sx .. sx+3
             } else {
-                for (int k = 0; k < 4 && sx + k < w; ++k) PANO_AT(l0, ro + sx + k, n0, 324) = from_f32<Ts>(v[k]);
+                for (int k = 0; k < 4 && sx + k < w; ++k) PANO_AT(l0, ro + sx + k, n0, 324) = from_f32<Ts>(v[it][k]);
             }
         }
     }
@@ -445,6 +534,24 @@ cudaError_t pyr_tail_prepare(int max_smem_bytes) {
     return prepare_tail_t<__half>(max_smem_bytes);
 }
 
+// f(storage type, image kind) for the images of one launch, which share their
+// sample type and channels.
+template <class F>
+static cudaError_t with_luma_types(int pyr, const ImageDesc* in, int count, F f) {
+    for (int i = 1; i < count; ++i)
+        if (in[i].dtype != in[0].dtype || in[i].c != in[0].c) return cudaErrorInvalidValue;
+    auto kinds = [&](auto ts) {
+        if (in[0].dtype == 0) return in[0].c == 3 ? f(ts, ImageKind<0, 3>{}) : f(ts, ImageKind<0, 1>{});
+        return in[0].c == 3 ? f(ts, ImageKind<1, 3>{}) : f(ts, ImageKind<1, 1>{});
+    };
+    switch (pyr) {
+        case kPyrF32: return kinds(float{});
+        case kPyrBF16: return kinds(__nv_bfloat16{});
+        case kPyrF16: return kinds(__half{});
+        default: return cudaErrorInvalidValue;
+    }
+}
+
 cudaError_t launch_luma_reduce(const LumaReduceArgs& a, cudaStream_t s) {
     if (a.count < 1 || a.count > kMaxPlanes) return cudaErrorInvalidValue;
     int hd = 0, wd = 0;
@@ -454,12 +561,9 @@ cudaError_t launch_luma_reduce(const LumaReduceArgs& a, cudaStream_t s) {
     }
     dim3 block(256);
     dim3 grid((wd + kPdTW - 1) / kPdTW, (hd + kPdTH - 1) / kPdTH, a.count);
-    switch (a.pyr) {
-        case kPyrF32: return launch_dependent(luma_reduce_kernel<float>, grid, block, 0, s, 0, a);
-        case kPyrBF16: return launch_dependent(luma_reduce_kernel<__nv_bfloat16>, grid, block, 0, s, 0, a);
-        case kPyrF16: return launch_dependent(luma_reduce_kernel<__half>, grid, block, 0, s, 0, a);
-        default: return cudaErrorInvalidValue;
-    }
+    return with_luma_types(a.pyr, a.in, a.count, [&](auto ts, auto kind) {
+        return launch_dependent(luma_reduce_kernel<decltype(ts), decltype(kind)>, grid, block, 0, s, 0, a);
+    });
 }
 
 PANO_BOUNDS_READER(bounds_read_pyramid)
@@ -474,12 +578,9 @@ cudaError_t launch_luma(const LumaArgs& a, cudaStream_t s) {
     // 64 x 4 threads, four pixels each: 256 x 4 pixels per block
     dim3 block(64, 4);
     dim3 grid((w + 4 * 64 - 1) / (4 * 64), (h + 3) / 4, a.count);
-    switch (a.pyr) {
-        case kPyrF32: return launch_dependent(luma_kernel<float>, grid, block, 0, s, 0, a);
-        case kPyrBF16: return launch_dependent(luma_kernel<__nv_bfloat16>, grid, block, 0, s, 0, a);
-        case kPyrF16: return launch_dependent(luma_kernel<__half>, grid, block, 0, s, 0, a);
-        default: return cudaErrorInvalidValue;
-    }
+    return with_luma_types(a.pyr, a.in, a.count, [&](auto ts, auto kind) {
+        return launch_dependent(luma_kernel<decltype(ts), decltype(kind)>, grid, block, 0, s, 0, a);
+    });
 }
 
 cudaError_t launch_pyr_down(const PyrDownArgs& a, cudaStream_t s) {

@@ -95,7 +95,23 @@ def test_fused_luma_and_reduce_equal_the_separate_kernels_and_the_oracle(shape, 
     np.testing.assert_allclose(host(Y1), oracle.pyr_down(Yo), rtol=0, atol=1e-6)
 
 
-@pytest.mark.parametrize("shape,nlev", [((300, 200), 6), ((37, 53), 5), ((1, 1), 4), ((130, 17), 7), ((64, 64), 3),
+@pytest.mark.parametrize("c,dtype", [(1, np.uint8), (3, np.uint8), (1, np.float32), (3, np.float32)])
+@pytest.mark.parametrize("h,w,x0", [(3, 4, 0), (4, 5, 1), (5, 6, 2), (6, 7, 3), (35, 131, 1), (9, 138, 3), (33, 257, 2)])
+def test_luma_of_rows_at_any_alignment(h, w, x0, c, dtype):
+    # crops whose rows start at every byte (float: every element) of a 16-byte word
+    g = rng(34)
+    big = g.integers(0, 256, size=(h, w + 9, c)).astype(np.uint8) if dtype == np.uint8 else \
+        g.uniform(0, 1, size=(h, w + 9, c)).astype(np.float32)
+    view = cuda(big if c == 3 else big[..., 0])[:, x0:x0 + w]
+    img = big[:, x0:x0 + w] if c == 3 else big[:, x0:x0 + w, 0]
+    ref = oracle.luma(oracle.to_unit(img))
+    np.testing.assert_allclose(host(binding.stage_luma(view)), ref, rtol=0, atol=1e-6)
+    Y, Y1 = binding.stage_luma_pyr(view)
+    np.testing.assert_allclose(host(Y), ref, rtol=0, atol=1e-6)
+    np.testing.assert_allclose(host(Y1), oracle.pyr_down(ref), rtol=0, atol=1e-6)
+
+
+@pytest.mark.parametrize("shape,nlev", [((8000, 8016), 5), ((300, 200), 6), ((37, 53), 5), ((1, 1), 4), ((130, 17), 7), ((64, 64), 3),
                                         ((2000, 750), 6)])
 def test_multi_level_reduce_equals_one_level_steps_and_the_oracle(shape, nlev):
     Y = cuda(rng(33).uniform(0, 1, size=shape).astype(np.float32))
