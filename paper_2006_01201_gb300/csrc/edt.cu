@@ -15,8 +15,8 @@
 //   rows:    d2(x, y) = min over columns x' of (x - x')^2 + g(x', y)^2. The
 //            leftmost column that attains the minimum never moves left as x
 //            grows, so the columns of a few pixels bound those of the pixels
-//            between them (edt_near_kernel). Canvases with a side above
-//            kNearMaxSide, whose squared distances leave 32 bits, take the
+//            between them (edt_near_kernel). Canvases with a diagonal above
+//            kNearMaxDiagonal, whose squared distances leave 32 bits, take the
 //            lower envelope of one parabola per column instead
 //            (edt_row.cuh: banded envelopes merged in a tree).
 // Only the final ratio is rounded (FP32 square roots and one division).
@@ -204,43 +204,45 @@ __global__ void __launch_bounds__(kColW * kColTY, 2) edt_cols_kernel(const unsig
 }
 
 // ---------------------------------------------------------------------------
-// Row pass, sides up to kNearMaxSide: one CTA per row, both areas. The row's
+// Row pass, diagonals up to kNearMaxDiagonal: one CTA per row, both areas. The row's
 // columns are cut into groups of 64; only groups with an Area3 pixel matter.
 //   1  g of both areas to shared memory, with the least g of every block of 32
 //      columns; pixels of the other groups are written at once;
 //   2  the nearest column (leftmost of equals) for the first pixel of every
-//      group and the last pixel of the last one, by bisection over the groups:
-//      a warp searches between the columns of the two neighbours already
-//      known. A long range is searched by blocks: the least g bounds every
+//      group and the last pixel of every run of groups, by bisection over
+//      these points: a warp searches between the columns of the two neighbours
+//      already known. A long range is searched by blocks: the least g bounds every
 //      distance to a block from both sides, and only the blocks whose lower
 //      bound does not exceed the least upper bound are looked through;
 //   3  a lane per two pixels: the least distance over the columns between those of
-//      its group and of the next one, and Eq. (1). Where that range is long
-//      (the nearest column jumps from one seam to another), the bisection goes
-//      on over the group's lanes.
-// Distances are 32-bit integers (kNearMaxSide: the bound of step 2 adds 31
-// columns to the largest distance and still stays below 2^32).
-// What bounds it: the instructions of steps 2 and 3 (195 M warp instructions on
-// a 4000 x 9000 canvas, 64% of the issue rate); the g plane is read once.
-// 254 us there, against 457 + 505 us of the envelopes' two launches. Groups of
+//      its group's point and of the next one, and Eq. (1). Where that range is
+//      long (the nearest column jumps from one seam to another), the bisection
+//      goes on over the group's lanes.
+// Distances are 32-bit integers. In shared memory a column without a site has
+// g = kNearNone, the largest diagonal: no pixel is that far from a site, and its
+// square plus that of any distance within the row stays below 2^32.
+// What bounds it: the instructions of steps 2 and 3 (178 M warp instructions on
+// a 4000 x 9000 canvas, 65% of the issue rate); the g plane is read once.
+// 224 us there, against 457 + 505 us of the envelopes' two launches; 254 us
+// with points at first pixels only, whose ranges span the gaps between runs,
+// and with a test for the missing site at every column. Groups of
 // 32: 284 us; steps 2 and 3 alone without the bisection in step 3: a row whose
 // overlaps lie far apart looks through the columns between them, 935 us.
 // ---------------------------------------------------------------------------
 constexpr int kNearThreads = 256;
 constexpr int kNearWarps = kNearThreads / 32;
-constexpr int kNearMaxSide = 46000;
+constexpr int kNearMaxDiagonal = 46340;
+constexpr unsigned kNearNone = kNearMaxDiagonal;
 constexpr int kNearScan = 64;  // columns that a lane looks through one by one
 constexpr int kNearFew = 4;    // a shorter range is left for step 3
 
 struct NearSmem {
     int w4, nb, ng;  // columns rounded up to 4, blocks of 32 columns, groups of 64
     __host__ __device__ explicit NearSmem(int w) : w4((w + 3) / 4 * 4), nb((w + 31) / 32), ng((w + 63) / 64) {}
-    __host__ __device__ size_t bytes() const { return 4 * ((size_t)w4 + nb) + 2 * (4 * ((size_t)ng + 1) + ng); }
+    __host__ __device__ size_t bytes() const { return 4 * ((size_t)w4 + nb) + 2 * 5 * ((size_t)ng + 2); }
 };
 
-__device__ __forceinline__ unsigned near_cost(unsigned g, int dx) {
-    return g == edt::kNoSite ? 0xFFFFFFFFu : (unsigned)(dx * dx) + g * g;
-}
+__device__ __forceinline__ unsigned near_cost(unsigned g, int dx) { return (unsigned)dx * (unsigned)dx + g * g; }
 
 // Leftmost nearest column of pixel x among [lo, hi], by one warp; some column
 // of [lo, hi] is a nearest one of the whole row. gs and bm hold both areas'
@@ -262,13 +264,18 @@ __device__ __forceinline__ int near_search(const uint32_t* gs, const uint32_t* b
     }
     const int b0 = lo >> 5, b1 = hi >> 5;
     unsigned ub = 0xFFFFFFFFu;
-    for (int b = b0 + lane; b <= b1; b += 32)
-        ub = min(ub, near_cost(PANO_AT(bm, b, nb, 517) >> sh & 0xFFFFu, max(abs(x - 32 * b), abs(x - 32 * b - 31))));
+    for (int b = b0 + lane; b <= b1; b += 32) {
+        const unsigned g = PANO_AT(bm, b, nb, 517) >> sh & 0xFFFFu;
+        if (g != kNearNone) ub = min(ub, near_cost(g, max(abs(x - 32 * b), abs(x - 32 * b - 31))));
+    }
     ub = __reduce_min_sync(kAll, ub);
     for (int base = b0; base <= b1; base += 32) {
         const int b = base + lane;
         unsigned lb = 0xFFFFFFFFu;
-        if (b <= b1) lb = near_cost(PANO_AT(bm, b, nb, 518) >> sh & 0xFFFFu, max(0, max(32 * b - x, x - 32 * b - 31)));
+        if (b <= b1) {
+            const unsigned g = PANO_AT(bm, b, nb, 518) >> sh & 0xFFFFu;
+            if (g != kNearNone) lb = near_cost(g, max(0, max(32 * b - x, x - 32 * b - 31)));
+        }
         unsigned todo = __ballot_sync(kAll, lb <= ub && lb != 0xFFFFFFFFu);
         while (todo) {
             const int k = __ffs(todo) - 1;
@@ -278,7 +285,7 @@ __device__ __forceinline__ int near_search(const uint32_t* gs, const uint32_t* b
             const unsigned m = __reduce_min_sync(kAll, c);
             if (m < best) {
                 best = m;
-                bq = (int)__reduce_min_sync(kAll, c == m ? (unsigned)q : 0xFFFFFFFFu);
+                bq = 32 * (base + k) + __ffs(__ballot_sync(kAll, c == m)) - 1;
                 ub = min(ub, m);
             }
             todo &= __ballot_sync(kAll, lb <= ub && lb != 0xFFFFFFFFu) & ~((2u << k) - 1u);
@@ -298,9 +305,10 @@ __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const unsigned c
     const int w4 = L.w4, nb = L.nb, ng = L.ng;
     uint32_t* gs = reinterpret_cast<uint32_t*>(s_dyn);      // [w4] g of both areas
     uint32_t* bm = gs + w4;                                  // [nb] least g of a block, both areas
-    uint16_t* ql = reinterpret_cast<uint16_t*>(bm + nb);     // [2][ng + 1] the nearest column of point i lies
-    uint16_t* qh = ql + 2 * (ng + 1);                        // [2][ng + 1] between these two
-    uint16_t* list = qh + 2 * (ng + 1);                      // [ng] groups with an Area3 pixel
+    uint16_t* ql = reinterpret_cast<uint16_t*>(bm + nb);     // [2][ng + 2] the nearest column of point i lies
+    uint16_t* qh = ql + 2 * (ng + 2);                        // [2][ng + 2] between these two
+    uint16_t* list = qh + 2 * (ng + 2);                      // [ng + 2] points: 2 group (+ 1 for a run's last pixel)
+    uint16_t* flag = qh;                                     // [ng + 1] group with an Area3 pixel, before step 2
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, y = blockIdx.x;
     constexpr unsigned kAll = 0xffffffffu;
     const unsigned char* lab = label + (long long)y * pitch;
@@ -312,7 +320,7 @@ __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const unsigned c
     {
         const uint32_t* row = gb + (long long)y * gp;
         const bool vec = (((uintptr_t)row) & 15) == 0;
-        unsigned all = kAll;
+        unsigned all = kNearNone | kNearNone << 16;
         for (int v0 = 0; v0 < w4 / 4; v0 += kNearThreads) {
             const int v = v0 + tid;
             uint4 k = make_uint4(kAll, kAll, kAll, kAll);
@@ -325,17 +333,20 @@ __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const unsigned c
                     for (int i = 0; i < 4; ++i) e[i] = 4 * v + i < w ? PANO_AT(row, 4 * v + i, w, 506) : kAll;
                     k = make_uint4(e[0], e[1], e[2], e[3]);
                 }
+                const unsigned none = kNearNone | kNearNone << 16;
+                k = make_uint4(__vminu2(k.x, none), __vminu2(k.y, none), __vminu2(k.z, none), __vminu2(k.w, none));
                 PANO_VEC(uint4, gs, 4 * v, 4, w4, 507) = k;
             }
             unsigned m = __vminu2(__vminu2(k.x, k.y), __vminu2(k.z, k.w));
             m = __vminu2(m, __shfl_xor_sync(kAll, m, 1));
             m = __vminu2(m, __shfl_xor_sync(kAll, m, 2));
             m = __vminu2(m, __shfl_xor_sync(kAll, m, 4));
+            m = __vminu2(m, kNearNone | kNearNone << 16);
             if (v < w4 / 4 && (v & 7) == 0) PANO_AT(bm, v / 8, nb, 508) = m;
             all = __vminu2(all, m);
         }
-        if ((all & 0xFFFFu) != edt::kNoSite) s_any[0] = 1;
-        if (all >> 16 != edt::kNoSite) s_any[1] = 1;
+        if ((all & 0xFFFFu) != kNearNone) s_any[0] = 1;
+        if (all >> 16 != kNearNone) s_any[1] = 1;
     }
     // groups without an Area3 pixel are written now; the others are listed
     const bool lvec = (((uintptr_t)lab) & 3) == 0, ovec = (((uintptr_t)out) & 15) == 0;
@@ -352,7 +363,7 @@ __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const unsigned c
         }
         const unsigned three = __ballot_sync(kAll, __vcmpeq4(c, 0x03030303u) != 0u);
         const bool act = (lane < 16 ? three & 0xFFFFu : three >> 16) != 0u;
-        if ((lane & 15) == 0 && x < w) PANO_AT(list, x / 64, ng, 510) = act;
+        if ((lane & 15) == 0 && x < w) PANO_AT(flag, x / 64, ng + 1, 510) = act;
         if (act || x >= w) continue;
         float b[4];
 #pragma unroll
@@ -366,30 +377,34 @@ __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const unsigned c
             for (int i = 0; i < 4 && x + i < w; ++i) PANO_AT(out, x + i, w, 511) = b[i];
         }
     }
+    if (tid == 0) flag[ng] = 0;
     __syncthreads();
     if (wid == 0) {
+        // the points: the first pixel of every such group, the last one of every
+        // run of neighbouring groups
         int n = 0;
         for (int g0 = 0; g0 < ng; g0 += 32) {
-            const bool act = g0 + lane < ng && list[g0 + lane];
-            const unsigned m = __ballot_sync(kAll, act);
-            __syncwarp();
-            // written at or before the entries read so far
-            if (act) PANO_AT(list, n + __popc(m & ((1u << lane) - 1u)), ng, 512) = (uint16_t)(g0 + lane);
-            n += __popc(m);
+            const int g = g0 + lane;
+            const bool act = g < ng && PANO_AT(flag, g, ng + 1, 512), end = act && !PANO_AT(flag, g + 1, ng + 1, 512);
+            const unsigned ma = __ballot_sync(kAll, act), me = __ballot_sync(kAll, end), lt = (1u << lane) - 1u;
+            const int o = n + __popc(ma & lt) + __popc(me & lt);
+            if (act) PANO_AT(list, o, ng + 2, 512) = (uint16_t)(2 * g);
+            if (end) PANO_AT(list, o + 1, ng + 2, 512) = (uint16_t)(2 * g + 1);
+            n += __popc(ma) + __popc(me);
         }
         if (lane == 0) s_n = n;
     }
     __syncthreads();
-    const int n = s_n;
-    if (n == 0) return;
+    if (s_n == 0) return;
+    const int n = s_n - 1;  // the last point
     const bool any0 = s_any[0] != 0, any1 = s_any[1] != 0;
 
     // ---- 2: nearest columns of points 0 .. n
-    auto point_x = [&](int i) { return i < n ? 64 * (int)list[i] : min(w - 1, 64 * (int)list[n - 1] + 63); };
+    auto point_x = [&](int i) { return list[i] & 1 ? min(w - 1, 32 * (int)list[i] + 31) : 32 * (int)list[i]; };
     if (wid < 4) {
         const int a = wid & 1, i = wid < 2 ? 0 : n;
         const int q = (a ? any1 : any0) ? near_search(gs, bm, 16 * a, w, nb, point_x(i), 0, w - 1) : 0;
-        if (lane == 0) PANO_AT(ql, a * (ng + 1) + i, 2 * (ng + 1), 513) = PANO_AT(qh, a * (ng + 1) + i, 2 * (ng + 1), 513) = (uint16_t)q;
+        if (lane == 0) PANO_AT(ql, a * (ng + 2) + i, 2 * (ng + 2), 513) = PANO_AT(qh, a * (ng + 2) + i, 2 * (ng + 2), 513) = (uint16_t)q;
     }
     __syncthreads();
     int s = 1;
@@ -399,11 +414,11 @@ __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const unsigned c
         // a lane per point and area; the warp searches the long ranges together
         for (int t0 = 0; t0 < 2 * cnt; t0 += kNearThreads) {
             const int t = t0 + wid + kNearWarps * lane;
-            const int a = t & 1, i = s * (2 * (t >> 1) + 1), o = a * (ng + 1);
+            const int a = t & 1, i = s * (2 * (t >> 1) + 1), o = a * (ng + 2);
             int lo = 0, hi = 0;
             if (t < 2 * cnt) {
-                lo = PANO_AT(ql, o + i - s, 2 * (ng + 1), 514);
-                hi = PANO_AT(qh, o + min(i + s, n), 2 * (ng + 1), 515);
+                lo = PANO_AT(ql, o + i - s, 2 * (ng + 2), 514);
+                hi = PANO_AT(qh, o + min(i + s, n), 2 * (ng + 2), 515);
             }
             for (unsigned todo = __ballot_sync(kAll, hi - lo > kNearFew); todo; todo &= todo - 1) {
                 const int k = __ffs(todo) - 1;
@@ -418,18 +433,18 @@ __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const unsigned c
 
     // ---- 3: distances and Eq. (1)
     for (int i = wid; i < n; i += kNearWarps) {
-        const int X = 64 * (int)list[i], x = X + 2 * lane;
+        if (list[i] & 1) continue;
+        const int X = 32 * (int)list[i], x = X + 2 * lane;
         const unsigned c0 = x < w ? PANO_AT(lab, x, w, 545) : 0, c1 = x + 1 < w ? PANO_AT(lab, x + 1, w, 545) : 0;
         unsigned d0[2], d1[2];
 #pragma unroll
         for (int a = 0; a < 2; ++a) {
             unsigned b0 = 0xFFFFFFFFu, b1 = 0xFFFFFFFFu;
             if (a ? any1 : any0) {
-                int lo = ql[a * (ng + 1) + i], hi = qh[a * (ng + 1) + i + 1];
+                int lo = ql[a * (ng + 2) + i], hi = qh[a * (ng + 2) + i + 1];
                 if (hi - lo > kNearScan) {
-                    // the nearest column jumps in this group, or before the next
-                    // one: bisect on, over the lanes, where the range is long
-                    hi = near_search(gs, bm, 16 * a, w, nb, min(X + 63, w - 1), lo, hi);
+                    // the nearest column jumps in this group: bisect on, over the
+                    // lanes, where the range is long
                     for (int st = 16; st >= 1; st >>= 1)
                         for (int b = 0; b < 32; b += 2 * st) {
                             const int l = __shfl_sync(kAll, lo, b), u = __shfl_sync(kAll, hi, b), xm = X + 2 * (b + st);
@@ -439,11 +454,13 @@ __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const unsigned c
                             if (lane >= b + st && lane < b + 2 * st) lo = m;
                         }
                 }
-#pragma unroll 1
+                const uint16_t* ga = reinterpret_cast<const uint16_t*>(gs) + a;
+#pragma unroll 2
                 for (int q = lo; q <= hi; ++q) {
-                    const unsigned g = PANO_AT(gs, q, w, 546) >> (16 * a) & 0xFFFFu;
-                    b0 = min(b0, near_cost(g, x - q));
-                    b1 = min(b1, near_cost(g, x + 1 - q));
+                    const unsigned g = PANO_AT(ga, 2 * q, 2 * w - a, 546), g2 = g * g;
+                    const unsigned dx = (unsigned)(x - q);
+                    b0 = min(b0, g2 + dx * dx);
+                    b1 = min(b1, g2 + (dx + 1) * (dx + 1));
                 }
             }
             d0[a] = b0, d1[a] = b1;
@@ -681,7 +698,7 @@ size_t blend_coeff_row_smem(int w) { return (size_t)4 * w + (size_t)(5 * kRowThr
 
 cudaError_t blend_coeff_prepare(int max_smem_bytes) {
     cudaError_t e = cudaFuncSetAttribute(edt_near_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)NearSmem(kNearMaxSide).bytes());
+                                         (int)NearSmem(kNearMaxDiagonal).bytes());
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(edt_cols_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ColSmem));
     if (e != cudaSuccess) return e;
@@ -694,7 +711,7 @@ cudaError_t blend_coeff_prepare(int max_smem_bytes) {
 
 cudaError_t launch_blend_coeff(const unsigned char* label, int h, int w, long long pitch, float* blend,
                                int blend_pitch, void* scratch, cudaStream_t s) {
-    const bool near = h <= kNearMaxSide && w <= kNearMaxSide;
+    const bool near = (long long)h * h + (long long)w * w <= (long long)kNearMaxDiagonal * kNearMaxDiagonal;
     const dim3 grid((w + kColW - 1) / kColW), block(kColW, kColTY);
     cudaError_t e;
     if (near) {

@@ -175,7 +175,7 @@ def test_bad_arguments_raise():
 
 
 # The row pass works on groups of 32 columns (loads of 8) and bisects over the
-# groups with Area3; sides above 46000 take the other row pass. Sizes on either
+# groups with Area3; diagonals above 46340 take the other row pass. Sizes on either
 # side of each, areas that miss from whole columns, and one-group rows.
 @pytest.mark.parametrize("shape,p", [((9, 31), 0.5), ((9, 32), 0.5), ((9, 33), 0.5), ((7, 64), 0.02), ((7, 65), 0.02),
                                      ((5, 255), 0.01), ((5, 257), 0.003), ((3, 1025), 0.002), ((40, 700), 0.0004),
@@ -187,7 +187,8 @@ def test_sparse_areas_around_the_group_sizes(shape, p):
     np.testing.assert_allclose(gpu_blend(label), oracle.blend_coeff(label), rtol=0, atol=TOL)
 
 
-@pytest.mark.parametrize("shape", [(3, 46000), (3, 46001), (46000, 3), (46001, 3)])
+@pytest.mark.parametrize("shape", [(3, 46000), (3, 46001), (46000, 3), (46001, 3), (3, 46339), (3, 46341),
+                                   (46339, 3), (46341, 3)])
 def test_sides_around_the_32_bit_distances(shape):
     # few sites, so that distances near the largest ones occur
     label = np.full(shape, 3, dtype=np.uint8)
