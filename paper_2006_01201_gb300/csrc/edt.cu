@@ -24,6 +24,7 @@
 #include <string.h>
 
 #include <climits>
+#include <type_traits>
 
 #include "bounds.cuh"
 #include "common.cuh"
@@ -43,17 +44,27 @@ namespace {
 // suffix minimum gives the first feature row at or after each block. The
 // second pass finds the nearest features above and below the thread's rows
 // from the masks of the other threads of its block (shared memory), the last
-// feature row of the blocks above and the first of the blocks below, and walks
-// its rows down and up with the last feature row seen. The masks of the first
-// kKeptBlocks blocks stay in shared memory between the two passes, so canvases
-// of up to 4096 rows are read once.
+// feature row of the blocks above and the first of the blocks below, and counts
+// the distance from row to row, down and up, both areas in the halves of a word.
+// Where a warp's 32 columns can be read as aligned words, a lane reads eight
+// rows of four columns, and the masks are put together by shuffles. The masks
+// of the first kKeptBlocks blocks stay in shared memory between the two passes,
+// so canvases of up to 4096 rows are read once.
 // kPacked: g of both areas in one 32-bit element (Area1 low, Area2 high), one
 // coalesced 4-byte store a pixel; otherwise a plane of 16-bit values each.
-// 99 us on a 4000 x 9000 canvas (0.18 GB: 27 us at the memory's rate), bound by
-// instructions (67 M); labels read twice, distances from shifted masks and two
-// 16-bit stores a pixel took 131 us (102 M).
-// edt::kNoSite where the column has no feature pixel. gp: elements per row.
+// 78 us on a 4000 x 9000 canvas (0.18 GB: 27 us at the memory's rate): 17 us
+// without reads and distances, 14 for the reads, 20 for the distances and 26
+// for the stores, one after the other in all CTAs. With a byte per load and a
+// row number per area and pixel instead 99 us (67 M warp instructions, now
+// 36 M). Without the barriers between the blocks of the second pass 82 us.
+// kNearNone (packed) or edt::kNoSite where the column has no feature pixel. gp:
+// elements per row.
 // ---------------------------------------------------------------------------
+// The row pass's 32-bit distances: the largest diagonal, and the g of a column
+// without a site there.
+constexpr int kNearMaxDiagonal = 46340;
+constexpr unsigned kNearNone = kNearMaxDiagonal;
+
 constexpr int kColW = 32;                     // columns per CTA
 constexpr int kColTY = 16;                    // threads along y, 32 rows each
 constexpr int kColBlock = 32 * kColTY;        // rows per block
@@ -69,17 +80,46 @@ struct ColSmem {
     uint32_t some[kKeptBlocks][2][kColW];     // bit k: thread row k of the block has a feature pixel
 };
 
-__device__ __forceinline__ void col_masks(const unsigned char* label, long long pitch, long long nl,
-                                          int h, int x, int y0, uint32_t* m1, uint32_t* m2) {
+// Bit 7 of every byte of c that equals k, shifted in from above: after eight
+// rows a byte holds their bits in order.
+__device__ __forceinline__ uint32_t shift_in_equal(uint32_t acc, uint32_t c, uint32_t k) {
+    const uint32_t v = c ^ k * 0x01010101u, z = ~(((v & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | v) & 0x80808080u;
+    return (acc >> 1 & 0x7F7F7F7Fu) | z;
+}
+
+// Masks of rows y0 .. y0 + 31 (< h) of column x, by a whole warp on columns
+// x - lane .. x - lane + 31. words: these are all in the canvas and 4-byte
+// aligned on every row; a lane then reads eight rows of four columns.
+__device__ __forceinline__ void col_masks(const unsigned char* label, long long pitch, long long nl, int h, int w, int x,
+                                          int y0, bool words, uint32_t* m1, uint32_t* m2) {
+    const int n = min(32, h - y0), lane = threadIdx.x;
     uint32_t a = 0, b = 0;
-    const int n = min(32, h - y0);
-    const unsigned char* p = label + (long long)y0 * pitch + x;
+    if (words) {
+        const int yq = 8 * (lane >> 3);
+        const long long o = (long long)(y0 + yq) * pitch + (x - lane) + 4 * (lane & 7);
+        uint32_t qa = 0, qb = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t c = yq + i < n ? PANO_VEC(const uint32_t, label, o + i * pitch, 4, nl, 500) : 0u;
+            qa = shift_in_equal(qa, c, 1);
+            qb = shift_in_equal(qb, c, 2);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t va = __shfl_sync(0xffffffffu, qa, 8 * q + (lane >> 2));
+            const uint32_t vb = __shfl_sync(0xffffffffu, qb, 8 * q + (lane >> 2));
+            a |= (va >> 8 * (lane & 3) & 0xFFu) << 8 * q;
+            b |= (vb >> 8 * (lane & 3) & 0xFFu) << 8 * q;
+        }
+    } else if (x < w) {
+        const unsigned char* p = label + (long long)y0 * pitch + x;
 #pragma unroll 8
-    for (int i = 0; i < 32; ++i) {
-        if (i < n) {
-            const unsigned char c = PANO_AT(p, (long long)i * pitch, nl - ((long long)y0 * pitch + x), 501);
-            a |= (uint32_t)(c == 1) << i;
-            b |= (uint32_t)(c == 2) << i;
+        for (int i = 0; i < 32; ++i) {
+            if (i < n) {
+                const unsigned char c = PANO_AT(p, (long long)i * pitch, nl - ((long long)y0 * pitch + x), 501);
+                a |= (uint32_t)(c == 1) << i;
+                b |= (uint32_t)(c == 2) << i;
+            }
         }
     }
     *m1 = a;
@@ -97,6 +137,7 @@ __global__ void __launch_bounds__(kColW * kColTY, 2) edt_cols_kernel(const unsig
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kColW + tx;
     const int x = blockIdx.x * kColW + tx;
     const bool col_in = x < w;
+    const bool words = (((uintptr_t)label | (uintptr_t)pitch) & 3) == 0 && (blockIdx.x + 1) * kColW <= w;
     const int nblk = (h + kColBlock - 1) / kColBlock;
     const long long nl = (long long)(h - 1) * pitch + w, ng = (long long)h * gp;  // label and g elements
     (void)nl;
@@ -109,7 +150,7 @@ __global__ void __launch_bounds__(kColW * kColTY, 2) edt_cols_kernel(const unsig
     for (int rb = 0; rb < nblk; ++rb) {
         const int y0 = rb * kColBlock + ty * 32;
         uint32_t m1 = 0, m2 = 0;
-        if (col_in && y0 < h) col_masks(label, pitch, nl, h, x, y0, &m1, &m2);
+        if (y0 < h) col_masks(label, pitch, nl, h, w, x, y0, words, &m1, &m2);
         if (m1) atomicMin(&S.next[0][rb][tx], y0 + __ffs(m1) - 1);
         if (m2) atomicMin(&S.next[1][rb][tx], y0 + __ffs(m2) - 1);
         if (rb < kKeptBlocks) {
@@ -130,7 +171,7 @@ __global__ void __launch_bounds__(kColW * kColTY, 2) edt_cols_kernel(const unsig
             m[0] = S.mask[slot][0][ty][tx];
             m[1] = S.mask[slot][1][ty][tx];
         } else {
-            if (col_in && y0 < h) col_masks(label, pitch, nl, h, x, y0, &m[0], &m[1]);
+            if (y0 < h) col_masks(label, pitch, nl, h, w, x, y0, words, &m[0], &m[1]);
             if (tid < 2 * kColW) (&S.some[slot][0][0])[tid] = 0;
             S.mask[slot][0][ty][tx] = m[0];
             S.mask[slot][1][ty][tx] = m[1];
@@ -156,42 +197,55 @@ __global__ void __launch_bounds__(kColW * kColTY, 2) edt_cols_kernel(const unsig
             below[a] = n;
         }
         if (col_in && y0 < h) {
+            // Distances of both areas in the halves of a word, counted up from row
+            // to row: nothing leaves 16 bits, kCap + 1 included.
+            constexpr uint32_t kCap = kPacked ? kNearNone : edt::kNoSite - 1, kCap2 = kCap | kCap << 16;
+            auto both = [](unsigned d1, unsigned d2) { return min(d1, kCap) | min(d2, kCap) << 16; };
+            // a distance of 65534 is that of the last row of the highest canvas
+            // from the first, so the columns without a site are set apart
+            uint32_t none = 0;
+            if (!kPacked) {
+                if (!m[0] && above[0] == kAboveNone && below[0] == kBelowNone) none |= 0xFFFFu;
+                if (!m[1] && above[1] == kAboveNone && below[1] == kBelowNone) none |= 0xFFFF0000u;
+            }
+            auto at = [](uint32_t bits, int i) { return (bits >> i & 0x00010001u) * 0xFFFFu; };  // 0xFFFF where a site lies
             const int n = min(32, h - y0);
-            const unsigned kNone = edt::kNoSite;
 #pragma unroll 1
-            for (int i0 = 0; i0 < 32; i0 += 16) {
+            for (int i0 = 0; i0 < n; i0 += 16) {
                 // 16 rows at a time (their distances upwards stay in registers)
                 const uint32_t before[2] = {m[0] & ((1u << i0) - 1u), m[1] & ((1u << i0) - 1u)};
                 const uint32_t after[2] = {i0 ? 0u : m[0] & 0xFFFF0000u, i0 ? 0u : m[1] & 0xFFFF0000u};
-                uint32_t d[16];  // both areas in 16 bits each
-                int p1 = before[0] ? y0 + 31 - __clz(before[0]) : above[0], p2 = before[1] ? y0 + 31 - __clz(before[1]) : above[1];
-                const uint32_t k1 = m[0] >> i0, k2 = m[1] >> i0;
+                const uint32_t bits = (m[0] >> i0 & 0xFFFFu) | m[1] >> i0 << 16;
+                const int ya = y0 + i0 - 1, yb1 = y0 + i0 + 16;  // the rows before and after
+                const int p1 = before[0] ? y0 + 31 - __clz(before[0]) : above[0], p2 = before[1] ? y0 + 31 - __clz(before[1]) : above[1];
+                const int q1 = after[0] ? y0 + __ffs(after[0]) - 1 : below[0], q2 = after[1] ? y0 + __ffs(after[1]) - 1 : below[1];
+                uint32_t d[16];  // distance to the last site above
+                uint32_t v = both((unsigned)(ya - p1), (unsigned)(ya - p2));
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
-                    const int yy = y0 + i0 + i;
-                    if (k1 >> i & 1) p1 = yy;
-                    if (k2 >> i & 1) p2 = yy;
-                    d[i] = min((unsigned)(yy - p1), kNone) | min((unsigned)(yy - p2), kNone) << 16;
+                    v = __viaddmin_u16x2(v, 0x00010001u, kCap2) & ~at(bits, i);
+                    d[i] = v;
                 }
-                p1 = after[0] ? y0 + __ffs(after[0]) - 1 : below[0];
-                p2 = after[1] ? y0 + __ffs(after[1]) - 1 : below[1];
+                // the sums stay below 2^31 with kBelowNone too
+                v = both((unsigned)(q1 - yb1), (unsigned)(q2 - yb1));
+                const long long o = (long long)(y0 + i0) * gp + x;
+                auto up = [&](auto whole) {
 #pragma unroll
-                for (int i = 15; i >= 0; --i) {
-                    const int yy = y0 + i0 + i;
-                    if (k1 >> i & 1) p1 = yy;
-                    if (k2 >> i & 1) p2 = yy;
-                    // ints: rows < 2^16, the no-feature values keep both differences below 2^31
-                    const uint32_t v = __vminu2(d[i], min((unsigned)(p1 - yy), kNone) | min((unsigned)(p2 - yy), kNone) << 16);
-                    if (i0 + i < n) {
-                        const long long o = (long long)yy * gp + x;
-                        if constexpr (kPacked) {
-                            PANO_AT(gb, o, ng, 504) = v;
-                        } else {
-                            PANO_AT(g1, o, ng, 504) = (uint16_t)(v & 0xFFFFu);
-                            PANO_AT(g2, o, ng, 504) = (uint16_t)(v >> 16);
+                    for (int i = 15; i >= 0; --i) {
+                        v = __viaddmin_u16x2(v, 0x00010001u, kCap2) & ~at(bits, i);
+                        const uint32_t g = __vminu2(d[i], v) | none;
+                        if (decltype(whole)::value || i0 + i < n) {
+                            if constexpr (kPacked) {
+                                PANO_AT(gb, o + i * gp, ng, 504) = g;
+                            } else {
+                                PANO_AT(g1, o + i * gp, ng, 504) = (uint16_t)(g & 0xFFFFu);
+                                PANO_AT(g2, o + i * gp, ng, 504) = (uint16_t)(g >> 16);
+                            }
                         }
                     }
-                }
+                };
+                if (i0 + 16 <= n) up(std::true_type{});
+                else up(std::false_type{});
             }
         }
         __syncthreads();  // the masks and S.above are read
@@ -231,8 +285,6 @@ __global__ void __launch_bounds__(kColW * kColTY, 2) edt_cols_kernel(const unsig
 // ---------------------------------------------------------------------------
 constexpr int kNearThreads = 256;
 constexpr int kNearWarps = kNearThreads / 32;
-constexpr int kNearMaxDiagonal = 46340;
-constexpr unsigned kNearNone = kNearMaxDiagonal;
 constexpr int kNearScan = 64;  // columns that a lane looks through one by one
 constexpr int kNearFew = 4;    // a shorter range is left for step 3
 
@@ -320,28 +372,26 @@ __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const unsigned c
     {
         const uint32_t* row = gb + (long long)y * gp;
         const bool vec = (((uintptr_t)row) & 15) == 0;
-        unsigned all = kNearNone | kNearNone << 16;
+        constexpr unsigned kNone2 = kNearNone | kNearNone << 16;
+        unsigned all = kNone2;
         for (int v0 = 0; v0 < w4 / 4; v0 += kNearThreads) {
             const int v = v0 + tid;
-            uint4 k = make_uint4(kAll, kAll, kAll, kAll);
+            uint4 k = make_uint4(kNone2, kNone2, kNone2, kNone2);
             if (v < w4 / 4) {
                 if (vec && 4 * v + 4 <= w) {
                     k = PANO_VEC(const uint4, row, 4 * v, 4, w, 505);
                 } else {
                     uint32_t e[4];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) e[i] = 4 * v + i < w ? PANO_AT(row, 4 * v + i, w, 506) : kAll;
+                    for (int i = 0; i < 4; ++i) e[i] = 4 * v + i < w ? PANO_AT(row, 4 * v + i, w, 506) : kNone2;
                     k = make_uint4(e[0], e[1], e[2], e[3]);
                 }
-                const unsigned none = kNearNone | kNearNone << 16;
-                k = make_uint4(__vminu2(k.x, none), __vminu2(k.y, none), __vminu2(k.z, none), __vminu2(k.w, none));
                 PANO_VEC(uint4, gs, 4 * v, 4, w4, 507) = k;
             }
             unsigned m = __vminu2(__vminu2(k.x, k.y), __vminu2(k.z, k.w));
             m = __vminu2(m, __shfl_xor_sync(kAll, m, 1));
             m = __vminu2(m, __shfl_xor_sync(kAll, m, 2));
             m = __vminu2(m, __shfl_xor_sync(kAll, m, 4));
-            m = __vminu2(m, kNearNone | kNearNone << 16);
             if (v < w4 / 4 && (v & 7) == 0) PANO_AT(bm, v / 8, nb, 508) = m;
             all = __vminu2(all, m);
         }

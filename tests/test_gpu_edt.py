@@ -187,8 +187,20 @@ def test_sparse_areas_around_the_group_sizes(shape, p):
     np.testing.assert_allclose(gpu_blend(label), oracle.blend_coeff(label), rtol=0, atol=TOL)
 
 
+# The column pass reads aligned words where 32 columns fill a warp, eight rows a
+# lane, and keeps the masks of 4096 rows. Label values that differ from 1 and 2
+# in one bit only, or by a carry, belong to no area.
+@pytest.mark.parametrize("shape", [(7, 32), (8, 32), (33, 36), (31, 64), (17, 68), (4097, 32), (4129, 40)])
+def test_label_words(shape):
+    g = np.random.default_rng(shape[0])
+    label = g.choice(np.array([1, 2, 3, 0, 129, 130, 255, 5, 6], np.uint8), p=[.01, .01, .8, .03, .03, .03, .03, .03, .03],
+                     size=shape)
+    label[0, 0], label[-1, -1] = 1, 2
+    np.testing.assert_allclose(gpu_blend(label), oracle.blend_coeff(label), rtol=0, atol=TOL)
+
+
 @pytest.mark.parametrize("shape", [(3, 46000), (3, 46001), (46000, 3), (46001, 3), (3, 46339), (3, 46341),
-                                   (46339, 3), (46341, 3)])
+                                   (46339, 3), (46341, 3), (65535, 3)])
 def test_sides_around_the_32_bit_distances(shape):
     # few sites, so that distances near the largest ones occur
     label = np.full(shape, 3, dtype=np.uint8)
