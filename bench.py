@@ -39,7 +39,7 @@ WORKLOAD = {"workload": "pair_4000x1500_rgb_u8_lv6", "h": 4000, "w": 1500, "chan
 SMALL_WORKLOAD = {"workload": "pair_256x512_gray_f32_lv4", "h": 256, "w": 512, "channels": 1, "levels": 4,
                   "iters": 5, "radius": 2}
 L2_FLUSH_BYTES = 256 << 20   # > 129 MB L2
-STREAM_MIN_PIXELS = 50000    # levels with at least this many pixels use the streamed LK kernel
+STREAM_MIN_PIXELS = 50000    # rig_level_kernels' default: pairs of at least this many pixels are streamed
 SMALL_TILE_PIXELS = 16000    # tiled levels below this many pixels use 16 x 8 tiles
 # ncu counters of the dominant kernels (DRAM bytes and warp instructions per
 # launch), written by `--ingest-ncu` from a capture into profiles/ together
@@ -847,9 +847,9 @@ def run_blend_coeff(args):
                        "area3_fraction": float((lab == 3).mean())},
             "roofline": {"bound": "hbm", "achieved": alg / (ms * 1e-3) / 1e9, "peak": peak, "unit": "GB/s",
                          "frac": alg / (ms * 1e-3) / 1e9 / peak, "traffic": None,
-                         "kernel": "edt_cols_kernel + edt_row_kernel (Area1) + edt_row_kernel (Area2)", "alg_bytes_per_launch": alg,
+                         "kernel": "edt_cols_kernel + edt_near_kernel", "alg_bytes_per_launch": alg,
                          "peak_source": f"{src} hbm_gbs"},
-            "gpu_launches": 3 * args.steps, "clocks": clocks}
+            "gpu_launches": 2 * args.steps, "clocks": clocks}
     print(json.dumps(line), flush=True)
     return 0
 
