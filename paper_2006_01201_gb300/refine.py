@@ -59,19 +59,21 @@ class PyramidEnergy(torch.autograd.Function):
         T0, J0, u = ctx.saved_tensors
         need_T, need_J, need_u = ctx.needs_input_grad[:3]
         if T0.shape == J0.shape:   # the whole step in one call
-            du, dT, dJ = binding.refine_grad(T0, J0, u, ctx.level, ctx.alpha, gE, want_u=need_u, want_T=need_T,
+            du, dT, dJ = binding.refine_grad(T0, J0, u, ctx.level, ctx.alpha, want_u=need_u, want_T=need_T,
                                              want_J=need_J)
-            return dT, dJ, du, None, None
-        Tl = _levels(T0, ctx.level)          # rebuilt, not stored
-        Jl = _levels(J0, ctx.level)
-        shapes = [tuple(t.shape) for t in Tl]
-        _, gu, gt, gj = binding.energy_grad(Tl[-1].contiguous(), Jl[-1].contiguous(), u.contiguous(), ctx.alpha,
-                                            want_energy=False, want_u=need_u, want_T=need_T, want_J=need_J)
+        else:
+            Tl = _levels(T0, ctx.level)          # rebuilt, not stored
+            Jl = _levels(J0, ctx.level)
+            shapes = [tuple(t.shape) for t in Tl]
+            _, du, dT, dJ = binding.energy_grad(Tl[-1].contiguous(), Jl[-1].contiguous(), u.contiguous(), ctx.alpha,
+                                                want_energy=False, want_u=need_u, want_T=need_T, want_J=need_J)
+            dT = _reduce_transpose(dT, shapes) if need_T else None
+            dJ = _reduce_transpose(dJ, shapes) if need_J else None
+        # Scaled by tensor operations, not by the library: the gradients stay
+        # differentiable in gE (double backward, functional.jvp), and gE may be
+        # a batch (is_grads_batched), which has no pointer.
         s = gE.to(torch.float32)
-        dT = _reduce_transpose(gt, shapes) * s if need_T else None
-        dJ = _reduce_transpose(gj, shapes) * s if need_J else None
-        du = gu * s if need_u else None
-        return dT, dJ, du, None, None
+        return tuple(g * s if g is not None else None for g in (dT, dJ, du)) + (None, None)
 
 
 def pyramid_energy(T0, J0, u, level: int = 0, alpha: float = 0.05):

@@ -1,0 +1,54 @@
+"""The autograd function of the refinement on the host: what it does with the
+library's results, with stand-ins on CPU tensors for the calls that need a GPU."""
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2006_01201_gb300 import binding, refine  # noqa: E402
+
+
+@pytest.fixture
+def quadratic(monkeypatch):
+    """E(u) = sum u^2 (T0 and J0 do not matter) through the one-call entry
+    points, which fill plain buffers and read `scale` through its pointer."""
+
+    def energy(T0, J0, u, level, alpha):
+        return (u.detach().double() ** 2).sum()
+
+    def grad(T0, J0, u, level, alpha, scale=None, want_u=True, want_T=True, want_J=True):
+        f = 1.0
+        if scale is not None:
+            scale.data_ptr()
+            f = float(scale.detach())
+        zero = torch.zeros_like(T0)
+        return ((2 * f * u).detach() if want_u else None, zero if want_T else None, zero if want_J else None)
+
+    monkeypatch.setattr(binding, "refine_energy", energy)
+    monkeypatch.setattr(binding, "refine_grad", grad)
+    g = torch.Generator().manual_seed(3)
+    T, J = torch.rand((5, 7), generator=g), torch.rand((5, 7), generator=g)
+    return T, J, torch.randn((5, 7, 2), generator=g)
+
+
+def test_gradients_stay_differentiable_in_the_incoming_one(quadratic):
+    T, J, u = quadratic
+    v = torch.randn(u.shape, generator=torch.Generator().manual_seed(4))
+    # jvp differentiates the gradient by the incoming one
+    _, d = torch.autograd.functional.jvp(lambda x: refine.pyramid_energy(T, J, x), u, v)
+    assert float(d) == pytest.approx(float((2 * u * v).double().sum()), rel=1e-5)
+    x = u.clone().requires_grad_(True)
+    g = torch.ones((), dtype=torch.float64, requires_grad=True)
+    (du,) = torch.autograd.grad(refine.pyramid_energy(T, J, x), x, grad_outputs=g, create_graph=True)
+    assert du.requires_grad
+    (dg,) = torch.autograd.grad((du * v).sum(), g)
+    assert float(dg) == pytest.approx(float((2 * u * v).double().sum()), rel=1e-5)
+
+
+def test_a_batch_of_incoming_gradients(quadratic):
+    T, J, u = quadratic
+    x = u.clone().requires_grad_(True)
+    g = torch.tensor([1.0, -2.5, 0.25], dtype=torch.float64)
+    (du,) = torch.autograd.grad(refine.pyramid_energy(T, J, x), x, grad_outputs=g, is_grads_batched=True)
+    torch.testing.assert_close(du, g.float()[:, None, None, None] * 2 * u)
+    jac = torch.autograd.functional.jacobian(lambda y: refine.pyramid_energy(T, J, y), u, vectorize=True)
+    torch.testing.assert_close(jac.float(), 2 * u)
