@@ -210,8 +210,8 @@ PANO_API pano_status pano_blend_coeff(const unsigned char* label, int h, int w, 
 
 /* E and its gradients for template T and target J (h x w float32, row pitch
  * `pitch` floats) and flow u ((h, w, 2) float32 contiguous).
- * energy: device pointer to one double that receives E (summed per thread in
- * pairs of floats, exact to about 2^-46, then in FP64), or NULL. grad_u ((h, w, 2)), grad_T ((h, w)) and grad_J ((h, w)), all float32
+ * energy: device pointer to one double that receives E (summed with the bits
+ * of FP64), or NULL. grad_u ((h, w, 2)), grad_T ((h, w)) and grad_J ((h, w)), all float32
  * contiguous, receive dE/du, dE/dT and dE/dJ; any may be NULL. dE/dJ is
  * accumulated with atomic additions, so its last bits vary between runs.
  * Errors: INVALID_ARG, CUDA. */

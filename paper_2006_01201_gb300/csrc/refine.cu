@@ -28,22 +28,33 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// A sum of squares in two floats: the rounding errors of the products and of
-// the additions are kept in `lo` (Knuth's exact addition, Moller 1965), which
-// leaves about 2^-46 of the sum. `big` is the largest magnitude added: the
-// errors are exact while the squares neither overflow nor leave the normal
-// range, 1e-15 .. 1e15.
+// a + b rounded, and the rounding error (Knuth's exact addition).
+__device__ __forceinline__ float two_sum(float a, float b, float* err) {
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    *err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+    return s;
+}
+
+// A sum of squares in three floats: the rounding errors of the products and of
+// the additions to `hi` go to `mid`, those of the additions to `mid` to `lo`.
+// Over kSquares pixels (four squares each at most) that leaves less than the
+// last bit of a double; then the sum goes into one. `big` is the largest
+// magnitude added: the errors are exact, or below 2^-70 of the sum, for
+// squares of 1e-12 .. 1e15.
+constexpr int kSquares = 16;
 struct SquareSum {
-    float hi = 0.f, lo = 0.f, big = 0.f;
+    float hi = 0.f, mid = 0.f, lo = 0.f, big = 0.f;
     __device__ __forceinline__ void add(float v) {
         const float p = __fmul_rn(v, v), e = __fmaf_rn(v, v, -p);
-        const float s = __fadd_rn(hi, p), b = __fsub_rn(s, hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(p, b)), e));
-        hi = s;
+        float r, r1, r2;
+        hi = two_sum(hi, p, &r);
+        mid = two_sum(mid, r, &r1);
+        mid = two_sum(mid, e, &r2);
+        lo = __fadd_rn(lo, __fadd_rn(r1, r2));
         big = fmaxf(big, fabsf(v));
     }
-    __device__ __forceinline__ bool exact() const { return big == 0.f || (big >= 1e-15f && big <= 1e15f); }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+    __device__ __forceinline__ bool exact() const { return big == 0.f || (big >= 1e-12f && big <= 1e15f); }
+    __device__ __forceinline__ double value() const { return (double)hi + ((double)mid + (double)lo); }
 };
 
 // What a pixel's energy and gradients are made of.
@@ -114,12 +125,23 @@ __device__ __noinline__ double energy_in_doubles(const EnergyArgs& a) {
 
 // E alone. FP64 instructions run at 1/64 of the FP32 rate here: five squares a
 // pixel in doubles, and a double atomic per 256 pixels, took 39 us on 1024^2
-// pixels; two-float sums and one atomic per CTA of a fixed grid take the place
-// of both.
+// pixels; sums of as many bits in three floats (22 us) and one atomic per CTA of a
+// fixed grid take the place of both. A thread adds one double per kSquares
+// pixels, so there are fewer roundings than with a double per pixel.
 __global__ void __launch_bounds__(kEgThreads) energy_kernel(const __grid_constant__ EnergyArgs a) {
     __shared__ double s_part[kEgThreads / 32];
     grid_begin();
     SquareSum data, smooth;
+    double e = 0.0;
+    bool exact = true;
+    int n = 0;
+    auto flush = [&]() {
+        exact = exact && data.exact() && smooth.exact();
+        e += data.value() + (double)a.alpha * smooth.value();
+        data = SquareSum();
+        smooth = SquareSum();
+        n = 0;
+    };
     energy_tiles(a, [&](int x, int y) {
         if (x >= a.w || y >= a.h) return;
         const EnergyPixel q = energy_pixel(a, x, y);
@@ -128,8 +150,10 @@ __global__ void __launch_bounds__(kEgThreads) energy_kernel(const __grid_constan
         smooth.add(q.right.y);
         smooth.add(q.down.x);
         smooth.add(q.down.y);
+        if (++n == kSquares) flush();
     });
-    double e = data.exact() && smooth.exact() ? data.value() + (double)a.alpha * smooth.value() : energy_in_doubles(a);
+    flush();
+    if (!exact) e = energy_in_doubles(a);
     __syncwarp();
     e = warp_sum(e);
     if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = e;

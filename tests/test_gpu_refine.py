@@ -174,13 +174,38 @@ def test_adjoint_at_the_border_of_its_interior(shape):
 
 @pytest.mark.parametrize("factor", [1.0, 1e-12, 1e-18, 1e17, 0.0])
 def test_energy_of_very_small_and_large_differences(factor):
-    # beyond 1e-15 .. 1e15 the squares are summed in doubles
+    # beyond 1e-12 .. 1e15 the squares are summed in doubles
     g = np.random.default_rng(5)
     T = cuda(np.zeros((70, 90)))
     J = cuda(g.normal(0, 1, (70, 90)) * factor)
     u = cuda(np.zeros((70, 90, 2)))
     E = float(binding.energy_grad(T, J, u, ALPHA, want_u=False, want_T=False, want_J=False)[0])
     assert E == pytest.approx(float((J.double() ** 2).sum()), rel=1e-12)
+
+
+# More than one tile per thread of the energy's fixed grid (above 311296 pixels),
+# up to several rounds of the float sums. The residual does not depend on the
+# flow (a constant target), so a float64 sum of the same float32 residuals and
+# differences is E up to the order of the double additions: at most 1216 of them
+# across CTAs, 31 within one and n / 16 + 1 in a thread, 2^-53 of the sum each.
+@pytest.mark.parametrize("factor", [1.0, 1e-16, 1e18])
+@pytest.mark.parametrize("kind", ["constant", "random"])
+@pytest.mark.parametrize("h,w", [(1031, 777), (2003, 1999), (6007, 4001)])
+def test_energy_of_many_pixels_per_thread(h, w, kind, factor):
+    if kind == "constant":
+        T = torch.full((h, w), 0.3, device=DEV)
+        odd = (torch.arange(h, device=DEV)[:, None] + torch.arange(w, device=DEV)) % 2
+        u = torch.stack([0.37 * odd, -0.11 * odd], -1).float()
+    else:
+        g = torch.Generator(device=DEV).manual_seed(h)
+        T = torch.rand((h, w), generator=g, device=DEV)
+        u = torch.randn((h, w, 2), generator=g, device=DEV)
+    T, J, u = T * factor, torch.full((h, w), 0.21 * factor, device=DEV), (u * factor).contiguous()
+    E = float(binding.energy_grad(T, J, u, ALPHA, want_u=False, want_T=False, want_J=False)[0])
+    sq = lambda d: float((d.double() ** 2).sum())
+    ref = sq(J - T) + float(np.float32(ALPHA)) * (sq(u[:, 1:] - u[:, :-1]) + sq(u[1:] - u[:-1]))
+    n = h * w / (1216 * 256)
+    assert E == pytest.approx(ref, rel=(1216 + 31 + n / 16 + 1) * 2.0 ** -53)
 
 
 def test_energy_of_non_numbers():
