@@ -71,9 +71,9 @@ class PyramidEnergy(torch.autograd.Function):
             dJ = _reduce_transpose(dJ, shapes) if need_J else None
         # Scaled by tensor operations, not by the library: the gradients stay
         # differentiable in gE (double backward, functional.jvp), and gE may be
-        # a batch (is_grads_batched), which has no pointer.
-        s = gE.to(torch.float32)
-        return tuple(g * s if g is not None else None for g in (dT, dJ, du)) + (None, None)
+        # a batch (is_grads_batched), which has no pointer. (A float32 tensor times
+        # a float64 scalar tensor is float32.)
+        return tuple(g * gE if g is not None else None for g in (dT, dJ, du)) + (None, None)
 
 
 def pyramid_energy(T0, J0, u, level: int = 0, alpha: float = 0.05):
