@@ -780,12 +780,20 @@ def stage_warp(src, flow, scale=1.0, stream=None):
     return dst
 
 
+def _same_planes(T, J, u, nT: str, nJ: str) -> None:
+    """Refuse planes of two sizes or devices: the kernels read both by one."""
+    if T.shape != J.shape or T.device != J.device or T.device != u.device:
+        raise PanoError(PANO_ERR_INVALID_ARG, f"{nT}, {nJ} and u differ in size or device: {tuple(T.shape)} on {T.device}, "
+                                              f"{tuple(J.shape)} on {J.device}, u on {u.device}")
+
+
 def energy_grad(T, J, u, alpha: float, want_energy=True, want_u=True, want_T=True, want_J=True, stream=None):
     """(E as a float64 0-d tensor or None, dE/du, dE/dT, dE/dJ) on the GPU."""
     torch = _torch()
     for t, n in ((T, "T"), (J, "J")):
         if t.dtype != torch.float32 or t.dim() != 2 or not t.is_contiguous():
             raise PanoError(PANO_ERR_INVALID_ARG, f"{n} must be a contiguous float32 (H, W) tensor")
+    _same_planes(T, J, u, "T", "J")
     h, w = T.shape
     uptr = _flow_ptr(u, h, w, "u")
     dev = T.device
@@ -802,6 +810,7 @@ def energy_grad(T, J, u, alpha: float, want_energy=True, want_u=True, want_T=Tru
 def _refine_args(T0, J0, u, level: int):
     """(tensors to keep, leading C arguments, scratch) of the refinement calls."""
     torch = _torch()
+    _same_planes(T0, J0, u, "T0", "J0")
     if level == 0:
         T0, J0 = T0.contiguous(), J0.contiguous()
     for t, n in ((T0, "T0"), (J0, "J0")):

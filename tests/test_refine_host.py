@@ -52,3 +52,16 @@ def test_a_batch_of_incoming_gradients(quadratic):
     torch.testing.assert_close(du, g.float()[:, None, None, None] * 2 * u)
     jac = torch.autograd.functional.jacobian(lambda y: refine.pyramid_energy(T, J, y), u, vectorize=True)
     torch.testing.assert_close(jac.float(), 2 * u)
+
+
+@pytest.mark.parametrize("call", [lambda T, J, u: binding.energy_grad(T, J, u, 0.05),
+                                  lambda T, J, u: binding.refine_energy(T, J, u, 0, 0.05),
+                                  lambda T, J, u: binding.refine_grad(T, J, u, 0, 0.05)],
+                         ids=["energy_grad", "refine_energy", "refine_grad"])
+def test_planes_that_differ_are_refused(call):
+    # before anything is read: the kernels use T's size for both planes
+    T, u = torch.zeros((8, 6)), torch.zeros((8, 6, 2))
+    for J in (torch.zeros((7, 6)), torch.zeros((8, 5)), torch.zeros((9, 6)), torch.zeros((8, 6), device="meta")):
+        with pytest.raises(binding.PanoError, match="differ") as e:
+            call(T, J, u)
+        assert e.value.status == binding.PANO_ERR_INVALID_ARG
