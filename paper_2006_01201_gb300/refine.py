@@ -64,11 +64,10 @@ class PyramidEnergy(torch.autograd.Function):
         else:
             Tl = _levels(T0, ctx.level)          # rebuilt, not stored
             Jl = _levels(J0, ctx.level)
-            shapes = [tuple(t.shape) for t in Tl]
             _, du, dT, dJ = binding.energy_grad(Tl[-1].contiguous(), Jl[-1].contiguous(), u.contiguous(), ctx.alpha,
                                                 want_energy=False, want_u=need_u, want_T=need_T, want_J=need_J)
-            dT = _reduce_transpose(dT, shapes) if need_T else None
-            dJ = _reduce_transpose(dJ, shapes) if need_J else None
+            dT = _reduce_transpose(dT, [tuple(t.shape) for t in Tl]) if need_T else None
+            dJ = _reduce_transpose(dJ, [tuple(t.shape) for t in Jl]) if need_J else None
         # Scaled by tensor operations, not by the library: the gradients stay
         # differentiable in gE (double backward, functional.jvp), and gE may be
         # a batch (is_grads_batched), which has no pointer. (A float32 tensor times

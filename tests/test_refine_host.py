@@ -65,3 +65,21 @@ def test_planes_that_differ_are_refused(call):
         with pytest.raises(binding.PanoError, match="differ") as e:
             call(T, J, u)
         assert e.value.status == binding.PANO_ERR_INVALID_ARG
+
+
+def test_planes_of_two_sizes_with_equal_levels(monkeypatch):
+    # 100 and 99 rows are 50 at level 1: each plane's gradient has its own size
+    down = lambda t: torch.zeros(((t.shape[0] + 1) // 2, (t.shape[1] + 1) // 2))
+    monkeypatch.setattr(binding, "stage_pyr_down", down)
+
+    def adjoint(g, h, w):
+        assert tuple(g.shape) == ((h + 1) // 2, (w + 1) // 2)
+        return torch.ones((h, w))
+
+    monkeypatch.setattr(binding, "stage_pyr_down_adjoint", adjoint)
+    monkeypatch.setattr(binding, "energy_grad", lambda T, J, u, alpha, **k: (
+        torch.zeros((), dtype=torch.float64), torch.ones_like(u), torch.ones_like(T), torch.ones_like(J)))
+    T0, J0 = torch.zeros((100, 40), requires_grad=True), torch.zeros((99, 39), requires_grad=True)
+    u = torch.zeros((50, 20, 2), requires_grad=True)
+    refine.pyramid_energy(T0, J0, u, 1).backward()
+    assert T0.grad.shape == T0.shape and J0.grad.shape == J0.shape and u.grad.shape == u.shape
