@@ -189,6 +189,22 @@ def _stream_ptr(stream) -> int:
     return int(s.cuda_stream)
 
 
+def _on_stream(stream, call):
+    """call() with `stream` as the current one, so that what it allocates and
+    copies belongs to the stream it launches on: its scratch may be dropped
+    on return, and only that stream's later work can get the memory. The
+    results are kept for the caller's stream as well."""
+    torch = _torch()
+    s = stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(int(stream.cuda_stream))
+    caller = torch.cuda.current_stream()
+    with torch.cuda.stream(s):
+        res = call()
+    for t in res if isinstance(res, tuple) else (res,):
+        if t is not None:
+            t.record_stream(caller)
+    return res
+
+
 def image_desc(t) -> PanoImage:
     """pano_image for an (H, W) or (H, W, C) CUDA tensor."""
     torch = _torch()
@@ -829,17 +845,21 @@ def _refine_args(T0, J0, u, level: int):
 
 def refine_energy(T0, J0, u, level: int, alpha: float, stream=None):
     """E (float64 0-d tensor) at pyramid level `level` of T0 and J0 (pano_refine_energy)."""
+    if stream is not None:
+        return _on_stream(stream, lambda: refine_energy(T0, J0, u, level, alpha))
     torch = _torch()
     keep, args, scratch = _refine_args(T0, J0, u, level)
     E = torch.empty((), dtype=torch.float64, device=T0.device)
     sp, sn = (scratch.data_ptr(), scratch.numel()) if scratch is not None else (None, 0)
-    _check(load_library().pano_refine_energy(*args, float(alpha), E.data_ptr(), sp, sn, _stream_ptr(stream)))
+    _check(load_library().pano_refine_energy(*args, float(alpha), E.data_ptr(), sp, sn, _stream_ptr(None)))
     return E
 
 
 def refine_grad(T0, J0, u, level: int, alpha: float, scale=None, want_u=True, want_T=True, want_J=True, stream=None):
     """(dE/du, dE/dT0, dE/dJ0) times `scale`, a float64 0-d CUDA tensor or None
     (pano_refine_grad); None in the place of a gradient that is not wanted."""
+    if stream is not None:
+        return _on_stream(stream, lambda: refine_grad(T0, J0, u, level, alpha, scale, want_u, want_T, want_J))
     torch = _torch()
     keep, args, scratch = _refine_args(T0, J0, u, level)
     dev = T0.device
@@ -851,7 +871,7 @@ def refine_grad(T0, J0, u, level: int, alpha: float, scale=None, want_u=True, wa
     ptr = lambda t: None if t is None else t.data_ptr()
     sp, sn = (scratch.data_ptr(), scratch.numel()) if scratch is not None else (None, 0)
     _check(load_library().pano_refine_grad(*args, float(alpha), ptr(scale), ptr(gu), ptr(gt), ptr(gj), sp, sn,
-                                           _stream_ptr(stream)))
+                                           _stream_ptr(None)))
     return gu, gt, gj
 
 

@@ -216,3 +216,33 @@ def test_energy_of_non_numbers():
         # at the corner: every tap of the pixel is the value itself for T; J mixes inf - inf
         E = float(binding.energy_grad(cuda(A), T, u, ALPHA, want_u=False, want_T=False, want_J=False)[0])
         assert check(E)
+
+
+def _reuse_at_once(sizes):
+    """Allocate the sizes (bytes) on the current stream and overwrite them."""
+    kept = [torch.full((n,), 0x7F, dtype=torch.uint8, device=DEV) for n in sizes for _ in range(4)]
+    torch.cuda.current_stream().synchronize()
+    return kept
+
+
+def test_scratch_of_a_call_on_another_stream():
+    # the side stream is busy when the calls return: what the current stream
+    # allocates meanwhile must not be their scratch or copies
+    h, w, level = 301, 402, 2
+    T0, J0, u = _step_arrays(h, w, level, 11)
+    u = u.transpose(0, 1).contiguous().transpose(0, 1)      # copied by the call
+    E = binding.refine_energy(T0, J0, u, level, ALPHA)
+    want = binding.refine_grad(T0, J0, u, level, ALPHA)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    n = int(binding.load_library().pano_refine_scratch_bytes(h, w, level))
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(20_000_000)                       # some 10 ms
+    E1 = binding.refine_energy(T0, J0, u, level, ALPHA, stream=side)
+    got = binding.refine_grad(T0, J0, u, level, ALPHA, stream=side)
+    kept = _reuse_at_once([n, u.numel() * 4])
+    side.synchronize()
+    assert float(E1) == pytest.approx(float(E), rel=1e-12)
+    for a, b in zip(got, want):
+        assert (a - b).abs().max() <= 4e-6 * max(1.0, float(b.abs().max()))
+    del kept
