@@ -189,15 +189,19 @@ def _stream_ptr(stream) -> int:
     return int(s.cuda_stream)
 
 
+def _torch_stream(stream):
+    torch = _torch()
+    return stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(int(stream.cuda_stream))
+
+
 def _on_stream(stream, call):
     """call() with `stream` as the current one, so that what it allocates and
     copies belongs to the stream it launches on: its scratch may be dropped
     on return, and only that stream's later work can get the memory. The
     results are kept for the caller's stream as well."""
     torch = _torch()
-    s = stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(int(stream.cuda_stream))
     caller = torch.cuda.current_stream()
-    with torch.cuda.stream(s):
+    with torch.cuda.stream(_torch_stream(stream)):
         res = call()
     for t in res if isinstance(res, tuple) else (res,):
         if t is not None:
@@ -676,6 +680,11 @@ def blend_coeff(label, out=None, scratch=None, stream=None):
     1 = Area1, 2 = Area2, 3 = Area3 (overlap), other = neither; returns the
     float32 (H, W) Blend array. scratch: optional uint8 device tensor of
     pano_blend_coeff_scratch_bytes(H, W) bytes, reused across calls."""
+    if stream is not None and scratch is None:
+        if out is None:
+            return _on_stream(stream, lambda: blend_coeff(label))
+        with _torch().cuda.stream(_torch_stream(stream)):
+            return blend_coeff(label, out)
     torch = _torch()
     if label.dtype != torch.uint8 or label.dim() != 2 or not label.is_cuda or label.stride(1) != 1:
         raise PanoError(PANO_ERR_INVALID_ARG, "label must be a uint8 (H, W) CUDA tensor with contiguous rows")

@@ -174,6 +174,27 @@ def test_bad_arguments_raise():
         binding.blend_coeff(lab.float())
 
 
+def test_scratch_of_a_call_on_another_stream():
+    # the side stream is busy when the call returns: what the current stream
+    # allocates meanwhile must not be its scratch
+    label = np.random.default_rng(2).choice([1, 2, 3], size=(211, 307)).astype(np.uint8)
+    lab = torch.from_numpy(label).to(DEV)
+    want = binding.blend_coeff(lab)
+    out = torch.empty_like(want)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    n = int(binding.load_library().pano_blend_coeff_scratch_bytes(*label.shape))
+    for given in (None, out):
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(20_000_000)   # some 10 ms
+        got = binding.blend_coeff(lab, out=given, stream=side)
+        kept = [torch.full((n,), 0x7F, dtype=torch.uint8, device=DEV) for _ in range(4)]
+        torch.cuda.current_stream().synchronize()
+        side.synchronize()
+        assert torch.equal(got, want)
+        del kept
+
+
 # The row pass works on groups of 32 columns (loads of 8) and bisects over the
 # groups with Area3; diagonals above 46340 take the other row pass. Sizes on either
 # side of each, areas that miss from whole columns, and one-group rows.
