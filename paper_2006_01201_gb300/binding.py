@@ -832,6 +832,9 @@ def energy_grad(T, J, u, alpha: float, want_energy=True, want_u=True, want_T=Tru
     return E, gu, gt, gj
 
 
+REFINE_LEVELS = 12   # pyramid levels that pano_refine_energy / pano_refine_grad take
+
+
 def _refine_args(T0, J0, u, level: int):
     """(tensors to keep, leading C arguments, scratch) of the refinement calls."""
     torch = _torch()

@@ -38,13 +38,20 @@ def _reduce_transpose(g: torch.Tensor, shapes: List[Tuple[int, int]]) -> torch.T
     return g
 
 
+def _one_call(T0: torch.Tensor, J0: torch.Tensor, level: int) -> bool:
+    """Whether pano_refine_energy / pano_refine_grad take the step: planes of one
+    size, and a level below their limit of 12. Else the per-stage calls do (a
+    negative level is level 0 there)."""
+    return T0.shape == J0.shape and 0 <= level < binding.REFINE_LEVELS
+
+
 class PyramidEnergy(torch.autograd.Function):
     """E at pyramid level `level` of T0, J0 for the flow u (float64 scalar)."""
 
     @staticmethod
     def forward(ctx, T0, J0, u, level: int, alpha: float):
         ctx.save_for_backward(T0, J0, u)
-        if T0.shape == J0.shape:
+        if _one_call(T0, J0, level):
             E = binding.refine_energy(T0, J0, u, level, alpha)
         else:
             T = _levels(T0, level)[-1]
@@ -58,7 +65,7 @@ class PyramidEnergy(torch.autograd.Function):
     def backward(ctx, gE):
         T0, J0, u = ctx.saved_tensors
         need_T, need_J, need_u = ctx.needs_input_grad[:3]
-        if T0.shape == J0.shape:   # the whole step in one call
+        if _one_call(T0, J0, ctx.level):
             du, dT, dJ = binding.refine_grad(T0, J0, u, ctx.level, ctx.alpha, want_u=need_u, want_T=need_T,
                                              want_J=need_J)
         else:

@@ -83,3 +83,22 @@ def test_planes_of_two_sizes_with_equal_levels(monkeypatch):
     u = torch.zeros((50, 20, 2), requires_grad=True)
     refine.pyramid_energy(T0, J0, u, 1).backward()
     assert T0.grad.shape == T0.shape and J0.grad.shape == J0.shape and u.grad.shape == u.shape
+
+
+@pytest.mark.parametrize("level", [12, -1])
+def test_levels_beyond_the_one_call_form(monkeypatch, quadratic, level):
+    # pano_refine_* take levels 0 .. 11; the per-stage calls have no limit
+    def refuse(*a, **k):
+        raise binding.PanoError(binding.PANO_ERR_INVALID_ARG, "level not in 0..11")
+
+    T, J, _ = quadratic
+    monkeypatch.setattr(binding, "refine_energy", refuse)
+    monkeypatch.setattr(binding, "refine_grad", refuse)
+    monkeypatch.setattr(binding, "stage_pyr_down",
+                        lambda t: torch.zeros(((t.shape[0] + 1) // 2, (t.shape[1] + 1) // 2)))
+    monkeypatch.setattr(binding, "stage_pyr_down_adjoint", lambda g, h, w: torch.ones((h, w)))
+    monkeypatch.setattr(binding, "energy_grad", lambda T, J, u, alpha, **k: (
+        torch.zeros((), dtype=torch.float64), torch.ones_like(u), torch.ones_like(T), torch.ones_like(J)))
+    T, u = T.clone().requires_grad_(True), torch.zeros((1, 1, 2), requires_grad=True)
+    refine.pyramid_energy(T, J, u, level).backward()
+    assert T.grad.shape == T.shape and u.grad.shape == u.shape
