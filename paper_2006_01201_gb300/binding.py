@@ -842,7 +842,7 @@ def _refine_args(T0, J0, u, level: int):
     if level == 0:
         T0, J0 = T0.contiguous(), J0.contiguous()
     for t, n in ((T0, "T0"), (J0, "J0")):
-        if t.dtype != torch.float32 or t.dim() != 2 or t.stride(1) != 1 or not t.is_cuda:
+        if t.dtype != torch.float32 or t.dim() != 2 or (level > 0 and t.stride(1) != 1) or not t.is_cuda:
             raise PanoError(PANO_ERR_INVALID_ARG, f"{n} must be a float32 (H, W) CUDA tensor with contiguous rows")
     h, w = T0.shape
     hl, wl = h, w
@@ -852,7 +852,10 @@ def _refine_args(T0, J0, u, level: int):
     uptr = _flow_ptr(u, hl, wl, "u")
     need = int(load_library().pano_refine_scratch_bytes(h, w, level))
     scratch = torch.empty(need, dtype=torch.uint8, device=T0.device) if need else None
-    return (T0, J0, u), (T0.data_ptr(), J0.data_ptr(), h, w, T0.stride(0), J0.stride(0), level, uptr), scratch
+    # a contiguous plane's strides are not always (w, 1): those of sides of one
+    # element are free
+    pT, pJ = (w, w) if level == 0 else (T0.stride(0), J0.stride(0))
+    return (T0, J0, u), (T0.data_ptr(), J0.data_ptr(), h, w, pT, pJ, level, uptr), scratch
 
 
 def refine_energy(T0, J0, u, level: int, alpha: float, stream=None):

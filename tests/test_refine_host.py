@@ -102,3 +102,14 @@ def test_levels_beyond_the_one_call_form(monkeypatch, quadratic, level):
     T, u = T.clone().requires_grad_(True), torch.zeros((1, 1, 2), requires_grad=True)
     refine.pyramid_energy(T, J, u, level).backward()
     assert T.grad.shape == T.shape and u.grad.shape == u.shape
+
+
+@pytest.mark.parametrize("plane", [torch.zeros((7, 1)).t(), torch.empty_strided((7, 1), (1, 7)), torch.zeros((1, 9))[:, ::3],
+                                   torch.zeros((3, 1, 2))[:, :, 1], torch.zeros((6, 8))[:, 2:5]])
+def test_strides_of_planes_at_level_0(monkeypatch, plane):
+    # planes are made contiguous at level 0, whatever their strides; the stride
+    # of a side of one element says nothing
+    monkeypatch.setattr(torch.Tensor, "is_cuda", True, raising=False)
+    h, w = plane.shape
+    _, args, _ = binding._refine_args(plane, plane, torch.zeros((h, w, 2)), 0)
+    assert args[2:7] == (h, w, w, w, 0)
