@@ -926,9 +926,12 @@ pano_status check_refine(const float* T0, const float* J0, int h, int w, int pit
     if (((uintptr_t)T0) % 4 || ((uintptr_t)J0) % 4 || ((uintptr_t)u) % 8)
         return fail(PANO_ERR_INVALID_ARG, "T0, J0 or u misaligned");
     if (!(alpha >= 0.f) || !(alpha < 1e30f)) return fail(PANO_ERR_INVALID_ARG, "alpha must be finite and >= 0");
-    if ((double)h * (double)(pitch_T > pitch_J ? pitch_T : pitch_J) > (double)INT_MAX)
-        return fail(PANO_ERR_UNSUPPORTED, "more than 2^31 elements");
-    const size_t need = RefineScratch(h, w, level, nullptr).bytes;
+    const RefineScratch r(h, w, level, nullptr);
+    // the level's plane only: REDUCE and its transpose index with 64 bits
+    const int pitch = level ? r.w[level] : pitch_T > pitch_J ? pitch_T : pitch_J;
+    if ((double)r.h[level] * (double)pitch > (double)INT_MAX)
+        return fail(PANO_ERR_UNSUPPORTED, "more than 2^31 elements at level %d", level);
+    const size_t need = r.bytes;
     if (need && (!scratch || ((uintptr_t)scratch) % 16 || scratch_bytes < need))
         return fail(PANO_ERR_INVALID_ARG, "scratch is NULL, not 16-byte aligned or of less than %zu bytes", need);
     return PANO_OK;

@@ -234,3 +234,26 @@ def test_static_flow_rejects_bad_arguments_before_any_device_call(lib):
     big = binding.PanoImage(0x100000, 2048, 2048, 1, 8192, binding.PANO_F32)
     assert call(L=big, R=big, rl=0x200000 + 2048 * 2048 * 8) == inv
     assert b"scratch" in lib.pano_last_error(None)
+
+
+def test_refine_limits_the_plane_of_its_level(lib):
+    """2^31 elements is the limit of the plane whose energy is formed, as in
+    pano_energy_grad; the planes above it may be larger. (The scratch is
+    looked at last: the calls end there, on the host.)"""
+    inv, uns = binding.PANO_ERR_INVALID_ARG, binding.PANO_ERR_UNSUPPORTED
+
+    def energy(h, w, pitch, level):
+        return lib.pano_refine_energy(0x100000, 0x200000, h, w, pitch, pitch, level, 0x300000, 0.05, 0x400000, None, 0, None)
+
+    def grad(h, w, pitch, level):
+        return lib.pano_refine_grad(0x100000, 0x200000, h, w, pitch, pitch, level, 0x300000, 0.05, None, 0x400000, None,
+                                    None, None, 0, None)
+
+    for call in (energy, grad):
+        assert call(50000, 50000, 50000, 1) == inv          # 625 M elements at level 1
+        assert b"scratch" in lib.pano_last_error(None)
+        assert call(1000, 1000, 3000000, 1) == inv          # only the pitch is large
+        assert b"scratch" in lib.pano_last_error(None)
+        assert call(50000, 50000, 50000, 0) == uns
+        assert call(1000, 1000, 3000000, 0) == uns
+        assert call(100000, 100000, 100000, 1) == uns       # 2.5 G elements at level 1
