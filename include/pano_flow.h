@@ -64,7 +64,7 @@ typedef enum pano_status {
     PANO_ERR_UNSUPPORTED = 2,  /* valid request this build does not implement */
     PANO_ERR_OOM = 3,          /* device allocation failed (create only) */
     PANO_ERR_CUDA = 4,         /* a CUDA call or launch failed */
-    PANO_ERR_TIMEOUT = 5       /* reserved: a bounded device wait gave up */
+    PANO_ERR_TIMEOUT = 5       /* a bounded device wait gave up (pano_wait_status) */
 } pano_status;
 
 typedef enum pano_dtype {
@@ -410,6 +410,21 @@ PANO_API pano_status pano_stage_warp(const pano_image* src, const float* flow, f
  * first). In the normal build it writes zeros and returns UNSUPPORTED.
  * Errors: INVALID_ARG (out NULL), UNSUPPORTED, CUDA. */
 PANO_API pano_status pano_debug_bounds(unsigned* out);
+
+/* ----------------------------------------------------------------------
+ * Device waits. The blocks of the streamed LK kernel wait for rows of their
+ * neighbours. Every such wait is limited (65536 tries, about a quarter of a
+ * second; at most two waits a step); the flows that needed rows that never came
+ * are not-a-number, and the wait is counted.
+ * pano_wait_status returns PANO_ERR_TIMEOUT if any wait on the current device
+ * gave up since the last call, which clears the count; it reads device memory,
+ * so call it after the work has completed, outside stream capture. With
+ * PANO_DEBUG=sync the call that gave up returns PANO_ERR_TIMEOUT itself.
+ * pano_debug_wait enqueues a wait that nothing ends (one warp)
+ * in the check variant; UNSUPPORTED in the normal build.
+ * Errors: TIMEOUT, UNSUPPORTED, CUDA. */
+PANO_API pano_status pano_wait_status(void);
+PANO_API pano_status pano_debug_wait(void* cuda_stream);
 
 #ifdef __cplusplus
 }

@@ -78,6 +78,8 @@ SIGNATURES = {
     "pano_flow_pair": ([_VP, _IMG, _IMG, _VP, _VP, _VP], _I),
     "pano_blend_pair": ([_VP, _IMG, _IMG, _VP, _VP, _VP, _IMG, _VP], _I),
     "pano_debug_bounds": ([ctypes.POINTER(ctypes.c_uint)], _I),
+    "pano_wait_status": ([], _I),
+    "pano_debug_wait": ([_VP], _I),
     "pano_compose_pair": ([_PAR, _IMG, _IMG, _VP, ctypes.c_size_t, _VP, _I, _VP, _VP, _I, _I, _I, _I, _IMG, _VP], _I),
     "pano_flow_destroy": ([_VP], _I),
     "pano_last_error": ([_VP], ctypes.c_char_p),
@@ -153,6 +155,12 @@ def debug_bounds():
     out = (ctypes.c_uint * 4)()
     _check(load_library().pano_debug_bounds(out))
     return tuple(out)
+
+
+def wait_status() -> None:
+    """Raise PanoError (PANO_ERR_TIMEOUT) if a bounded wait of a kernel gave up
+    since the last call (pano_wait_status); synchronise before calling."""
+    _check(load_library().pano_wait_status())
 
 
 def _check(status: int) -> None:

@@ -37,6 +37,8 @@ pano_status fail(pano_status st, const char* fmt, ...) {
 }
 
 pano_status cuda_fail(cudaError_t e, const char* what) {
+    if (e == cudaErrorLaunchTimeout)  // from debug_check: a wait in a kernel gave up
+        return fail(PANO_ERR_TIMEOUT, "%s: a bounded device wait gave up", what);
     return fail(PANO_ERR_CUDA, "%s: %s (%s)", what, cudaGetErrorName(e), cudaGetErrorString(e));
 }
 
@@ -247,7 +249,10 @@ cudaError_t debug_check(cudaStream_t s) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone) return cudaSuccess;
     cudaError_t e = cudaStreamSynchronize(s);
-    return e != cudaSuccess ? e : cudaGetLastError();
+    if (e == cudaSuccess) e = cudaGetLastError();
+    unsigned lost = 0;
+    if (e == cudaSuccess) e = lk_stream_lost(&lost);
+    return e == cudaSuccess && lost ? cudaErrorLaunchTimeout : e;
 }
 
 NvtxRange::NvtxRange(const char* name) { nvtxRangePushA(name); }
@@ -658,6 +663,26 @@ pano_status pano_debug_bounds(unsigned* out) {
     return PANO_OK;
 #else
     return fail(PANO_ERR_UNSUPPORTED, "this build has no index checks (build the check variant)");
+#endif
+}
+
+pano_status pano_wait_status(void) {
+    unsigned lost = 0;
+    const cudaError_t e = lk_stream_lost(&lost);
+    if (e != cudaSuccess) return cuda_fail(e, "reading the record of device waits");
+    if (lost) return fail(PANO_ERR_TIMEOUT, "%u threads gave up a wait for rows of a neighbouring block", lost);
+    return PANO_OK;
+}
+
+pano_status pano_debug_wait(void* cuda_stream) {
+#ifdef PANO_BOUNDS_CHECK
+    cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+    cudaError_t e = launch_lost_halo(s);
+    if (e == cudaSuccess) e = debug_check(s);
+    return e == cudaSuccess ? PANO_OK : cuda_fail(e, "wait that nothing ends");
+#else
+    (void)cuda_stream;
+    return fail(PANO_ERR_UNSUPPORTED, "this build has no failing wait (build the check variant)");
 #endif
 }
 

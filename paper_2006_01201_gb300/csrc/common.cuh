@@ -341,6 +341,12 @@ inline bool lk_auto_streams(int iters, int radius) { return iters >= 1 && iters 
 cudaError_t lk_stream_prepare(int max_smem_bytes);
 cudaError_t launch_lk_stream(const LkArgs& a, int ndirs, cudaStream_t s);
 cudaError_t launch_lk_stream_batch(const LkBatch& b, cudaStream_t s, int* kernels);
+// Threads of the streamed kernel that gave up a wait for their neighbours'
+// rows since the last call, which clears the count (synchronous).
+cudaError_t lk_stream_lost(unsigned* n);
+cudaError_t lost_read_lk_stream_bf16(unsigned* n);
+cudaError_t lost_read_lk_stream_f16(unsigned* n);
+cudaError_t launch_lost_halo(cudaStream_t s);  // check variant: one such wait
 size_t lk_smem_bytes(int tile_w, int tile_h, int iters, int radius);
 cudaError_t lk_prepare(int max_smem_bytes);
 cudaError_t launch_blend(const BlendArgs& a, cudaStream_t s);

@@ -13,6 +13,34 @@ PANO_LKS_EXTERN(__half)
 }  // namespace lks
 
 PANO_BOUNDS_READER(bounds_read_lk_stream)
+PANO_LKS_LOST_READER(lost_read_lk_stream)
+
+cudaError_t lk_stream_lost(unsigned* n) {
+    *n = 0;
+    cudaError_t e = lost_read_lk_stream(n);
+    if (e == cudaSuccess) e = lost_read_lk_stream_bf16(n);
+    return e == cudaSuccess ? lost_read_lk_stream_f16(n) : e;
+}
+
+#ifdef PANO_BOUNDS_CHECK
+namespace {
+// a warp that waits for 16 bytes that nobody sends
+__global__ void lost_halo_kernel() {
+    __shared__ __align__(8) unsigned long long s_bar;
+    const unsigned bar = (unsigned)__cvta_generic_to_shared(&s_bar);
+    if (threadIdx.x == 0) {
+        lks::bar_init(bar);
+        lks::bar_expect(bar, 16);
+    }
+    __syncwarp();
+    if (!lks::bar_wait(bar, 0)) atomicAdd(&g_lost_halos, 1u);
+}
+}  // namespace
+cudaError_t launch_lost_halo(cudaStream_t s) {
+    lost_halo_kernel<<<1, 32, 0, s>>>();
+    return cudaGetLastError();
+}
+#endif
 
 bool lk_stream_supports(int iters, int radius) { return iters >= 1 && iters <= 5 && radius >= 1 && radius <= 3; }
 

@@ -7,4 +7,5 @@ namespace lks {
 PANO_LKS_INSTANTIATE(__half)
 }  // namespace lks
 PANO_BOUNDS_READER(bounds_read_lk_stream_f16)
+PANO_LKS_LOST_READER(lost_read_lk_stream_f16)
 }  // namespace pano

@@ -66,6 +66,10 @@
 #include "bounds.cuh"
 #include "common.cuh"
 
+namespace {
+__device__ unsigned g_lost_halos;  // threads that gave up a wait, since the last read
+}  // namespace
+
 namespace pano {
 namespace lks {
 
@@ -143,8 +147,12 @@ __device__ __forceinline__ void bar_expect(unsigned bar, unsigned bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 // Waits until the phase of this parity has ended; false if it has not after
-// a bounded number of tries (some 0.1 s at least), which no launch that the
-// host checks let through reaches.
+// kWaitTries tries, a quarter of a second (a try that fails takes 3.9 us). No
+// launch that the host checks let through comes to that: a cluster is scheduled
+// as a whole. (A limit by the clock instead, or no further waits for a thread
+// that has given up once, cost 2 to 4% of the pairs and rigs: a flag carried
+// from wait to wait, and spills.)
+constexpr int kWaitTries = 1 << 16;
 __device__ __forceinline__ bool bar_try(unsigned bar, unsigned parity) {
     unsigned done;
     asm volatile(
@@ -155,7 +163,7 @@ __device__ __forceinline__ bool bar_try(unsigned bar, unsigned parity) {
     return done != 0;
 }
 __device__ __forceinline__ bool bar_retry(unsigned bar, unsigned parity) {
-    for (int n = 0; n < (1 << 22); ++n)
+    for (int n = 0; n < kWaitTries; ++n)
         if (bar_try(bar, parity)) return true;
     return false;
 }
@@ -653,6 +661,7 @@ __device__ __forceinline__ void lk_stream_item(const LkArgs& a, int dir, int ox,
         if (c0) PANO_AT(uo, o, NUO, 154) = make_float2(ux[j].x + end.x, uy[j].x + end.y);
         if (c1) PANO_AT(uo, o + 1, NUO, 155) = make_float2(ux[j].y + end.x, uy[j].y + end.y);
     }
+    if (__builtin_expect(lost, 0)) atomicAdd(&g_lost_halos, 1u);
 }
 
 // How a level is cut: nb bands, ns segments (clusters) per band of csize CTAs
@@ -844,6 +853,17 @@ cudaError_t stream_prepare(int max_smem_bytes) {
     if ((e = prepare_rad_stream<2, Ts>(max_smem_bytes)) != cudaSuccess) return e;
     return prepare_rad_stream<3, Ts>(max_smem_bytes);
 }
+
+// host: add this unit's count of given-up waits to *n and clear it
+#define PANO_LKS_LOST_READER(fn)                                                \
+    cudaError_t fn(unsigned* n) {                                               \
+        unsigned v = 0;                                                         \
+        cudaError_t e = cudaMemcpyFromSymbol(&v, g_lost_halos, sizeof(v));      \
+        if (e != cudaSuccess || v == 0) return e;                               \
+        *n += v;                                                                \
+        v = 0;                                                                  \
+        return cudaMemcpyToSymbol(g_lost_halos, &v, sizeof(v));                 \
+    }
 
 #define PANO_LKS_INSTANTIATE(Ts)                                                      \
     template cudaError_t stream_launch<Ts>(const LkArgs&, int, cudaStream_t);        \

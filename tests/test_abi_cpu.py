@@ -144,6 +144,7 @@ def test_release_build_has_no_index_checks():
     assert lib.pano_debug_bounds(out) == binding.PANO_ERR_UNSUPPORTED
     assert tuple(out) == (0, 0, 0, 0)
     assert lib.pano_debug_bounds(None) == binding.PANO_ERR_INVALID_ARG
+    assert lib.pano_debug_wait(None) == binding.PANO_ERR_UNSUPPORTED
 
 
 def test_missing_library_fails_loudly(tmp_path, monkeypatch):

@@ -57,3 +57,28 @@ def test_sync_mode_gives_the_same_results(monkeypatch):
         rig.run([L], [R], canvas=canvas, use_graph=True)  # capture: no synchronisation inside it
         torch.cuda.synchronize()
         assert torch.equal(canvas, ref[2])
+
+
+def test_a_wait_that_nothing_ends_is_reported(monkeypatch):
+    # one warp of the check variant waits for rows that nobody sends, until its
+    # limit of a quarter of a second; the context stays usable
+    lib = binding.open_library(gpu_build.build(variant="check"))
+    monkeypatch.setattr(binding, "_lib", lib)
+    binding.wait_status()
+    stream = torch.cuda.current_stream().cuda_stream
+    t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    t0.record()
+    assert lib.pano_debug_wait(stream) == binding.PANO_OK      # only enqueued
+    t1.record()
+    torch.cuda.synchronize()
+    assert 50 < t0.elapsed_time(t1) < 2000
+    with pytest.raises(binding.PanoError) as ei:
+        binding.wait_status()
+    assert ei.value.status == binding.PANO_ERR_TIMEOUT
+    binding.wait_status()                                      # reported once
+    monkeypatch.setenv("PANO_DEBUG", "sync")
+    assert lib.pano_debug_wait(stream) == binding.PANO_ERR_TIMEOUT
+    z = torch.zeros((64, 300), dtype=torch.float32, device=DEV)
+    with binding.FlowContext(binding.Params(levels=3), 64, 300, 1) as ctx:
+        assert torch.count_nonzero(ctx.flow_pair(z, z)[0]) == 0
+    binding.wait_status()
