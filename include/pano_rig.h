@@ -11,9 +11,10 @@
  *   luma of all strips          one launch
  *   REDUCE of all strips        one launch per level
  *   LK, both directions, every  per level, one launch of the streamed
- *   pair                        kernel over every (pair, direction, band,
- *                               segment) and/or one tiled
- *                               grid per tile shape over those pairs
+ *   pair                        kernel per CTA shape and cluster size over
+ *                               every (pair, direction, band, segment),
+ *                               and/or one tiled grid per tile shape over
+ *                               those pairs
  *   blend into the canvas       one launch
  *
  * The whole sequence can be captured once in a CUDA graph and replayed. The
@@ -104,8 +105,8 @@ PANO_API pano_status pano_rig_run(pano_rig* rig, const pano_image* L, const pano
 /* Autotune the LK kernel of every level on the strips L, R (flows kept in
  * the rig): after one full run, each level is timed with CUDA events, `reps`
  * launches per candidate after one warm-up launch, over PANO_LK_AUTO, the
- * streamed kernel with segment heights {auto, 64, 96, 128, 192, 256, 384}
- * and the tiled kernel with every tile of {32x8, 32x16, 16x16, 64x8, 64x16,
+ * streamed kernel with every cluster size (1 to 8 CTAs, as seg_rows) that
+ * cuts the level in another way, and the tiled kernel with every tile of {32x8, 32x16, 16x16, 64x8, 64x16,
  * 32x32} that fits the device's shared memory; the fastest (median) becomes
  * the level's tuning. Synchronises cuda_stream. Errors: INVALID_ARG, CUDA. */
 PANO_API pano_status pano_rig_autotune(pano_rig* rig, const pano_image* L, const pano_image* R, int reps,

@@ -339,6 +339,12 @@ cudaError_t launch_lk_tile_batch(const LkBatch& b, cudaStream_t s);
 bool lk_stream_supports(int iters, int radius);
 inline bool lk_auto_streams(int iters, int radius) { return iters >= 1 && iters * radius <= kStreamMaxReach; }
 cudaError_t lk_stream_prepare(int max_smem_bytes);
+// CTAs of a cluster that a level is cut with (1 <= iters, iters * radius up to
+// kStreamMaxReach), and the seg_rows that ask for clusters of csize CTAs, 1 to
+// kStreamMaxCluster (0: not for this level).
+constexpr int kStreamMaxCluster = 8;  // the portable limit
+int lk_stream_cluster(int w, int h, int iters, int radius, int seg_rows);
+int lk_stream_seg_rows(int w, int h, int iters, int radius, int csize);
 cudaError_t launch_lk_stream(const LkArgs& a, int ndirs, cudaStream_t s);
 cudaError_t launch_lk_stream_batch(const LkBatch& b, cudaStream_t s, int* kernels);
 // Threads of the streamed kernel that gave up a wait for their neighbours'

@@ -44,6 +44,22 @@ cudaError_t launch_lost_halo(cudaStream_t s) {
 
 bool lk_stream_supports(int iters, int radius) { return iters >= 1 && iters <= 5 && radius >= 1 && radius <= 3; }
 
+int lk_stream_cluster(int w, int h, int iters, int radius, int seg_rows) {
+    switch (radius) {
+        case 1: return lks::stream_plan<1>(w, h, iters, seg_rows).csize;
+        case 2: return lks::stream_plan<2>(w, h, iters, seg_rows).csize;
+        default: return lks::stream_plan<3>(w, h, iters, seg_rows).csize;
+    }
+}
+
+int lk_stream_seg_rows(int w, int h, int iters, int radius, int csize) {
+    switch (radius) {
+        case 1: return lks::stream_seg_rows<1>(w, h, iters, csize);
+        case 2: return lks::stream_seg_rows<2>(w, h, iters, csize);
+        default: return lks::stream_seg_rows<3>(w, h, iters, csize);
+    }
+}
+
 cudaError_t lk_stream_prepare(int max_smem_bytes) {
     cudaError_t e;
     if ((e = lks::stream_prepare<float>(max_smem_bytes)) != cudaSuccess) return e;

@@ -75,7 +75,6 @@ namespace lks {
 
 constexpr int kMX = 16;           // target box margin, columns
 constexpr int kMY = 5;            // target box margin, rows
-constexpr int kMaxCluster = 8;    // CTAs per cluster (the portable limit)
 
 template <int RAD, int R, int WX, int WY>
 struct StreamGeom {
@@ -743,11 +742,11 @@ StreamPlan stream_plan(int w, int h, int iters, int seg_rows) {
     const int c_min = 2 * halo / RH + 1;  // a region must be larger than its halo
     if (seg_rows > 0) {
         const long long c = ((long long)seg_rows + 2 * halo + RH - 1) / RH;
-        p.csize = c < c_min ? c_min : c > kMaxCluster ? kMaxCluster : (int)c;
+        p.csize = c < c_min ? c_min : c > kStreamMaxCluster ? kStreamMaxCluster : (int)c;
     } else {
         p.csize = c_min;
         long long best = -1;
-        for (int c = c_min; c <= kMaxCluster; ++c) {
+        for (int c = c_min; c <= kStreamMaxCluster; ++c) {
             const long long n = (long long)parts(h, c * RH) * c;
             if (best < 0 || n < best) {
                 best = n;
@@ -757,6 +756,16 @@ StreamPlan stream_plan(int w, int h, int iters, int seg_rows) {
     }
     p.ns = parts(h, p.csize * RH);
     return p;
+}
+
+// Rows of a segment that is a cluster of csize CTAs by itself, as seg_rows asks
+// for it; 0 where the halo needs more CTAs, or fewer cover the level.
+template <int RAD>
+int stream_seg_rows(int w, int h, int iters, int csize) {
+    const StreamPlan p = stream_plan<RAD>(w, h, iters, 0);
+    const int RH = p.small ? CfgGeom<RAD, true>::RH : CfgGeom<RAD, false>::RH;
+    const int rows = csize * RH - 2 * stream_halo(iters, RAD);
+    return rows > 0 && (csize - 1) * RH < h ? rows : 0;
 }
 
 template <int RAD, class Ts>

@@ -254,6 +254,43 @@ cudaError_t enqueue_lk_level(pano_rig* r, const RunCall& c, int l, const pano_ri
     return cudaSuccess;
 }
 
+// What pano_rig_autotune times on level l: AUTO; the streamed kernel once per
+// way of cutting the pairs (a cluster size, asked for through the rows of its
+// segments) that differs from AUTO's and from the earlier ones; the tiled kernel.
+std::vector<pano_rig_tuning> level_candidates(const pano_rig* r, int l) {
+    std::vector<pano_rig_tuning> cand;
+    pano_rig_tuning t;
+    memset(&t, 0, sizeof(t));
+    cand.push_back(t);  // PANO_LK_AUTO
+    if (lk_stream_supports(r->p.iters, r->p.radius)) {
+        auto cut = [&](int seg) {
+            std::vector<int> c;
+            for (int k = 0; k < r->d.n_pairs; ++k)
+                c.push_back(lk_stream_cluster(r->ws[k][l], r->hs[l], r->p.iters, r->p.radius, seg));
+            return c;
+        };
+        std::vector<std::vector<int>> seen = {cut(0)};
+        for (int c = 1; c <= kStreamMaxCluster; ++c)
+            for (int k = 0; k < r->d.n_pairs; ++k) {
+                const int seg = lk_stream_seg_rows(r->ws[k][l], r->hs[l], r->p.iters, r->p.radius, c);
+                if (seg == 0 || std::find(seen.begin(), seen.end(), cut(seg)) != seen.end()) continue;
+                seen.push_back(cut(seg));
+                t.kernel = PANO_LK_STREAM;
+                t.seg_rows = seg;
+                cand.push_back(t);
+            }
+    }
+    static const int tiles[][2] = {{32, 8}, {32, 16}, {16, 16}, {64, 8}, {64, 16}, {32, 32}};
+    for (auto& tl : tiles) {
+        memset(&t, 0, sizeof(t));
+        t.kernel = PANO_LK_TILE;
+        t.tile_w = tl[0];
+        t.tile_h = tl[1];
+        if (lk_smem_bytes(t.tile_w, t.tile_h, r->p.iters, r->p.radius) <= (size_t)r->max_smem) cand.push_back(t);
+    }
+    return cand;
+}
+
 // The whole rig step on stream s. Kernel launches are added to *kernels.
 cudaError_t enqueue_all(pano_rig* r, const RunCall& c, cudaStream_t s, bool trace, int* kernels) {
     const int n = r->d.n_pairs;
@@ -575,27 +612,6 @@ pano_status pano_rig_autotune(pano_rig* r, const pano_image* L, const pano_image
     r->launches += kernels;
     if (e != cudaSuccess) return cuda_fail(e, "rig launch");
 
-    std::vector<pano_rig_tuning> cand;
-    pano_rig_tuning t;
-    memset(&t, 0, sizeof(t));
-    cand.push_back(t);  // PANO_LK_AUTO
-    if (lk_stream_supports(r->p.iters, r->p.radius)) {
-        static const int segs[] = {0, 64, 96, 128, 192, 256, 384};
-        for (int sg : segs) {
-            t.kernel = PANO_LK_STREAM;
-            t.seg_rows = sg;
-            cand.push_back(t);
-        }
-    }
-    static const int tiles[][2] = {{32, 8}, {32, 16}, {16, 16}, {64, 8}, {64, 16}, {32, 32}};
-    for (auto& tl : tiles) {
-        memset(&t, 0, sizeof(t));
-        t.kernel = PANO_LK_TILE;
-        t.tile_w = tl[0];
-        t.tile_h = tl[1];
-        if (lk_smem_bytes(t.tile_w, t.tile_h, r->p.iters, r->p.radius) <= (size_t)r->max_smem) cand.push_back(t);
-    }
-
     cudaEvent_t ev[2] = {nullptr, nullptr};
     if ((e = cudaEventCreate(&ev[0])) != cudaSuccess || (e = cudaEventCreate(&ev[1])) != cudaSuccess) {
         if (ev[0]) cudaEventDestroy(ev[0]);
@@ -604,6 +620,7 @@ pano_status pano_rig_autotune(pano_rig* r, const pano_image* L, const pano_image
     pano_status out = PANO_OK;
     std::vector<float> times(reps);
     for (int l = 0; l < r->nlev && out == PANO_OK; ++l) {
+        const std::vector<pano_rig_tuning> cand = level_candidates(r, l);
         float best = -1.f;
         pano_rig_tuning pick = cand[0];
         for (const pano_rig_tuning& ct : cand) {

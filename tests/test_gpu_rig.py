@@ -225,6 +225,27 @@ def test_autotune_sets_valid_tunings_and_keeps_results(small_rig_pairs):
                 assert float((a - b).abs().mean()) <= 1e-3
 
 
+def test_autotune_times_each_way_of_cutting_a_level_once():
+    # One level of 200 x 90 pixels per pair, radius 2, 5 steps: CTAs of 16 rows
+    # and a halo of 10. A cluster of c CTAs leaves 16 c - 20 rows (c >= 2), AUTO
+    # takes the fewest CTAs that cover the rows, so c = 2 .. 8 less AUTO's own;
+    # all six tiles fit. Levels of 40 rows: c = 2 and 3, AUTO's is 3.
+    def parts(h, c):
+        return 1 if h <= 16 * c else -(-(h - 20) // (16 * c - 20))
+
+    for h in (200, 40):
+        sizes = [c for c in range(2, 9) if 16 * (c - 1) < h]
+        auto = min(range(2, 9), key=lambda c: (parts(h, c) * c, c))
+        img = torch.zeros((h, 90), dtype=torch.float32, device=DEV)
+        with binding.Rig(binding.Params(levels=1), h, [90, 90], c=1, dtype=torch.float32, canvas_hw=(h, 180),
+                         canvas_x0=[0, 90]) as rig:
+            rig.run([img] * 2, [img] * 2)
+            run = rig.launches
+            rig.autotune([img] * 2, [img] * 2, reps=1)
+            # a warm-up and a timed launch per candidate
+            assert rig.launches - 2 * run == 2 * (1 + len(set(sizes) - {auto}) + 6), (h, sizes, auto)
+
+
 def test_float_gray_rig_equals_single_pair_path():
     geom = dict(h=160, widths=(96, 130), x0=(0, 90), canvas=(160, 300), y0=0, levels=3)
     pairs = [synth.pair_small_gray(seed=50 + k, h=160, w=w, levels=3) for k, w in enumerate(geom["widths"])]
