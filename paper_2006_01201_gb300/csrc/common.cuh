@@ -319,15 +319,17 @@ cudaError_t pyr_tail_prepare(int max_smem_bytes);
 constexpr long long kStreamSmallWork = 1600000;
 constexpr int kStreamSmallHalo = 16;  // half of a small region is left
 constexpr int kStreamMaxReach = 24;
-// Levels below kSmallTilePixels use small tiles (kSmallTileW x kSmallTileH):
-// their few large tiles would leave most SMs idle, and the time of such a
-// level is the latency of one tile. (Measured on GB300: a 5.9k-pixel level
-// takes 15 us on 16x8 tiles and 21 us on 32x16.)
+// Levels below kSmallTilePixels that the tiled kernel works on (a rig's tuning,
+// or iters 0) use small tiles (kSmallTileW x kSmallTileH): their few large tiles
+// would leave most SMs idle, and the time of such a level is the latency of one
+// tile. (5 steps at radius 2, 16 x 8 / 32 x 16 tiles: 5.9k pixels 15.1 / 20.4 us,
+// 16k 18.9 / 20.6, 23.5k 26.7 / 21.2.) A default tile that is smaller still, the
+// only one whose halo fits in shared memory, stays.
 constexpr long long kSmallTilePixels = 16000;
 constexpr int kSmallTileW = 16, kSmallTileH = 8;
 // Tile of the tiled kernel for a level of w x h pixels, given the default.
 inline void lk_level_tile(int w, int h, int def_w, int def_h, int* tw, int* th) {
-    const bool small = (long long)w * h < kSmallTilePixels;
+    const bool small = (long long)w * h < kSmallTilePixels && kSmallTileW * kSmallTileH <= def_w * def_h;
     *tw = small ? kSmallTileW : def_w;
     *th = small ? kSmallTileH : def_h;
 }

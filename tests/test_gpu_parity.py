@@ -283,6 +283,23 @@ def test_auto_beyond_five_steps_on_either_side_of_its_lines(h, w, iters, radius)
     assert np.abs(got - ref).max() <= 1e-3
 
 
+@pytest.mark.parametrize("iters,radius", [(13, 2), (9, 3)])
+def test_small_levels_at_the_largest_reach(iters, radius):
+    # only the smallest tile fits in shared memory with a halo of 26 or 27 pixels
+    pair = synth.pair_small_gray(h=60, w=80, levels=2)
+    prm = binding.Params(levels=2, iters=iters, radius=radius)
+    olr, orl = oracle.flow_pair(pair.L, pair.R, oracle.Params(levels=2, iters=iters, radius=radius))
+    L, R = cuda(pair.L), cuda(pair.R)
+    with binding.FlowContext(prm, 60, 80, 1) as ctx:
+        flows = [ctx.flow_pair(L, R), binding.flow_pair_static(prm, L, R)]
+    with binding.Rig(prm, 60, [80], c=1, dtype=torch.float32, canvas_hw=(60, 80), canvas_x0=[0]) as rig:
+        rig.run([L], [R])
+        flows.append(rig.flows(0))
+        torch.cuda.synchronize()
+    for lr, rl in flows:
+        assert epe(lr.cpu().numpy(), olr).max() <= 1e-3 and epe(rl.cpu().numpy(), orl).max() <= 1e-3
+
+
 def test_streamed_kernel_refuses_more_than_five_steps():
     T = texture(64, 64, 23).astype(np.float32)
     with pytest.raises(binding.PanoError) as ei:
