@@ -39,7 +39,6 @@ WORKLOAD = {"workload": "pair_4000x1500_rgb_u8_lv6", "h": 4000, "w": 1500, "chan
 SMALL_WORKLOAD = {"workload": "pair_256x512_gray_f32_lv4", "h": 256, "w": 512, "channels": 1, "levels": 4,
                   "iters": 5, "radius": 2}
 L2_FLUSH_BYTES = 256 << 20   # > 129 MB L2
-STREAM_MIN_PIXELS = 50000    # rig_level_kernels' default: pairs of at least this many pixels are streamed
 SMALL_TILE_PIXELS = 16000    # tiled levels below this many pixels use 16 x 8 tiles
 # ncu counters of the dominant kernels (DRAM bytes and warp instructions per
 # launch), written by `--ingest-ncu` from a capture into profiles/ together
@@ -224,14 +223,13 @@ def tuning_key(t) -> list:
 PYR_DTYPES = {"f32": (1, 0, 4), "bf16": (2, 1, 2), "f16": (3, 2, 2)}
 
 
-def rig_level_kernels(h: int, widths, levels: int, kernels, tiles=None, stream_min=STREAM_MIN_PIXELS):
+def rig_level_kernels(h: int, widths, levels: int, kernels, tiles=None):
     """Kernel launches of each LK level of a rig, in launch order: for level
     l, [(kernel name, [pairs])], the streamed batch first, then one tiled
     launch per tile shape (in the order of the first pair with it).
     kernels[l] is the level's PANO_LK_* tuning and tiles[l] its (tile_w,
-    tile_h), (0, 0) for the default. AUTO streams the pairs of at least
-    stream_min pixels at the level (0: all of them, as the library does while
-    iters * radius is at most 24)."""
+    tile_h), (0, 0) for the default. AUTO streams every pair, as the library
+    does while iters * radius is at most 24."""
     out = []
     for l in range(levels):
         hl = h
@@ -242,8 +240,7 @@ def rig_level_kernels(h: int, widths, levels: int, kernels, tiles=None, stream_m
         tile = tuple(tiles[l]) if tiles else (0, 0)
         st, groups = [], {}
         for k, w in enumerate(ws):
-            use = kernels[l] == PANO_LK_STREAM or (kernels[l] == PANO_LK_AUTO and hl * w >= stream_min)
-            if use:
+            if kernels[l] != PANO_LK_TILE:
                 st.append(k)
                 continue
             shape = tile if tile != (0, 0) else ("small" if hl * w < SMALL_TILE_PIXELS else "default")
@@ -986,7 +983,7 @@ def measure_rig(dev, pairs, pyr_dtype: str, steps: int, warmup: int, world: int 
         recs = rig.trace_read(64 * steps)
         rig.trace_enable(0, 0)
         plan = rig_level_kernels(h, widths, levels, [t["kernel"] for t in tunings],
-                                 [(t["tile_w"], t["tile_h"]) for t in tunings], stream_min=0)
+                                 [(t["tile_w"], t["tile_h"]) for t in tunings])
         names = {1: "luma_kernel", 2: "pyr_down_kernel", 8: "rig_blend_kernel", 16: "luma_reduce_kernel",
                  32: "pyr_tail_kernel"}
         per_kind, lk_seen = {}, {}
