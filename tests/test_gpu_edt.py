@@ -195,10 +195,12 @@ def test_scratch_of_a_call_on_another_stream():
         del kept
 
 
-# The row pass works on groups of 32 columns (loads of 8) and bisects over the
-# groups with Area3; diagonals above 46340 take the other row pass. Sizes on either
-# side of each, areas that miss from whole columns, and one-group rows.
+# The row pass works on groups of 64 columns (loads of 4, block minima of 32) and
+# bisects over the groups with Area3. Sizes on either side of each, areas that miss
+# from whole columns, and one-group rows.
 @pytest.mark.parametrize("shape,p", [((9, 31), 0.5), ((9, 32), 0.5), ((9, 33), 0.5), ((7, 64), 0.02), ((7, 65), 0.02),
+                                     ((7, 63), 0.02), ((6, 127), 0.01), ((6, 128), 0.01), ((6, 129), 0.01), ((5, 130), 0.01),
+                                     ((4, 3), 0.3), ((4, 4), 0.3), ((4, 5), 0.3),
                                      ((5, 255), 0.01), ((5, 257), 0.003), ((3, 1025), 0.002), ((40, 700), 0.0004),
                                      ((1, 7), 0.3), ((2, 8), 0.3), ((300, 40), 0.001)])
 def test_sparse_areas_around_the_group_sizes(shape, p):
