@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(kColW * kColTY, 2) edt_cols_kernel(const unsig
 // Distances are 32-bit integers. In shared memory a column without a site has
 // g = kNearNone, the largest diagonal: no pixel is that far from a site, and its
 // square plus that of any distance within the row stays below 2^32.
-// What bounds it: the instructions of steps 2 and 3 (178 M warp instructions on
+// What bounds it: the instructions of steps 2 and 3 (177 M warp instructions on
 // a 4000 x 9000 canvas, 65% of the issue rate); the g plane is read once.
 // 224 us there, against 457 + 505 us of the envelopes' two launches; 254 us
 // with points at first pixels only, whose ranges span the gaps between runs,
@@ -485,7 +485,7 @@ __global__ void __launch_bounds__(kNearThreads) edt_near_kernel(const unsigned c
     for (int i = wid; i < n; i += kNearWarps) {
         if (list[i] & 1) continue;
         const int X = 32 * (int)list[i], x = X + 2 * lane;
-        const unsigned c0 = x < w ? PANO_AT(lab, x, w, 545) : 0, c1 = x + 1 < w ? PANO_AT(lab, x + 1, w, 545) : 0;
+        const unsigned c0 = x < w ? PANO_AT(lab, x, w, 548) : 0, c1 = x + 1 < w ? PANO_AT(lab, x + 1, w, 548) : 0;
         unsigned d0[2], d1[2];
 #pragma unroll
         for (int a = 0; a < 2; ++a) {

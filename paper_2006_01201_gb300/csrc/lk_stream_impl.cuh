@@ -28,18 +28,19 @@
 // cluster's top and bottom carry a halo of K r pixels, that the steps eat up
 // from outside (108 x 204 of 128 x 224 pixels are left at K r = 10).
 //
-// What bounds it (level 0 of a 4000 x 1500 pair, both directions, 300 us by
-// itself): the issue of instructions (half of the slots) and the shared-memory
-// pipe (57%), at 128 registers a thread and 16 warps an SM. Before, 768
-// threads worked through 12-row chunks of a ring in shared memory, eleven
-// CTA-wide barriers a chunk: 352 M warp instructions and 494 us. Registers
-// instead of the ring, and two pixels per paired instruction: 200 M. Measured
-// with the same arithmetic, on the whole pair (603 us): one barrier.cluster a
-// step, sent before and awaited after the inner rows' work, 3% slower (every
-// thread's fence in it); counted halos without the inner rows in between 10%;
-// the image's border masked behind a branch per row 2.5%; clusters of at most
-// 4 CTAs 1 to 3%, of up to 12 4%, runs of 6 rows 2 to 6%, of 4 rows with 24
-// warps an SM 6%, 256-column regions 17%.
+// What bounds it (level 0 of a 4000 x 1500 pair with smooth flows, both
+// directions, 300 us in a CUDA graph of launches): the issue of instructions
+// (half of the slots) and the shared-memory pipe (57%), at 128 registers a
+// thread and 16 warps an SM. Before, 768 threads worked through 12-row chunks of
+// a ring in shared memory, eleven CTA-wide barriers a chunk: 494 us, timed the
+// same way. Registers instead of the ring, and two pixels per paired instruction:
+// 353 to 197 M warp instructions (and 613 to 440 us, cold, under ncu on a pair
+// with depth steps). Measured with the same arithmetic, on the whole smooth pair
+// (603 us): one barrier.cluster a step, sent before and awaited after the inner
+// rows' work, 3% slower (every thread's fence in it); counted halos without the
+// inner rows in between 10%; the image's border masked behind a branch per row
+// 2.5%; clusters of at most 4 CTAs 1 to 3%, of up to 12 4%, runs of 6 rows 2 to
+// 6%, of 4 rows with 24 warps an SM 6%, 256-column regions 17%.
 //
 // The two halves of a warp own two runs on top of each other, the lower one
 // upside down. "Outer" rows (towards another warp) and "inner" rows (towards
